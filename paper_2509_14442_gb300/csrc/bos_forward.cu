@@ -8,6 +8,7 @@
 #include "bos_device.cuh"
 #include "bos_full.cuh"
 #include "bos_internal.h"
+#include "bos_march.cuh"
 
 namespace bos {
 
@@ -129,11 +130,89 @@ struct Sums {
     double I, du, dv, hu, hv;
 };
 
+// Sharma steps of one ray through the cell marcher, in the scaled variables V = dt dv and
+// a = (dt^2 / 6) D (metres per step), so that
+//   p2 = S(n+1/2) + dr + V/2 + 3a/4,   p3 = S(n+1) + dr + V + 3b
+//   dr += V + a + 2b,                  V += a + 4b + c
+// with a, b, c taken at dr, p2 and p3, and every constant exact in float32.  The next step's
+// first point and p3 differ by a - b, second order in the step: where that is below the resolution of a float32
+// fraction (kSamePoint cells; the usual case, ~1e-9 cells on a half-cell step), the two are
+// one point and a' = c, which leaves two field evaluations per step; where it is not (a
+// coarse step through a steep field), that lane evaluates a' at its own point.  The path
+// excess sum |dS + inc| - |dS| is d.(sum of inc) + sum (|inc|^2 - (d.inc)^2) / (2L + d.inc):
+// the first term is the end deviation, so only the small second one is summed.
+template <class E>
+__device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
+                                          float dr_end[3], float dv_end[3], float& excess_end, double& eta_in) {
+    MarchLine L;
+    MarchCell m;
+    const double sl = R.ell / (double)R.N;
+    double u0[3], du[3];
+    for (int a = 0; a < 3; ++a) {
+        u0[a] = (rs[a] + R.t_in * R.d[a] - S.g.origin[a]) * S.g.inv_h[a] - 0.5;
+        du[a] = (0.5 * sl) * R.d[a] * S.g.inv_h[a];
+    }
+    march_line(F.inv_h, u0, du, L, m);
+    const P3 d = p3(kept((float)R.d[0]), kept((float)R.d[1]), kept((float)R.d[2]));
+    const float near = kSamePoint / fmaxf(F.inv_h[0], fmaxf(F.inv_h[1], F.inv_h[2]));
+    const float len2 = kept((float)(2.0 * sl));
+    P3 dr = {0.0f, 0ull}, cr = dr, V = dr, cv = dr;
+    float excess = 0.0f;
+    f32x2 h = 0ull;   // half step, in both halves
+    const Cell2 v0 = march_value<true>(F, L, m, h, dr);
+    eta_in = 1.0 + (double)lo2(v0.lo);
+    // dt = (ell / N) / eta_in; dt^2 / 6 scales every acceleration of the ray, so it is rounded
+    // once, from float64 (one Newton step on the float32 reciprocal)
+    const double ie0 = (double)(1.0f / (float)eta_in), dt = sl * (ie0 * (2.0 - eta_in * ie0));
+    const float s = kept((float)(dt * dt * (1.0 / 6.0))), idt = kept(1.0f / (float)dt);
+    P3 a = march_accel(v0, s);
+    int n = 0;
+    while (n < R.N) {
+        if (lo2(h) >= 2.0f * kLineSteps) {
+            for (int q = 0; q < 3; ++q) {
+                u0[q] = (rs[q] + R.t_in * R.d[q] - S.g.origin[q]) * S.g.inv_h[q] - 0.5 +
+                        2.0 * n * ((0.5 * sl) * R.d[q] * S.g.inv_h[q]);
+                du[q] = (0.5 * sl) * R.d[q] * S.g.inv_h[q];
+            }
+            march_line(F.inv_h, u0, du, L, m);   // the cell is found again: back to cell 0 first
+            h = 0ull;
+            Frac3 f;
+            march_point<true>(F, L, m, h, dr, f);
+        }
+        const int n1 = min(R.N, n + kLineSteps);
+        for (; n < n1; ++n) {
+            h = add2(h, splat2(1.0f));
+            const P3 b = march_accel(march_value(F, L, m, h, fma3(0.75f, a, fma3(0.5f, V, dr))), s);
+            h = add2(h, splat2(1.0f));
+            P3 p = fma3(3.0f, b, add3(dr, V));
+            const P3 t = fma3(2.0f, b, a);
+            const P3 y = add3(t, sub3(V, cr));
+            const bool same = maxabs3(sub3(a, b)) <= near;
+            kahan3(dr, cr, y);
+            P3 c;
+#pragma unroll 1
+            for (int pass = 0;; ++pass) {
+                a = march_accel(march_value(F, L, m, h, p), s);
+                if (pass == 0) c = a;
+                if (same || pass == 1 || n + 1 == R.N) break;
+                p = dr;
+            }
+            kahan3(V, cv, sub3(add3(fma3(2.0f, b, t), c), cv));
+            const float di = dot3(d, y);
+            excess = fmaf(fmaf(-di, di, dot3(y, y)), rcp_approx(__fadd_rn(len2, di)), excess);
+        }
+    }
+    const P3 e = sub3(dr, cr), w = mul3(idt, sub3(V, cv));
+    dr_end[0] = e.x, dr_end[1] = lo2(e.yz), dr_end[2] = hi2(e.yz);
+    dv_end[0] = w.x, dv_end[1] = lo2(w.yz), dv_end[2] = hi2(w.yz);
+    excess_end = excess + dot3(d, e);
+}
+
 // Integrate one ray of the comp path (N > 0) from the pinhole rs; optionally store its
 // checkpoints every K steps in `state` (slot `ray`).  Leaves the end state in st.  CACHE:
 // the Sharma stages go through the ray's cell cache (the refracted connection's kernels,
 // which hold a second ray's state, go without: at 96 registers they spill).
-template <class E, int INTEG, bool CACHE = true>
+template <class E, int INTEG, bool CACHE>
 __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
                                          const CkptDev& ck, float4* state, long long ray, CompState& st,
                                          double& eta_in) {
@@ -283,24 +362,38 @@ __device__ __forceinline__ void comp_end(const CompState& st, float dr[3], float
     }
 }
 
+// End deviation, path excess and entry index of a ray: Sharma without checkpoints marches from
+// cell to cell, everything else goes stage by stage.
+template <class E, int INTEG, bool CONN, bool SAVE>
+__device__ __forceinline__ void trace_end(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
+                                          const CkptDev& ck, float4* state, long long ray, float dr[3], float dv[3],
+                                          float& excess, double& eta_in) {
+    if constexpr (INTEG == 0 && !SAVE) {
+        march_run(S, F, rs, R, dr, dv, excess, eta_in);
+    } else {
+        CompState st;
+        comp_run<E, INTEG, !CONN>(S, F, rs, R, ck, state, ray, st, eta_in);
+        comp_end(st, dr, dv);
+        excess = st.excess;
+    }
+}
+
 // Trace one camera ray of the comp path (checkpoints every K steps when ck.state is set).
 // With CONN (light mode 2) the luminance is read at the refracted projector connection of
 // the wall point x_w = x_ref + dx: M rounds of a <- a + (x_w - y(a)) from a = x_w, y(a) the
 // wall hit of the projector ray aimed at a (traced like a camera ray), so that
 // a = x_ref + e with e <- dx - (y(a) - (P + t_w d_p)) - ((P + t_w d_p) - a).
-template <class E, int INTEG, bool CONN>
+template <class E, int INTEG, bool CONN, bool SAVE>
 __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, const Ray& R, const CkptDev& ck,
                                 long long ray, bool want_hit, unsigned long long& steps) {
     WallRel h;
     if (R.N > 0) {
-        CompState st;
+        float dr[3], dv[3], excess;
         double eta_in;
-        comp_run<E, INTEG, !CONN>(S, F, S.cam.pos, R, ck, ck.state, ray, st, eta_in);
-        if (ck.state != nullptr) ck.excess[ray] = st.excess;
+        trace_end<E, INTEG, CONN, SAVE>(S, F, S.cam.pos, R, ck, ck.state, ray, dr, dv, excess, eta_in);
+        if (ck.state != nullptr) ck.excess[ray] = excess;
         steps += (unsigned long long)R.N;
-        float dr[3], dv[3];
-        comp_end(st, dr, dv);
-        h = comp_wall(S, R, eta_in, dr, dv, st.excess);
+        h = comp_wall(S, R, eta_in, dr, dv, excess);
     } else {   // straight camera ray (only with CONN: the projector rays may still bend)
         h.dx[0] = h.dx[1] = h.dx[2] = 0.0f;
         h.cosw = (float)(R.d[0] * S.w.normal[0] + R.d[1] * S.w.normal[1] + R.d[2] * S.w.normal[2]);
@@ -318,12 +411,11 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, const 
                 const Ray Rp = projector_setup(S, xref, e);
                 float yrel[3] = {0.0f, 0.0f, 0.0f};
                 if (Rp.wall && Rp.N > 0) {
-                    CompState sp;
                     double eta_p;
-                    comp_run<E, INTEG, !CONN>(S, F, P, Rp, ck, m == 0 ? ck.pstate : nullptr, ray, sp, eta_p);
+                    float pr[3], pv[3], pexcess;
+                    trace_end<E, INTEG, CONN, SAVE>(S, F, P, Rp, ck, m == 0 ? ck.pstate : nullptr, ray, pr, pv, pexcess,
+                                                    eta_p);
                     steps += (unsigned long long)Rp.N;
-                    float pr[3], pv[3];
-                    comp_end(sp, pr, pv);
                     const WallRel hp = comp_wall(S, Rp, eta_p, pr, pv, 0.0f);
                     if (hp.valid)
                         for (int a = 0; a < 3; ++a) yrel[a] = hp.dx[a];
@@ -401,17 +493,17 @@ __device__ RayResult trace_full(const SceneDev& S, const FullField<T>& F, const 
 template <int MODE>   // 0 straight, 1 comp fp32, 2 comp bf16, 3 full fp32, 4 full fp64
 struct Tracer;
 
-template <int MODE, int INTEG, bool CONN>
+template <int MODE, int INTEG, bool CONN, bool SAVE>
 __device__ __forceinline__ RayResult trace_ray(const SceneDev& S, const Ray& R, const CkptDev& ck, long long ray,
                                                bool want_hit, unsigned long long& steps) {
     if constexpr (MODE == 0) {
         return straight_epilogue(S, R, want_hit);
     } else if constexpr (MODE == 1) {
         const CompField<F4P> F = comp_field<F4P>(S.g);
-        return trace_comp<F4P, INTEG, CONN>(S, F, R, ck, ray, want_hit, steps);
+        return trace_comp<F4P, INTEG, CONN, SAVE>(S, F, R, ck, ray, want_hit, steps);
     } else if constexpr (MODE == 2) {
         const CompField<B4P> F = comp_field<B4P>(S.g);
-        return trace_comp<B4P, INTEG, CONN>(S, F, R, ck, ray, want_hit, steps);
+        return trace_comp<B4P, INTEG, CONN, SAVE>(S, F, R, ck, ray, want_hit, steps);
     } else if constexpr (MODE == 3) {
         FullField<float> F = {S.g};
         steps += (unsigned long long)R.N;
@@ -423,23 +515,28 @@ __device__ __forceinline__ RayResult trace_ray(const SceneDev& S, const Ray& R, 
     }
 }
 
+// Resident 128-thread blocks per SM that each tracer's register budget is cut for.
 #ifndef BOS_FWD_MIN_BLOCKS
-#define BOS_FWD_MIN_BLOCKS 6              // resident 128-thread blocks per SM the register budget is cut for
+#define BOS_FWD_MIN_BLOCKS 6
+#endif
+#ifndef BOS_FWD_MARCH_MIN_BLOCKS
+#define BOS_FWD_MARCH_MIN_BLOCKS 4        // Sharma through the cell marcher (32 polynomial values per ray)
 #endif
 #ifndef BOS_FWD_CACHED_MIN_BLOCKS
-#define BOS_FWD_CACHED_MIN_BLOCKS 5       // the same for the Sharma tracer on the paired stores, whose cell
-#endif                                    // cache holds 32 more values per ray (96 registers)
-#ifndef BOS_FWD_QUASI_MIN_BLOCKS
-#define BOS_FWD_QUASI_MIN_BLOCKS 3        // the same for quasi-linear tracing (more registers, more overlap)
+#define BOS_FWD_CACHED_MIN_BLOCKS 5       // Sharma with checkpoints, whose cell cache holds 32 values per ray
 #endif
-constexpr int render_min_blocks(int mode, int integ, bool conn) {
+#ifndef BOS_FWD_QUASI_MIN_BLOCKS
+#define BOS_FWD_QUASI_MIN_BLOCKS 3        // quasi-linear tracing (more registers, more overlap)
+#endif
+constexpr int render_min_blocks(int mode, int integ, bool conn, bool save) {
     return integ == 2 ? BOS_FWD_QUASI_MIN_BLOCKS
-                      : ((mode == 1 || mode == 2) && integ == 0 && !conn && BOS_FWD_PIPELINE) ? BOS_FWD_CACHED_MIN_BLOCKS
-                                                                                             : BOS_FWD_MIN_BLOCKS;
+           : (mode != 1 && mode != 2) || integ != 0 ? BOS_FWD_MIN_BLOCKS
+           : !save ? BOS_FWD_MARCH_MIN_BLOCKS
+           : !conn && BOS_FWD_PIPELINE ? BOS_FWD_CACHED_MIN_BLOCKS : BOS_FWD_MIN_BLOCKS;
 }
 // One warp tile of a render: the rays of its (up to) 32 lanes, averaged per pixel, written
 // to the outputs; adds the traced ray-steps to my_steps.
-template <int MODE, int INTEG, bool CONN>
+template <int MODE, int INTEG, bool CONN, bool SAVE>
 __device__ __forceinline__ void render_tile(const SceneDev& S, const RenderOut& out, const WorkDev& wk,
                                             const CkptDev& ck, const TileShape& ts, int t, int lane,
                                             unsigned long long& my_steps) {
@@ -468,7 +565,7 @@ __device__ __forceinline__ void render_tile(const SceneDev& S, const RenderOut& 
                     else ck.excess[ray] = 0.0f;
                 }
             } else {
-                r = trace_ray<MODE, INTEG, CONN>(S, R, ck, ray, out.hit != nullptr, my_steps);
+                r = trace_ray<MODE, INTEG, CONN, SAVE>(S, R, ck, ray, out.hit != nullptr, my_steps);
             }
             acc.I += r.I;
             acc.du += r.disp[0];
@@ -506,8 +603,9 @@ __device__ __forceinline__ void add_steps(unsigned long long* steps, unsigned lo
 
 // FEW: the form for launches with few warp tiles (a pixel minibatch), without a register
 // cap: the GPU is not full either way, and each ray finishes sooner without spills.
-template <int MODE, int INTEG, bool CONN, bool FEW = false>
-__global__ void __launch_bounds__(128, FEW ? 1 : render_min_blocks(MODE, INTEG, CONN))
+// SAVE (Sharma on the paired stores): with checkpoints; the other tracers look at ck.state.
+template <int MODE, int INTEG, bool CONN, bool FEW = false, bool SAVE = true>
+__global__ void __launch_bounds__(128, FEW ? 1 : render_min_blocks(MODE, INTEG, CONN, SAVE))
     render_kernel(SceneDev S, RenderOut out, WorkDev wk, CkptDev ck) {
     const TileShape ts = tile_shape(S.cam.width, S.cam.height, S.cam.spp);
     const int ntiles = tile_count(S, ts);
@@ -518,7 +616,7 @@ __global__ void __launch_bounds__(128, FEW ? 1 : render_min_blocks(MODE, INTEG, 
         if (lane == 0) t = atomicAdd(wk.tile_counter, 1);
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= ntiles) break;
-        render_tile<MODE, INTEG, CONN>(S, out, wk, ck, ts, t, lane, my_steps);
+        render_tile<MODE, INTEG, CONN, SAVE>(S, out, wk, ck, ts, t, lane, my_steps);
     }
     add_steps(wk.steps, my_steps, lane);
 }
@@ -528,7 +626,7 @@ __global__ void __launch_bounds__(128, FEW ? 1 : render_min_blocks(MODE, INTEG, 
 // jobs[j + 1].first and is that job's tile jobs[j].tile0 + (g - jobs[j].first).  Warps
 // pull items in order, so the jobs' tiles are interleaved as they are listed.
 template <int MODE, int INTEG>
-__global__ void __launch_bounds__(128, render_min_blocks(MODE, INTEG, false))
+__global__ void __launch_bounds__(128, render_min_blocks(MODE, INTEG, false, true))
     render_batch_kernel(const BatchJob* __restrict__ jobs, int njobs, int total, int* counter) {
     const int lane = threadIdx.x & 31;
     for (;;) {
@@ -540,7 +638,11 @@ __global__ void __launch_bounds__(128, render_min_blocks(MODE, INTEG, false))
         const BatchJob& J = jobs[j];
         const TileShape ts = tile_shape(J.S.cam.width, J.S.cam.height, J.S.cam.spp);
         unsigned long long my_steps = 0;
-        render_tile<MODE, INTEG, false>(J.S, J.out, J.wk, J.ck, ts, J.tile0 + (g - J.first), lane, my_steps);
+        const int t = J.tile0 + (g - J.first);
+        if (INTEG == 0 && J.ck.state == nullptr)
+            render_tile<MODE, INTEG, false, false>(J.S, J.out, J.wk, J.ck, ts, t, lane, my_steps);
+        else
+            render_tile<MODE, INTEG, false, true>(J.S, J.out, J.wk, J.ck, ts, t, lane, my_steps);
         add_steps(J.wk.steps, my_steps, lane);
     }
 }
@@ -629,14 +731,14 @@ cudaError_t launch_build_store(const GridDev& g, const float* T, void* store, cu
     return cudaGetLastError();
 }
 
-template <int MODE, int INTEG, bool CONN, bool FEW = false>
+template <int MODE, int INTEG, bool CONN, bool FEW = false, bool SAVE = true>
 static cudaError_t launch_render_c(const SceneDev& S, const RenderOut& o, const WorkDev& w, const CkptDev& ck,
                                    int num_sms, cudaStream_t st) {
     int per_sm = 0;
-    cudaError_t e = occupancy_prefer_l1(render_kernel<MODE, INTEG, CONN, FEW>, 128, 0, per_sm);
+    cudaError_t e = occupancy_prefer_l1(render_kernel<MODE, INTEG, CONN, FEW, SAVE>, 128, 0, per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    render_kernel<MODE, INTEG, CONN, FEW><<<num_sms * per_sm, 128, 0, st>>>(S, o, w, ck);
+    render_kernel<MODE, INTEG, CONN, FEW, SAVE><<<num_sms * per_sm, 128, 0, st>>>(S, o, w, ck);
     return cudaGetLastError();
 }
 
@@ -646,6 +748,13 @@ template <int MODE, int INTEG>
 static cudaError_t launch_render_t(const SceneDev& S, const RenderOut& o, const WorkDev& w, const CkptDev& ck,
                                    int num_sms, cudaStream_t st) {
     if constexpr (MODE == 1 || MODE == 2) {
+        // Sharma without checkpoints marches from cell to cell; with them the image, which seeds
+        // a gradient, keeps the stage-by-stage arithmetic that the adjoint's recompute repeats
+        if constexpr (INTEG == 0) {
+            if (ck.state == nullptr)
+                return S.L.mode == 2 ? launch_render_c<MODE, INTEG, true, false, false>(S, o, w, ck, num_sms, st)
+                                     : launch_render_c<MODE, INTEG, false, false, false>(S, o, w, ck, num_sms, st);
+        }
         if (S.L.mode == 2) return launch_render_c<MODE, INTEG, true>(S, o, w, ck, num_sms, st);
         // quasi-linear tracing of a few tiles (up to 8 warps per SM): the uncapped form
         if constexpr (INTEG == 2) {
