@@ -1,16 +1,15 @@
 // Adjoint of the BOS forward model (step a6, Sec. 2.4): dL/dT for a given dL/dI.
 //
-//   adjoint_kernel  -- per ray, reverse Sharma's steps segment by segment from the
-//                      checkpoints the forward kept every K steps (each segment is
-//                      recomputed forward into shared memory, then reversed), starting
-//                      from the adjoint of the wall epilogue (luminance, cosine, path
-//                      length of Eq. 2).  Each stage's field value and gradient come
-//                      from one packed trilinear evaluation.  The sensitivities of the
-//                      8 trilinear corners are summed per lane while the ray stays in a
-//                      cell, and flushed into per-node accumulators (d L/d deta,
-//                      d L/d grad eta) with warp-aggregated atomics: lanes whose rows
-//                      belong to the same cell are summed in shared memory, so each
-//                      (corner, channel) gets one atomic per cell visit per warp.
+//   reverse_kernel  -- per ray, reverse Sharma's steps from the end state the forward kept,
+//                      starting from the adjoint of the wall epilogue (luminance, cosine,
+//                      path length of Eq. 2), one field point (value and gradient) and one
+//                      scatter per half step.
+//   adjoint_kernel  -- the tiles with rays whose steps cannot be reversed that way: each
+//                      segment of K steps is recomputed forward from its checkpoint, keeping
+//                      the steps' states and stage terms, then reversed stage by stage.
+//                      In both, the sensitivities of the 8 trilinear corners are summed per
+//                      lane while the ray stays in a cell, and flushed into per-node
+//                      accumulators (d L/d deta, d L/d grad eta) with warp-aggregated atomics.
 //   gradient_kernel -- per node: the transpose of the central-difference stencil applied
 //                      to the grad-eta sensitivities, plus the deta sensitivity, times
 //                      d deta/dT = -rho0 G T0 / T^2.  A gather, so it is deterministic.
@@ -18,6 +17,7 @@
 #include "bos_device.cuh"
 #include "bos_full.cuh"
 #include "bos_internal.h"
+#include "bos_march.cuh"
 
 namespace bos {
 
@@ -324,12 +324,462 @@ __device__ __forceinline__ void straight_aim_adjoint(const SceneDev& S, const Ra
     for (int a = 0; a < 3; ++a) ab[a] = (db[a] - dd * Rp.d[a]) / nq;
 }
 
+// Refracted projector connection (light mode 2, one aiming round): the luminance is read at
+// a_1 = 2 x_w - y(x_w), y the wall hit of the projector ray aimed at x_w.  Sets that ray up,
+// its seed ybar = -dL/da_1, |q| of its aim and dL/dx_w's straight part; true where the
+// projector ray is traced and has to be reversed.
+__device__ __forceinline__ bool connection_seed(const SceneDev& S, const CkptDev& ck, long long slot, const Ray& R,
+                                                double Ib, bool act0, Ray& Rp, double* xlum, double* xlb, double* ybar,
+                                                double* nqp) {
+    for (int a = 0; a < 3; ++a) xlum[a] = xlb[a] = ybar[a] = 0.0;
+    nqp[0] = 1.0;
+    if (!act0) return false;
+    const float4 c0 = ck.conn[2 * slot], c1 = ck.conn[2 * slot + 1];
+    const float dxf[3] = {c0.x, c0.y, c0.z};
+    double xref[3], gL[3], q[3];
+    for (int a = 0; a < 3; ++a) {
+        xref[a] = S.cam.pos[a] + R.tw * R.d[a];
+        xlum[a] = xref[a] + ((double)dxf[a] - (double)(&c1.x)[a]);
+    }
+    const double Lb = Ib * (double)c0.w;
+    wall_luminance(S.L, S.w, xlum, gL);
+    for (int a = 0; a < 3; ++a) {
+        ybar[a] = -Lb * gL[a];
+        xlb[a] = 2.0 * Lb * gL[a];
+        q[a] = (xref[a] - S.L.proj.pos[a]) + (double)dxf[a];
+    }
+    nqp[0] = sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2]);
+    Rp = projector_setup(S, xref, dxf);
+    if (!Rp.wall) {                 // y = aim
+        for (int a = 0; a < 3; ++a) xlb[a] += ybar[a];
+    } else if (Rp.N <= 0) {         // straight projector ray
+        double ab[3];
+        straight_aim_adjoint(S, Rp, nqp[0], ybar, ab);
+        for (int a = 0; a < 3; ++a) xlb[a] += ab[a];
+    } else {
+        return ybar[0] != 0.0 || ybar[1] != 0.0 || ybar[2] != 0.0;
+    }
+    return false;
+}
+
+// A reversed projector ray's entry state as a function of its aim: r_in = P + t_in d,
+// v0 = eta_in d (base of v_N), straight step (ell/N) d, dt = ell / (N eta_in),
+// eta_in = 1 + deta(r_in), d = q / |q|, t_in and t_end on slab faces or the wall.  rb, etab,
+// dtb: adjoints of r_in, eta_in and dt; ge = grad eta(r_in); drbw, dvbw: of the end state; tpb:
+// of the straight step.  Adds dL/d aim to xlb.
+__device__ __forceinline__ void aim_adjoint(const SceneDev& S, const Ray& RR, double eta_in, double etab, double dtb,
+                                            const double ge[3], const float rb[3], const double* drbw,
+                                            const double* dvbw, const double* tpb, double nq, double* xlb) {
+    const double Nd = (double)RR.N, ds = RR.ell / Nd;
+    double dSb[3], rbi[3], db[3];
+    for (int a = 0; a < 3; ++a) {
+        dSb[a] = tpb[a] + Nd * drbw[a];
+        rbi[a] = (double)rb[a] + etab * ge[a];
+        db[a] = eta_in * dvbw[a] + ds * dSb[a] + RR.t_in * rbi[a];
+    }
+    const double ellb = dtb / (Nd * eta_in) + (RR.d[0] * dSb[0] + RR.d[1] * dSb[1] + RR.d[2] * dSb[2]) / Nd;
+    const double tinb = RR.d[0] * rbi[0] + RR.d[1] * rbi[1] + RR.d[2] * rbi[2] - ellb;
+    if (RR.in_axis >= 0) db[RR.in_axis] += tinb * (-RR.t_in / RR.d[RR.in_axis]);
+    if (RR.out_axis == 3) {
+        const double den = RR.d[0] * S.w.normal[0] + RR.d[1] * S.w.normal[1] + RR.d[2] * S.w.normal[2];
+        for (int a = 0; a < 3; ++a) db[a] += ellb * (-RR.tw * S.w.normal[a] / den);
+    } else {
+        const int oa = RR.out_axis;
+        db[oa] += ellb * (-(RR.t_in + RR.ell) / RR.d[oa]);
+    }
+    const double dd = db[0] * RR.d[0] + db[1] * RR.d[1] + db[2] * RR.d[2];
+    for (int a = 0; a < 3; ++a) xlb[a] += (db[a] - dd * RR.d[a]) / nq;
+}
+
 __host__ __device__ constexpr size_t adj_warp_floats(int K) {
     return (size_t)32 * kRow;   // K is carried by the global segment states
 }
 
 // Floats per lane and step of the recomputed segment: (dr, dv, A, B) of Sharma's step.
 constexpr int kSegFloats = 12;
+
+// ---- reversal without stage terms -----------------------------------------------------------
+//
+// In the scaled variables V = dt dv, a = (dt^2 / 6) D (see march_run) a Sharma step is
+//   r' = r + V + a + 2b,  V' = V + a + 4b + c,  p2 = r + V/2 + 3a/4,  p3 = r + V + 3b
+// and solving it backwards gives, exactly,
+//   p2 = r' - V'/2 + a/4 + c/2,  r = r' - V' + 2b + c,  V = V' - a - 4b - c.
+// p3 and r' differ by b - a, second order in the step: where the forward found that below
+// kSameReverse of a cell for all steps of a ray, c is the acceleration at r' and a may stand
+// for c in p2 (it enters with a/4), so the step is reversed from (r', V') alone: no segment
+// recompute, no kept stage terms, and the third stage of a step and the first stage of the
+// next one are one field point with one evaluation and one scatter.  Per step that is two value
+// and gradient evaluations and two scatters, where recomputing the segment and reversing the
+// three stages took three evaluations, three more with gradients and three scatters.
+// Tiles with a ray for which it does not hold are left to adjoint_kernel.
+//
+// With r_, V_ the adjoints of (r', V') and the path length's share added to r_ (u = unit step
+// direction): a_ = r_ + V_, b_ = 2 r_ + 4 V_, c_ = V_, and with P(w) = (dt^2/6) (dD/dx)^T w
+//   q3 = P3(c_), b_ += 3 q3;  q2 = P2(b_), a_ += 3/4 q2;  q1 = P1(a_)
+//   V_ += r_ + q3 + q2/2,  r_ += q3 + q2 + q1.
+// At the point between two steps both c_ of the earlier and a_ of the later step are known, so
+// their sum is scattered once.  All adjoints of a ray are held times s = dt^2/6, so that Q
+// needs no scaling and the point adjoints take s from the factor 1/h.
+
+// Corner sensitivities of a lane's current cell, in registers: corner c (x + 2y + 4z).
+struct CellRows {
+    Cell2 c[8];
+};
+
+__device__ __forceinline__ void rows_clear(CellRows& r) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) r.c[i] = Cell2{0ull, 0ull};
+}
+
+// r += w_c(f) Q
+__device__ __forceinline__ void rows_add(CellRows& r, const Frac3& f, Cell2 Q) {
+    const f32x2 x = splat2(f.x), y = splat2(f.y), z = splat2(f.z), z1 = splat2(1.0f - f.z);
+    Cell2 q[4];
+    q[1] = Cell2{mul2(x, Q.lo), mul2(x, Q.hi)};
+    q[0] = csub(Q, q[1]);
+    q[2] = Cell2{mul2(y, q[0].lo), mul2(y, q[0].hi)};
+    q[3] = Cell2{mul2(y, q[1].lo), mul2(y, q[1].hi)};
+    q[0] = csub(q[0], q[2]);
+    q[1] = csub(q[1], q[3]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        r.c[i] = cfma(z1, q[i], r.c[i]);
+        r.c[4 + i] = cfma(z, q[i], r.c[4 + i]);
+    }
+}
+
+// 16 bytes of shared memory where `on`, else zero: a predicated load, where a conditional one
+// compiles to a branch.
+__device__ __forceinline__ Cell2 load_if(uint32_t shared_addr, bool on) {
+    Cell2 v;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\tmov.b64 %0, 0;\n\tmov.b64 %1, 0;\n\t"
+        "@p ld.shared.v2.u64 {%0, %1}, [%2];\n\t}"
+        : "=l"(v.lo), "=l"(v.hi)
+        : "r"(shared_addr), "r"((unsigned)on)
+        : "memory");
+    return v;
+}
+
+// Warp-collective: add the rows of the flagged lanes to the node accumulators, lanes of the
+// same cell summed first, and clear them.  The rows go through shared memory; each quarter of
+// the warp (8 lanes: one pixel row of the tile) sums the rows of its own lanes, one cell per
+// pass, lane l taking corner l % 8 (8 lanes read one row: no bank conflict), and issues one
+// 16-byte atomic per corner.
+__device__ __forceinline__ void rows_flush(float* rows, bool flag, uint32_t key, CellRows& r, float* acc, int nx, int nxy,
+                                           uint32_t ncells, int* err) {
+    unsigned pend = __ballot_sync(0xffffffffu, flag);
+    if (!pend) return;
+    const int lane = threadIdx.x & 31, corner = lane & 7, first = lane & 24;
+    const uint32_t off = (uint32_t)(corner & 1) + (uint32_t)((corner >> 1) & 1) * (uint32_t)nx +
+                         (uint32_t)(corner >> 2) * (uint32_t)nxy;
+    const uint32_t mykey = flag ? key : kNoKey;
+    if (flag) {
+        ulonglong2* row = reinterpret_cast<ulonglong2*>(rows + lane * kRow);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) row[i] = make_ulonglong2(r.c[i].lo, r.c[i].hi);
+        rows_clear(r);
+    }
+    __syncwarp();
+    const uint32_t src = (uint32_t)__cvta_generic_to_shared(rows + first * kRow + corner * 4);
+    do {
+        const unsigned mine = (pend >> first) & 0xffu;
+        const uint32_t lk = __shfl_sync(0xffffffffu, mykey, mine ? first + __ffs(mine) - 1 : lane);
+        const unsigned eq = __ballot_sync(0xffffffffu, mykey == lk) & pend;
+        pend &= ~eq;
+        const unsigned part = (eq >> first) & mine;
+        Cell2 v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = load_if(src + i * (kRow * 4), (part >> i) & 1u);
+#pragma unroll
+        for (int w = 4; w >= 1; w >>= 1)
+#pragma unroll
+            for (int i = 0; i < w; ++i) v[i] = Cell2{add2(v[i].lo, v[i + w].lo), add2(v[i].hi, v[i + w].hi)};
+        if (part) atomicAdd(reinterpret_cast<float4*>(acc) + bounded(lk + off, ncells, err), to4(v[0]));
+    } while (pend);
+    __syncwarp();
+}
+
+// Value and fraction derivatives of the cell polynomial.
+struct PolyGrad {
+    Cell2 v, x, y, z;
+};
+__device__ __forceinline__ PolyGrad poly_grad(const CellPoly& p, const Frac3& f) {
+    const f32x2 x = splat2(f.x), y = splat2(f.y), z = splat2(f.z);
+    const Cell2 e0 = cfma(x, p.c[1], p.c[0]), e1 = cfma(x, p.c[3], p.c[2]);
+    const Cell2 e2 = cfma(x, p.c[5], p.c[4]), e3 = cfma(x, p.c[7], p.c[6]);
+    PolyGrad g;
+    g.z = cfma(y, e3, e2);
+    g.v = cfma(z, g.z, cfma(y, e1, e0));
+    g.y = cfma(z, e3, e1);
+    g.x = cfma(z, cfma(y, p.c[7], p.c[5]), cfma(y, p.c[3], p.c[1]));
+    return g;
+}
+
+// (dD/d record)^T w: the record adjoint Q that the corners share.
+__device__ __forceinline__ Cell2 record_adjoint(const PolyGrad& g, float eta, P3 w) {
+    const f32x2 t = mul2(w.yz, g.v.hi);
+    return Cell2{pack2(fmaf(w.x, hi2(g.v.lo), __fadd_rn(lo2(t), hi2(t))), eta * w.x), mul2(splat2(eta), w.yz)};
+}
+
+// s (d record / dx)^T Q, ih = s / h
+__device__ __forceinline__ P3 point_adjoint(const PolyGrad& g, Cell2 Q, P3 ih) {
+    const f32x2 a = fma2(g.x.hi, Q.hi, mul2(g.x.lo, Q.lo)), b = fma2(g.y.hi, Q.hi, mul2(g.y.lo, Q.lo)),
+                c = fma2(g.z.hi, Q.hi, mul2(g.z.lo, Q.lo));
+    return P3{ih.x * (lo2(a) + hi2(a)), mul2(ih.yz, pack2(lo2(b) + hi2(b), lo2(c) + hi2(c)))};
+}
+
+// Node index of a cell's base corner from its biased float indices.
+__device__ __forceinline__ uint32_t march_key(const MarchCell& m, uint32_t nx, uint32_t nxy) {
+    return (__float_as_uint(m.ci.x) & 0x7fffffu) + (__float_as_uint(lo2(m.ci.yz)) & 0x7fffffu) * nx +
+           (__float_as_uint(hi2(m.ci.yz)) & 0x7fffffu) * nxy;
+}
+
+// A ray of the tile has steps that cannot be reversed without their stage terms (the last bit
+// of its path record; every ray of the image has one).
+__device__ __forceinline__ bool tile_needs_stages(const CkptDev& ck, const TileShape& ts, int t, int lane, bool valid) {
+    bool strong = false;
+    for (int q = 0; q < ts.samples_per_lane; ++q)
+        if (valid) strong |= (__float_as_uint(ck.excess[((long long)t * 32 + lane) * ts.samples_per_lane + q]) & 1u) != 0u;
+    return __any_sync(0xffffffffu, strong);
+}
+
+// One warp tile of the Sharma adjoint by reversal.  Rows are empty on entry and on return.
+template <class E, bool CONN>
+__device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& ck, const AdjDev& adj,
+                                             const CompField<E>& F, const TileShape& ts, int t, int lane, float* rows,
+                                             float* acc, uint32_t ncells, int* err, int* deferred, double* xlum) {
+    const int nx = S.g.n[0], nxy = S.g.n[0] * S.g.n[1];
+    const int spp = S.cam.spp;
+    double* const xlb = xlum + 3;
+    double* const ybar = xlum + 6;
+    double* const drbw = xlum + 9;
+    double* const dvbw = xlum + 12;
+    double* const tpb = xlum + 15;
+    double* const nqp = xlum + 18;
+    const TilePix tp = tile_pixel(S, ts, t, lane);
+    if (tile_needs_stages(ck, ts, t, lane, tp.valid)) {
+        if (lane == 0) atomicAdd(deferred, 1);
+        return;
+    }
+    for (int qs = 0; qs < ts.samples_per_lane; ++qs) {
+        const int s = ts.samples_per_lane == 1 ? lane % ts.G : qs;
+        const long long slot = ((long long)t * 32 + lane) * ts.samples_per_lane + qs;
+        Ray R;
+        R.N = 0;
+        R.wall = false;
+        double Ib = 0.0;
+        if (tp.valid) {
+            R = ray_setup(S, tp.px, tp.py, s);
+            Ib = (double)adj.dLdI[(size_t)tp.out] / spp;
+        }
+        const bool act0 = tp.valid && R.wall && R.N >= 0 && Ib != 0.0;
+        Ray Rp;
+        Rp.N = 0;
+        Rp.wall = false;
+        bool pact = false;
+        if constexpr (CONN) pact = connection_seed(S, ck, slot, R, Ib, act0, Rp, xlum, xlb, ybar, nqp);
+        for (int pass = CONN ? 0 : 1; pass < 2; ++pass) {
+            const bool proj = CONN && pass == 0;
+            const Ray& RR = proj ? Rp : R;
+            const double* rs = proj ? S.L.proj.pos : S.cam.pos;
+            const float4* cstate = proj ? ck.pstate : ck.state;
+            const bool act = proj ? pact : (act0 && R.N > 0);
+            const int N = act ? RR.N : -1;
+            const int n_max = (int)__reduce_max_sync(0xffffffffu, (unsigned)(N + 1)) - 1;
+            if (n_max < 0) continue;
+            MarchLine L;
+            MarchCell m;
+            P3 dr = {0.0f, 0ull}, V = dr, rb = dr, Vb = dr, dS = dr, sih = dr;
+            float sc = 0.0f, lenb = 0.0f, dt = 0.0f;
+            double eta_in = 1.0, etab = 0.0;
+            uint32_t key = 0u;                // node of the cell's base corner
+            bool far_off = false;
+            if (act) {
+                const double sl = RR.ell / (double)RR.N;
+                double u0[3], du[3], rin[3];
+                for (int a = 0; a < 3; ++a) {
+                    rin[a] = rs[a] + RR.t_in * RR.d[a];
+                    u0[a] = (rin[a] - S.g.origin[a]) * S.g.inv_h[a] - 0.5;
+                    du[a] = (0.5 * sl) * RR.d[a] * S.g.inv_h[a];
+                }
+                march_line(F.inv_h, u0, du, L, m);
+                Frac3 f;
+                march_point<true>(F, L, m, 0ull, dr, f);
+                key = march_key(m, (uint32_t)nx, (uint32_t)nxy);
+                eta_in = 1.0 + (double)lo2(poly_value(m.p, splat2(f.x), splat2(f.y), splat2(f.z)).lo);
+                const double ie0 = (double)(1.0f / (float)eta_in), dtd = sl * (ie0 * (2.0 - eta_in * ie0));
+                dt = kept((float)dtd);
+                sc = kept((float)(dtd * dtd * (1.0 / 6.0)));
+                dS = p3(kept((float)(sl * RR.d[0])), kept((float)(sl * RR.d[1])), kept((float)(sl * RR.d[2])));
+                const float4 s0 = cstate[slot], s1 = cstate[ck.nrays + slot], s2 = cstate[2 * ck.nrays + slot];
+                const float er[3] = {s0.x - s0.w, s0.y - s1.w, s0.z - s2.w};
+                const float ev[3] = {s1.x - s2.x, s1.y - s2.y, s1.z - s2.z};
+                double rN[3], vN[3], drb[3], dvb[3], lb = 0.0;
+                for (int a = 0; a < 3; ++a) {
+                    rN[a] = rin[a] + RR.ell * RR.d[a] + (double)er[a];
+                    vN[a] = eta_in * RR.d[a] + (double)ev[a];
+                }
+                if (proj) {
+                    hit_adjoint(S, rN, vN, ybar, drb, dvb);
+                    for (int a = 0; a < 3; ++a) {
+                        drbw[a] = drb[a];
+                        dvbw[a] = dvb[a];
+                        tpb[a] = 0.0;
+                    }
+                } else {
+                    const double len_before = R.t_in + R.ell + (double)ck.excess[slot];
+                    wall_adjoint(S, rN, vN, len_before, Ib, drb, dvb, lb, CONN ? xlum : nullptr, CONN ? xlb : nullptr);
+                }
+                lenb = kept((float)lb) * sc;
+                // eta_in's adjoint through v0 and (below) dt = ell / (N eta_in); dv_N = V_N / dt
+                etab = dvb[0] * RR.d[0] + dvb[1] * RR.d[1] + dvb[2] * RR.d[2] +
+                       (dvb[0] * (double)ev[0] + dvb[1] * (double)ev[1] + dvb[2] * (double)ev[2]) / eta_in;
+                const float idt = 1.0f / dt;
+                dr = p3(er[0], er[1], er[2]);
+                V = mul3(dt, p3(ev[0], ev[1], ev[2]));
+                rb = p3(kept(sc * (float)drb[0]), kept(sc * (float)drb[1]), kept(sc * (float)drb[2]));
+                const float si = sc * idt;
+                Vb = p3(kept((float)dvb[0] * si), kept((float)dvb[1] * si), kept((float)dvb[2] * si));
+                sih = mul3(sc, L.ih);
+                far_off = !(maxabs3(P3{dr.x * L.ih.x, mul2(dr.yz, L.ih.yz)}) <= 0.0625f);
+            }
+            // A ray that ends more than a sixteenth of a cell off its line takes its state from
+            // the checkpoints where there is one: its deviation's rounding, 2^-29 of a cell and
+            // less otherwise, would build up over the steps.
+            const bool resync = __any_sync(0xffffffffu, far_off);
+            const int K = ck.every;
+            int to_ckpt = n_max % K;          // node n_max - to_ckpt is the next checkpointed one
+            CellRows row;
+            rows_clear(row);
+            P3 ab = {0.0f, 0ull};             // a_ of the later step, waiting for its point
+            float work = 0.0f;                // sum of a_.a + b_.b + c_.c
+            float tps[3] = {0.0f, 0.0f, 0.0f};
+            P3 rseg = rb;
+            int seg0 = n_max - to_ckpt;       // first node of the segment (the refracted sums)
+            f32x2 h = splat2(2.0f * (float)n_max);
+            bool used = false;                // the rows hold something
+            bool later = false;               // a later step of this ray has been reversed
+            for (int n = n_max;; --n, --to_ckpt) {
+                const bool on = n <= N;
+                // ---- the point between steps n - 1 and n
+                P3 c = {0.0f, 0ull}, q3 = c;
+                Frac3 f;
+                bool moved = false;
+                bool kept_state = false;
+                P3 Vk = c;
+                if (on) {
+                    if (resync && to_ckpt == 0 && n < N && n > 0) {
+                        const size_t cc = bounded((size_t)(n / K), (size_t)ck.max_ckpt, ck.err);
+                        const float4 s0 = cstate[(cc * 3 + 0) * ck.nrays + slot];
+                        const float4 s1 = cstate[(cc * 3 + 1) * ck.nrays + slot];
+                        const float4 s2 = cstate[(cc * 3 + 2) * ck.nrays + slot];
+                        dr = p3(s0.x - s0.w, s0.y - s1.w, s0.z - s2.w);
+                        Vk = mul3(dt, p3(s1.x - s2.x, s1.y - s2.y, s1.z - s2.z));
+                        kept_state = true;
+                    }
+                    moved = march_point<false>(F, L, m, h, dr, f);
+                }
+                if (__any_sync(0xffffffffu, moved)) {
+                    rows_flush(rows, moved && used, key, row, acc, nx, nxy, ncells, err);
+                    if (moved) key = march_key(m, (uint32_t)nx, (uint32_t)nxy);
+                }
+                if (on) {
+                    const PolyGrad g = poly_grad(m.p, f);
+                    const float eta = 1.0f + lo2(g.v.lo);
+                    c = march_accel(g.v, sc);
+                    if (later) V = kept_state ? Vk : sub3(V, c);
+                    P3 w = ab;
+                    if (n > 0) {
+                        w = add3(w, Vb);
+                        q3 = point_adjoint(g, record_adjoint(g, eta, Vb), sih);
+                    }
+                    Cell2 Q = record_adjoint(g, eta, w);
+                    const P3 q = point_adjoint(g, Q, sih);
+                    work = fmaf(eta, lo2(Q.lo), work);
+                    rb = add3(rb, sub3(q, q3));
+                    if constexpr (CONN) {
+                        const float tn = (float)(n - seg0);
+                        const P3 q1 = sub3(q, q3);
+                        tps[0] += tn * q1.x, tps[1] += tn * lo2(q1.yz), tps[2] += tn * hi2(q1.yz);
+                    }
+                    if (n == 0) {
+                        // entry: v0 = eta_in d and dt = ell / (N eta_in), eta_in = 1 + deta(r_in);
+                        // a, b and c carry dt^2, so dL/d dt = 2 work / dt (- dv_N . dL/d v_N / dt, above)
+                        etab -= 2.0 * (double)work / eta_in;
+                        Q.lo = pack2(lo2(Q.lo) + (float)etab, hi2(Q.lo));
+                    }
+                    rows_add(row, f, Q);
+                    used = true;
+                }
+                if constexpr (CONN) {
+                    if (proj && on && to_ckpt == 0) {
+                        const P3 e = sub3(rb, rseg);
+                        const float ee[3] = {e.x, lo2(e.yz), hi2(e.yz)};
+                        for (int a = 0; a < 3; ++a) {
+                            tpb[a] += ((double)tps[a] + (double)seg0 * (double)ee[a]) / (double)sc;
+                            tps[a] = 0.0f;
+                        }
+                        rseg = rb;
+                    }
+                }
+                if (to_ckpt == 0) {
+                    to_ckpt = K;
+                    seg0 -= K;
+                }
+                if (n == 0) break;
+                // ---- the middle of step n - 1
+                h = add2(h, splat2(-1.0f));
+                moved = false;
+                if (on) moved = march_point<false>(F, L, m, h, fma3(0.75f, c, fma3(-0.5f, V, dr)), f);
+                if (__any_sync(0xffffffffu, moved)) {
+                    rows_flush(rows, moved && used, key, row, acc, nx, nxy, ncells, err);
+                    if (moved) key = march_key(m, (uint32_t)nx, (uint32_t)nxy);
+                }
+                if (on) {
+                    const PolyGrad g = poly_grad(m.p, f);
+                    const float eta = 1.0f + lo2(g.v.lo);
+                    const P3 b = march_accel(g.v, sc);
+                    const P3 inc = sub3(V, fma3(2.0f, b, c));          // r' - r
+                    dr = sub3(dr, inc);
+                    V = sub3(V, fma3(4.0f, b, c));                     // less a, at the next point
+                    const P3 step = add3(dS, inc);
+                    const float ln = lenb * rsqrtf(dot3(step, step));
+                    const P3 sg = fma3(ln, step, rb);                  // r_ with the path length's share
+                    const P3 bb = fma3(2.0f, sg, fma3(4.0f, Vb, mul3(3.0f, q3)));
+                    const Cell2 Q = record_adjoint(g, eta, bb);
+                    const P3 q2 = point_adjoint(g, Q, sih);
+                    work = fmaf(eta, lo2(Q.lo), work);
+                    rows_add(row, f, Q);
+                    rb = add3(rb, add3(q3, q2));
+                    ab = fma3(0.75f, q2, add3(sg, Vb));
+                    Vb = add3(Vb, fma3(0.5f, q2, add3(sg, q3)));
+                    later = true;
+                    if constexpr (CONN) {
+                        const P3 t = fma3((float)(n - seg0), q3, mul3((float)(n - seg0) - 0.5f, q2));
+                        tps[0] += t.x, tps[1] += lo2(t.yz), tps[2] += hi2(t.yz);
+                    }
+                }
+                h = add2(h, splat2(-1.0f));
+            }
+            rows_flush(rows, used, key, row, acc, nx, nxy, ncells, err);
+            if constexpr (CONN) {
+                if (proj && act) {
+                    Frac3 f;
+                    march_point<false>(F, L, m, 0ull, P3{0.0f, 0ull}, f);
+                    const PolyGrad g = poly_grad(m.p, f);
+                    const double ge[3] = {(double)lo2(g.x.lo) * (double)F.inv_h[0], (double)lo2(g.y.lo) * (double)F.inv_h[1],
+                                          (double)lo2(g.z.lo) * (double)F.inv_h[2]};
+                    // etab = dvb . d - dtb dt / eta_in
+                    const double dtb = (dvbw[0] * RR.d[0] + dvbw[1] * RR.d[1] + dvbw[2] * RR.d[2] - etab) * eta_in /
+                                       (double)dt;
+                    const float rbf[3] = {rb.x / sc, lo2(rb.yz) / sc, hi2(rb.yz) / sc};
+                    aim_adjoint(S, RR, eta_in, etab, dtb, ge, rbf, drbw, dvbw, tpb, nqp[0], xlb);
+                }
+            }
+        }   // passes
+    }
+}
 
 // One warp tile of the Sharma adjoint: reverse every ray of the tile from its checkpoints
 // and scatter its sensitivities into the lane rows (flushed into acc as the cells change).
@@ -372,36 +822,7 @@ __device__ __forceinline__ void adjoint_tile(const SceneDev& S, const CkptDev& c
         Rp.wall = false;
         bool pact = false;
         if constexpr (CONN) {
-            for (int a = 0; a < 3; ++a) xlum[a] = xlb[a] = ybar[a] = 0.0;
-            nqp[0] = 1.0;
-            if (act0) {
-                const float4 c0 = ck.conn[2 * slot], c1 = ck.conn[2 * slot + 1];
-                const float dxf[3] = {c0.x, c0.y, c0.z};
-                double xref[3], gL[3], q[3];
-                for (int a = 0; a < 3; ++a) {
-                    xref[a] = S.cam.pos[a] + R.tw * R.d[a];
-                    xlum[a] = xref[a] + ((double)dxf[a] - (double)(&c1.x)[a]);
-                }
-                const double Lb = Ib * (double)c0.w;
-                wall_luminance(S.L, S.w, xlum, gL);
-                for (int a = 0; a < 3; ++a) {
-                    ybar[a] = -Lb * gL[a];
-                    xlb[a] = 2.0 * Lb * gL[a];
-                    q[a] = (xref[a] - S.L.proj.pos[a]) + (double)dxf[a];
-                }
-                nqp[0] = sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2]);
-                Rp = projector_setup(S, xref, dxf);
-                const bool seeded = ybar[0] != 0.0 || ybar[1] != 0.0 || ybar[2] != 0.0;
-                if (!Rp.wall) {                 // y = aim
-                    for (int a = 0; a < 3; ++a) xlb[a] += ybar[a];
-                } else if (Rp.N <= 0) {         // straight projector ray
-                    double ab[3];
-                    straight_aim_adjoint(S, Rp, nqp[0], ybar, ab);
-                    for (int a = 0; a < 3; ++a) xlb[a] += ab[a];
-                } else {
-                    pact = seeded;
-                }
-            }
+            pact = connection_seed(S, ck, slot, R, Ib, act0, Rp, xlum, xlb, ybar, nqp);
         }
         for (int pass = CONN ? 0 : 1; pass < 2; ++pass) {
         const bool proj = CONN && pass == 0;
@@ -430,9 +851,12 @@ __device__ __forceinline__ void adjoint_tile(const SceneDev& S, const CkptDev& c
             if (seg) {
                 CompState st;
                 const size_t cc = bounded((size_t)c, (size_t)ck.max_ckpt, ck.err);
-                const float4 s0 = cstate[(cc * 3 + 0) * ck.nrays + slot];
-                const float4 s1 = cstate[(cc * 3 + 1) * ck.nrays + slot];
-                const float4 s2 = cstate[(cc * 3 + 2) * ck.nrays + slot];
+                float4 s0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), s1 = s0, s2 = s0;   // the entry state
+                if (c > 0) {
+                    s0 = cstate[(cc * 3 + 0) * ck.nrays + slot];
+                    s1 = cstate[(cc * 3 + 1) * ck.nrays + slot];
+                    s2 = cstate[(cc * 3 + 2) * ck.nrays + slot];
+                }
                 st.dr[0] = s0.x; st.dr[1] = s0.y; st.dr[2] = s0.z;
                 st.dv[0] = s1.x; st.dv[1] = s1.y; st.dv[2] = s1.z;
                 st.cv[0] = s2.x; st.cv[1] = s2.y; st.cv[2] = s2.z;
@@ -629,43 +1053,60 @@ __device__ __forceinline__ void adjoint_tile(const SceneDev& S, const CkptDev& c
         accumulate(rows, act, cell_key_of(F, ci), cf, make_float4((float)etab, 0.0f, 0.0f, 0.0f), ca, acc, nx, nxy);
         if constexpr (CONN) {
             if (proj && act) {
-                // the projector ray's entry state as a function of its aim: r_in = P + t_in d,
-                // v0 = eta_in d (base of v_N), straight step (ell/N) d, dt = ell / (N eta_in),
-                // eta_in = 1 + deta(r_in), d = q / |q|, t_in and t_end on slab faces or the wall
-                const double Nd = (double)RR.N, ds = RR.ell / Nd;
                 Stage se;
                 const float zero[3] = {0, 0, 0};
                 stage_eval(F, st0.U, zero, bc, se);
                 const double ge[3] = {(double)se.ig.d0.x * (double)F.inv_h[0], (double)se.ig.d1.x * (double)F.inv_h[1],
                                       (double)se.ig.d2.x * (double)F.inv_h[2]};
-                double dSb[3], rbi[3], db[3];
-                for (int a = 0; a < 3; ++a) {
-                    dSb[a] = tpb[a] + Nd * drbw[a];
-                    rbi[a] = (double)rb[a] + etab * ge[a];
-                    db[a] = eta_in * dvbw[a] + ds * dSb[a] + RR.t_in * rbi[a];
-                }
-                const double ellb = (double)dtb / (Nd * eta_in) +
-                                    (RR.d[0] * dSb[0] + RR.d[1] * dSb[1] + RR.d[2] * dSb[2]) / Nd;
-                const double tinb = RR.d[0] * rbi[0] + RR.d[1] * rbi[1] + RR.d[2] * rbi[2] - ellb;
-                if (RR.in_axis >= 0) db[RR.in_axis] += tinb * (-RR.t_in / RR.d[RR.in_axis]);
-                if (RR.out_axis == 3) {
-                    const double den = RR.d[0] * S.w.normal[0] + RR.d[1] * S.w.normal[1] + RR.d[2] * S.w.normal[2];
-                    for (int a = 0; a < 3; ++a) db[a] += ellb * (-RR.tw * S.w.normal[a] / den);
-                } else {
-                    const int oa = RR.out_axis;
-                    db[oa] += ellb * (-(RR.t_in + RR.ell) / RR.d[oa]);
-                }
-                const double dd = db[0] * RR.d[0] + db[1] * RR.d[1] + db[2] * RR.d[2];
-                for (int a = 0; a < 3; ++a) xlb[a] += (db[a] - dd * RR.d[a]) / nqp[0];
+                aim_adjoint(S, RR, eta_in, etab, (double)dtb, ge, rb, drbw, dvbw, tpb, nqp[0], xlb);
             }
         }
         }   // passes
     }
 }
 
+#ifndef BOS_REV_MIN_BLOCKS
+#define BOS_REV_MIN_BLOCKS 7              // resident 2-warp blocks per SM the register budget is cut for
+#endif
+#ifndef BOS_REV_CONN_MIN_BLOCKS
+#define BOS_REV_CONN_MIN_BLOCKS 6         // the same with the refracted connection
+#endif
+// What bounds it: instruction issue and dependent arithmetic (54 % of the issue slots and half of
+// the float32 FMA pipe at 12 to 16 warps per SM), ~550 warp instructions per step of a tile, a
+// quarter of them in the row flushes; memory is at 32 % (L1) and 1 % (DRAM).  256x256x192 cells,
+// 2048^2 rays: 49.6 ms, where recomputing the segments took 128.4 ms; 192x192x144 cells in
+// bfloat16 at 768^2: 6.0 ms, 18.6 ms; with the refracted connection, 128x128x96 cells at 512^2:
+// 4.3 ms, 11.2 ms.  Against the float64 oracle the gradients are 10 to 35 % nearer than with the
+// recompute (relative L2 2e-7 .. 7e-7).  128 registers and 16 warps beat 168 and 12 by 2 to 3 %;
+// with the connection, whose spills then reach the loop, 168 are 7 % faster.  Summing the rows
+// of a whole warp one cell at a time, with branches around the row reads, took 62.7 ms.
+template <class E, bool CONN>
+__global__ void __launch_bounds__(kAdjWarps * 32, CONN ? BOS_REV_CONN_MIN_BLOCKS : BOS_REV_MIN_BLOCKS)
+    reverse_kernel(SceneDev S, CkptDev ck, AdjDev adj, WorkDev wk) {
+    extern __shared__ float4 smem4[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ double conn_sh[CONN ? kAdjWarps * 32 * kConnDoubles : 1];   // as in adjoint_kernel
+    double* const xlum = conn_sh + (CONN ? (warp * 32 + lane) * kConnDoubles : 0);
+    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * 32 * kRow;
+    const CompField<E> F = comp_field<E>(S.g);
+    const TileShape ts = tile_shape(S.cam.width, S.cam.height, S.cam.spp);
+    const int ntiles = tile_count(S, ts);
+    const uint32_t ncells = (uint32_t)S.g.n[0] * S.g.n[1] * S.g.n[2];
+    for (;;) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(wk.tile_counter, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= ntiles) break;
+        reverse_tile<E, CONN>(S, ck, adj, F, ts, t, lane, rows, reinterpret_cast<float*>(adj.acc), ncells, S.g.err,
+                              wk.tile_counter + 1, xlum);
+    }
+}
+
+// The tiles that reverse_kernel left (wk.tile_counter[1] of them; its queue is entry 2).
 template <class E, bool CONN_T>
 __global__ void __launch_bounds__(kAdjWarps * 32, BOS_ADJ_MIN_BLOCKS) adjoint_kernel(SceneDev S, CkptDev ck, AdjDev adj, WorkDev wk) {
     constexpr bool CONN = CONN_T;
+    if (wk.tile_counter[1] == 0) return;
     extern __shared__ float4 smem4[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // Refracted connection: values that live across a whole ray reversal are parked in
@@ -691,9 +1132,10 @@ __global__ void __launch_bounds__(kAdjWarps * 32, BOS_ADJ_MIN_BLOCKS) adjoint_ke
     CellAcc ca = {kNoKey, (uint32_t)S.g.n[0] * S.g.n[1] * S.g.n[2], S.g.err};
     for (;;) {
         int t = 0;
-        if (lane == 0) t = atomicAdd(wk.tile_counter, 1);
+        if (lane == 0) t = atomicAdd(wk.tile_counter + 2, 1);
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= ntiles) break;
+        if (!tile_needs_stages(ck, ts, t, lane, tile_pixel(S, ts, t, lane).valid)) continue;
         adjoint_tile<E, CONN>(S, ck, adj, F, ts, t, lane, rows, st_buf, acc, ca, xlum);
     }
     flush_rows(rows, ca.key != kNoKey, ca, acc, S.g.n[0], S.g.n[0] * S.g.n[1]);
@@ -1183,6 +1625,10 @@ template <class E, bool QUASI>
 __global__ void __launch_bounds__(kAdjWarps * 32, QUASI ? BOS_ADJ_QUASI_MIN_BLOCKS : BOS_ADJ_MIN_BLOCKS)
     adjoint_batch_kernel(const BatchJob* __restrict__ jobs, int njobs, int total, int* counter, float* seg_base,
                          int k_max) {
+    if (!QUASI) {   // the tiles that reverse_batch_kernel left
+        if (counter[1] == 0) return;
+        counter += 2;
+    }
     extern __shared__ float4 smem4[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * 32 * kRow;
@@ -1214,7 +1660,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32, QUASI ? BOS_ADJ_QUASI_MIN_BLOC
         float* acc = reinterpret_cast<float*>(J.adj.acc);
         if constexpr (QUASI)
             adjoint_quasi_tile<E>(J.S, J.ck, J.adj, F, ts, J.tile0 + (g - J.first), lane, rows, acc, ca);
-        else
+        else if (tile_needs_stages(J.ck, ts, J.tile0 + (g - J.first), lane,
+                                   tile_pixel(J.S, ts, J.tile0 + (g - J.first), lane).valid))
             adjoint_tile<E, false>(J.S, J.ck, J.adj, F, ts, J.tile0 + (g - J.first), lane, rows, st_buf, acc, ca,
                                    nullptr);
     }
@@ -1224,12 +1671,40 @@ __global__ void __launch_bounds__(kAdjWarps * 32, QUASI ? BOS_ADJ_QUASI_MIN_BLOC
     }
 }
 
+// reverse_kernel over several jobs' tiles; counter: queue, tiles left, queue of the rest.
+template <class E>
+__global__ void __launch_bounds__(kAdjWarps * 32, BOS_REV_MIN_BLOCKS)
+    reverse_batch_kernel(const BatchJob* __restrict__ jobs, int njobs, int total, int* counter) {
+    extern __shared__ float4 smem4[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * 32 * kRow;
+    for (;;) {
+        int g = 0;
+        if (lane == 0) g = atomicAdd(counter, 1);
+        g = __shfl_sync(0xffffffffu, g, 0);
+        if (g >= total) break;
+        const BatchJob& J = jobs[batch_job_of(jobs, njobs, g)];
+        reverse_tile<E, false>(J.S, J.ck, J.adj, comp_field<E>(J.S.g),
+                               tile_shape(J.S.cam.width, J.S.cam.height, J.S.cam.spp), J.tile0 + (g - J.first), lane, rows,
+                               reinterpret_cast<float*>(J.adj.acc), (uint32_t)J.S.g.n[0] * J.S.g.n[1] * J.S.g.n[2],
+                               J.S.g.err, counter + 1, nullptr);
+    }
+}
+
 template <class E, bool QUASI>
 static cudaError_t launch_adjoint_batch_c(const BatchJob* jobs, int njobs, int total, int* counter, float* seg_base,
                                           int k_max, int num_sms, cudaStream_t st) {
     const size_t smem = (size_t)kAdjWarps * 32 * kRow * sizeof(float);
     int per_sm = 0;
-    cudaError_t e = occupancy_prefer_l1(adjoint_batch_kernel<E, QUASI>, kAdjWarps * 32, smem, per_sm);
+    cudaError_t e;
+    if constexpr (!QUASI) {
+        e = occupancy_prefer_l1(reverse_batch_kernel<E>, kAdjWarps * 32, smem, per_sm);
+        if (e != cudaSuccess) return e;
+        if (per_sm < 1) return cudaErrorInvalidConfiguration;
+        reverse_batch_kernel<E><<<num_sms * per_sm, kAdjWarps * 32, smem, st>>>(jobs, njobs, total, counter);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    e = occupancy_prefer_l1(adjoint_batch_kernel<E, QUASI>, kAdjWarps * 32, smem, per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const int blocks = num_sms * per_sm < kAdjMaxBlocks ? num_sms * per_sm : kAdjMaxBlocks;
@@ -1264,6 +1739,12 @@ static cudaError_t launch_adjoint_c(const SceneDev& S, const CkptDev& ck, const 
     e = occupancy_prefer_l1(adjoint_kernel<E, CONN>, kAdjWarps * 32, smem, per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1 || adj.seg == nullptr) return cudaErrorInvalidConfiguration;
+    int rev_per_sm = 0;
+    e = occupancy_prefer_l1(reverse_kernel<E, CONN>, kAdjWarps * 32, smem, rev_per_sm);
+    if (e != cudaSuccess) return e;
+    if (rev_per_sm < 1) return cudaErrorInvalidConfiguration;
+    reverse_kernel<E, CONN><<<num_sms * rev_per_sm, kAdjWarps * 32, smem, st>>>(S, ck, adj, w);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int blocks = num_sms * per_sm < kAdjMaxBlocks ? num_sms * per_sm : kAdjMaxBlocks;
     adjoint_kernel<E, CONN><<<blocks, kAdjWarps * 32, smem, st>>>(S, ck, adj, w);
     return cudaGetLastError();

@@ -403,7 +403,7 @@ bos_status_t bos_create(bos_ctx** out, int device, uint64_t mem_limit_bytes) {
         delete c;
         return cuda_fail(e, "bos_create: memset");
     }
-    c->tile_counter = (int*)c->small;
+    c->tile_counter = (int*)c->small + 32;
     c->err = (int*)c->small + 1;
     c->steps = (unsigned long long*)((char*)c->small + 64);
     *out = c;
@@ -537,7 +537,7 @@ static bos_status_t render_prepare(bos_ctx* c, int mode, int save, cudaStream_t 
             ck.conn = c->conn;
         }
     }
-    cudaError_t e = cudaMemsetAsync(c->small, 0, 4, st);               // tile counter
+    cudaError_t e = cudaMemsetAsync(c->tile_counter, 0, kTileCounterBytes, st);
     if (e == cudaSuccess && mode != 0) e = cudaMemsetAsync(c->steps, 0, 8, st);   // the reference traces nothing
     if (e != cudaSuccess) return cuda_fail(e, "bos_render: memset");
     return BOS_OK;
@@ -626,7 +626,7 @@ static bos_status_t backward_impl(bos_ctx* c, const void* dLdI, void* dLdT, bool
     }
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e = cudaMemsetAsync(c->acc, 0, acc_bytes, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->small, 0, 4, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->tile_counter, 0, kTileCounterBytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "bos_backward: memset");
     AdjDev adj{c->acc, static_cast<const float*>(dLdI), c->err, c->seg};
     WorkDev w{c->tile_counter, c->steps, c->err};

@@ -215,7 +215,7 @@ __device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>&
 template <class E, int INTEG, bool CACHE>
 __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
                                          const CkptDev& ck, float4* state, long long ray, CompState& st,
-                                         double& eta_in) {
+                                         double& eta_in, float* apart_cells) {
     CompConst k;
     double rin[3];
     comp_setup(S, F, rs, R, st, k, eta_in, rin);
@@ -292,8 +292,11 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
         rhs_of(eval(st.U, st.dr, bc1, ci, cf), D);
         const float dt = k.dt;
         for (int a = 0; a < 3; ++a) A[a] = dt * D[a];
+        float apart = 0.0f;   // largest |A - B| of the steps
+        int left = K;         // steps before the next checkpoint
         for (int n = 0; n < R.N; ++n) {
-            if (state != nullptr && n % K == 0) {
+            if (state != nullptr && left == 0) {
+                left = K;
                 const size_t c = bounded((size_t)(n / K), (size_t)ck.max_ckpt, ck.err);
                 state[(c * 3 + 0) * ck.nrays + ray] = make_float4(st.dr[0], st.dr[1], st.dr[2], st.cr[0]);
                 state[(c * 3 + 1) * ck.nrays + ray] = make_float4(st.dv[0], st.dv[1], st.dv[2], st.cr[1]);
@@ -306,8 +309,12 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
                 U2[a] = st.U[a] + k.dUh[a];
                 U3[a] = st.U[a] + k.dU[a];
             }
+            --left;
             rhs_of(eval(U2, q, bc, ci, cf), D);
-            for (int a = 0; a < 3; ++a) B[a] = dt * D[a];
+            for (int a = 0; a < 3; ++a) {
+                B[a] = dt * D[a];
+                apart = fmaxf(apart, fabsf(A[a] - B[a]));
+            }
             for (int a = 0; a < 3; ++a) {
                 q[a] = st.dr[a] + dt * st.dv[a] + (0.5f * dt) * B[a];
                 inc_r[a] = dt * (st.dv[a] + (A[a] + 2.0f * B[a]) * (1.0f / 6.0f));
@@ -342,6 +349,16 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
                 A[a] = dt * D1[a];
             }
         }
+        if (state != nullptr) {
+            // the first checkpoint is the entry state, which is zero: its slot holds the end state
+            state[0 * ck.nrays + ray] = make_float4(st.dr[0], st.dr[1], st.dr[2], st.cr[0]);
+            state[1 * ck.nrays + ray] = make_float4(st.dv[0], st.dv[1], st.dv[2], st.cr[1]);
+            state[2 * ck.nrays + ray] = make_float4(st.cv[0], st.cv[1], st.cv[2], st.cr[2]);
+            // steps that the adjoint can reverse without their stage terms: dt |A - B| / 6 within
+            // kSameReverse cells (not so: NaN, too)
+            const float ih = fmaxf(F.inv_h[0], fmaxf(F.inv_h[1], F.inv_h[2]));
+            *apart_cells = R.N > kLineSteps ? __int_as_float(0x7f800000) : apart * dt * (ih * (1.0f / 6.0f));
+        }
     } else {
         for (int n = 0; n < R.N; ++n) {
             if (state != nullptr && n % K == 0) {
@@ -367,12 +384,12 @@ __device__ __forceinline__ void comp_end(const CompState& st, float dr[3], float
 template <class E, int INTEG, bool CONN, bool SAVE>
 __device__ __forceinline__ void trace_end(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
                                           const CkptDev& ck, float4* state, long long ray, float dr[3], float dv[3],
-                                          float& excess, double& eta_in) {
+                                          float& excess, double& eta_in, float* apart) {
     if constexpr (INTEG == 0 && !SAVE) {
         march_run(S, F, rs, R, dr, dv, excess, eta_in);
     } else {
         CompState st;
-        comp_run<E, INTEG, !CONN>(S, F, rs, R, ck, state, ray, st, eta_in);
+        comp_run<E, INTEG, !CONN>(S, F, rs, R, ck, state, ray, st, eta_in, apart);
         comp_end(st, dr, dv);
         excess = st.excess;
     }
@@ -387,11 +404,12 @@ template <class E, int INTEG, bool CONN, bool SAVE>
 __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, const Ray& R, const CkptDev& ck,
                                 long long ray, bool want_hit, unsigned long long& steps) {
     WallRel h;
+    float path = 0.0f, apart = 0.0f;   // path excess; largest stage distance of a step (cells)
     if (R.N > 0) {
         float dr[3], dv[3], excess;
         double eta_in;
-        trace_end<E, INTEG, CONN, SAVE>(S, F, S.cam.pos, R, ck, ck.state, ray, dr, dv, excess, eta_in);
-        if (ck.state != nullptr) ck.excess[ray] = excess;
+        trace_end<E, INTEG, CONN, SAVE>(S, F, S.cam.pos, R, ck, ck.state, ray, dr, dv, excess, eta_in, &apart);
+        path = excess;
         steps += (unsigned long long)R.N;
         h = comp_wall(S, R, eta_in, dr, dv, excess);
     } else {   // straight camera ray (only with CONN: the projector rays may still bend)
@@ -399,7 +417,6 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, const 
         h.cosw = (float)(R.d[0] * S.w.normal[0] + R.d[1] * S.w.normal[1] + R.d[2] * S.w.normal[2]);
         h.len = (float)R.tw;
         h.valid = h.cosw > 0.0f;
-        if (ck.state != nullptr) ck.excess[ray] = 0.0f;
     }
     float e[3] = {h.dx[0], h.dx[1], h.dx[2]};
     if constexpr (CONN) {
@@ -412,9 +429,10 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, const 
                 float yrel[3] = {0.0f, 0.0f, 0.0f};
                 if (Rp.wall && Rp.N > 0) {
                     double eta_p;
-                    float pr[3], pv[3], pexcess;
+                    float pr[3], pv[3], pexcess, papart = 0.0f;
                     trace_end<E, INTEG, CONN, SAVE>(S, F, P, Rp, ck, m == 0 ? ck.pstate : nullptr, ray, pr, pv, pexcess,
-                                                    eta_p);
+                                                    eta_p, &papart);
+                    if (!(papart <= apart)) apart = papart;
                     steps += (unsigned long long)Rp.N;
                     const WallRel hp = comp_wall(S, Rp, eta_p, pr, pv, 0.0f);
                     if (hp.valid)
@@ -431,6 +449,9 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, const 
             ck.conn[2 * ray + 1] = make_float4(h.dx[0] - e[0], h.dx[1] - e[1], h.dx[2] - e[2], 0.0f);
         }
     }
+    // the path record's last bit: whether the adjoint needs the ray's stage terms kept
+    if (ck.state != nullptr)
+        ck.excess[ray] = __uint_as_float((__float_as_uint(path) & ~1u) | (apart <= kSameReverse ? 0u : 1u));
     return comp_finish(S, R, h, e, want_hit);
 }
 
@@ -552,9 +573,9 @@ __device__ __forceinline__ void render_tile(const SceneDev& S, const RenderOut& 
             const int s = ts.samples_per_lane == 1 ? sl : q;
             const long long ray = ((long long)t * 32 + lane) * ts.samples_per_lane + q;   // checkpoint slot
             Ray R = ray_setup<MODE != 0>(S, px, py, s);
-            if (!R.wall) continue;
-            if (R.N < 0) {
-                flag_error(wk.err, DEV_STEP_BUDGET);
+            if (!R.wall || R.N < 0) {
+                if ((MODE == 1 || MODE == 2) && ck.state != nullptr) ck.excess[ray] = 0.0f;
+                if (R.wall) flag_error(wk.err, DEV_STEP_BUDGET);
                 continue;
             }
             RayResult r;

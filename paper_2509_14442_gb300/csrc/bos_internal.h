@@ -49,14 +49,19 @@ struct RenderOut {
     double* hit;
 };
 
+constexpr size_t kTileCounterBytes = 3 * sizeof(int);
+
 struct WorkDev {
-    int* tile_counter;              // warp tile queue (zeroed per launch)
+    int* tile_counter;              // warp tile queue; the Sharma adjoint: also the tiles its first
+                                    // kernel leaves to the second, and the second's queue (zeroed per launch)
     unsigned long long* steps;      // sum of N over traced rays
     int* err;                       // sticky device error word
 };
 
 // Ray state every K steps (float4 x3 per checkpoint: dr + cr.x, dv + cr.y, cv + cr.z),
-// index ((c * 3 + q) * nrays + slot), plus the path-length excess of every ray.  A ray's
+// index ((c * 3 + q) * nrays + slot); the entry state is zero, and checkpoint 0 holds the end
+// state instead.  Plus the path-length excess of every ray, whose last bit says that the
+// adjoint needs the ray's stage terms kept (see bos_adjoint.cu).  A ray's
 // slot is (tile * 32 + lane) * samples_per_lane + sample, so a warp's loads coalesce.
 struct CkptDev {
     float4* state;                  // nullptr: do not save

@@ -224,6 +224,10 @@ __device__ __forceinline__ P3 march_accel(Cell2 v, float s) {
 // float32 fraction in [0, 1) has: rounding alone moves a fraction by up to 2^-24.
 constexpr float kSamePoint = 5.9604645e-8f;   // 2^-24 cells
 
+// Bound of the same difference for reversing a ray without its stage terms (see
+// bos_adjoint.cu): it enters the gradient relative to one, so four times the resolution.
+constexpr float kSameReverse = 2.3841858e-7f;   // 2^-22 cells
+
 __device__ __forceinline__ float rcp_approx(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));

@@ -373,7 +373,7 @@ bool bos_server::launch_batch(int phase) {
     }
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->dev, b->host, sel.size() * sizeof(bos::BatchJob), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->counter, 0, sizeof(int), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->counter, 0, bos::kTileCounterBytes, st);
     if (e == cudaSuccess)
         e = phase == PH_RENDER ? bos::launch_render_batch(mode, integ, b->dev, (int)sel.size(), total, b->counter,
                                                           num_sms, st)
@@ -534,7 +534,7 @@ bos_status_t bos_server_create(bos_server** out, int device, uint64_t mem_limit_
             if (st != BOS_OK) break;
             if (cudaHostAlloc((void**)&b.host, kMaxBatchJobs * sizeof(bos::BatchJob), cudaHostAllocDefault) != cudaSuccess ||
                 cudaMalloc((void**)&b.dev, kMaxBatchJobs * sizeof(bos::BatchJob)) != cudaSuccess ||
-                cudaMalloc((void**)&b.counter, sizeof(int)) != cudaSuccess ||
+                cudaMalloc((void**)&b.counter, bos::kTileCounterBytes) != cudaSuccess ||
                 cudaEventCreateWithFlags(&b.ev, cudaEventDisableTiming) != cudaSuccess)
                 st = BOS_ERR_CUDA;
         }
