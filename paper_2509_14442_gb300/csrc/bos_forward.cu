@@ -14,28 +14,6 @@ namespace bos {
 
 // ===================================================================== a1: field store
 
-template <class E>
-__device__ __forceinline__ void store_cell(E* dst, double de, double gx, double gy, double gz);
-
-template <>
-__device__ __forceinline__ void store_cell<float4>(float4* dst, double de, double gx, double gy, double gz) {
-    *dst = make_float4(__double2float_rn(de), __double2float_rn(gx), __double2float_rn(gy), __double2float_rn(gz));
-}
-
-template <>
-__device__ __forceinline__ void store_cell<uint2>(uint2* dst, double de, double gx, double gy, double gz) {
-    uint32_t a = __bfloat16_as_ushort(__double2bfloat16(de)), b = __bfloat16_as_ushort(__double2bfloat16(gx));
-    uint32_t c = __bfloat16_as_ushort(__double2bfloat16(gy)), d = __bfloat16_as_ushort(__double2bfloat16(gz));
-    *dst = make_uint2(a | (b << 16), c | (d << 16));
-}
-
-template <>
-__device__ __forceinline__ void store_cell<D4>(D4* dst, double de, double gx, double gy, double gz) {
-    double2* p = reinterpret_cast<double2*>(dst);
-    p[0] = make_double2(de, gx);
-    p[1] = make_double2(gy, gz);
-}
-
 __device__ __forceinline__ double deta_at(const GridDev& g, const float* T, int i, int j, int k) {
     double t = (double)__ldg(T + ((size_t)k * g.n[1] + j) * g.n[0] + i);
     return ddiv(g.K, t);
@@ -75,13 +53,10 @@ __device__ __forceinline__ void write_elem(B4P* dst, const uint2* rec, int l, bo
     p.b = next ? rec[l + 1] : make_uint2(0u, 0u);
     *dst = p;
 }
-__device__ __forceinline__ void write_elem(D4* dst, const D4* rec, int l, bool) { store_cell<D4>(dst, rec[l].x, rec[l].y, rec[l].z, rec[l].w); }
 
-template <class R>
-__global__ void __launch_bounds__(256) build_store_kernel(GridDev g, const float* __restrict__ T,
-                                                          typename StoreElem<R>::type* __restrict__ store) {
+// The float64 store, evaluated in float64.
+__global__ void __launch_bounds__(256) build_store_kernel(GridDev g, const float* __restrict__ T, D4* __restrict__ store) {
     __shared__ double de[kHalo * kHalo * kHalo];
-    __shared__ __align__(32) R rec[kBrickCells];   // records are written with 16-byte stores
     const int b = blockIdx.x;
     const int bx = b % g.nb[0], by = (b / g.nb[0]) % g.nb[1], bz = b / (g.nb[0] * g.nb[1]);
     const int ox = bx * kBrick - 1, oy = by * kBrick - 1, oz = bz * kBrick - 1;
@@ -92,6 +67,7 @@ __global__ void __launch_bounds__(256) build_store_kernel(GridDev g, const float
         de[t] = deta_at(g, T, i, j, k);
     }
     __syncthreads();
+    const size_t slot = morton3((uint32_t)bx, (uint32_t)by, (uint32_t)bz);
     for (int local = threadIdx.x; local < kBrickCells; local += blockDim.x) {
         const int lx = local % kBrickSide, ly = (local / kBrickSide) % kBrickSide, lz = local / (kBrickSide * kBrickSide);
         const int c[3] = {min(bx * kBrick + lx, g.n[0] - 1), min(by * kBrick + ly, g.n[1] - 1),
@@ -114,11 +90,153 @@ __global__ void __launch_bounds__(256) build_store_kernel(GridDev g, const float
             }
             gr[a] = ddiv(dsub(at(hi[0], hi[1], hi[2]), at(lo[0], lo[1], lo[2])), den);
         }
-        store_cell<R>(rec + local, at(c[0], c[1], c[2]), gr[0], gr[1], gr[2]);
+        double2* dst = reinterpret_cast<double2*>(store + slot * kBrickCells + local);
+        dst[0] = make_double2(at(c[0], c[1], c[2]), gr[0]);
+        dst[1] = make_double2(gr[1], gr[2]);
+    }
+}
+
+// ---- float32 and bfloat16 records without the float64 pipe
+//
+// A record's values are float64 results rounded once to float32 or bfloat16: RN(K / T) and
+// RN(RN(K / T_hi - K / T_lo) / den).  GB300 runs float64 at a 64th of the float32 rate, and
+// build_store_kernel's seven divisions per cell kept that pipe busy for 1.66 ms on 256x256x192
+// cells.  Here the same values are formed from unevaluated sums of float32: K / T in three
+// terms (long division, each remainder exact by an fma; Dekker 1971), differences by two-sums
+// (Knuth), the product with 1 / den in two terms.  The result's float32 rounding f and what
+// is left, rho, are kept with a bound E of everything the float64 evaluation or the sums round
+// off; |rho| + E < ulp(f) / 2 proves that the float64 evaluation rounds to f too.  Otherwise
+// (one value in ~10^4 of a field with structure; smoother ones more often) the value is
+// evaluated in float64 as above.  The node values are the same bits.
+// What bounds it: issue (~150 instructions per record) and the store's 32 bytes per element;
+// 256x256x192 cells: 1.66 ms before, 324 us now (64^3: 44 us, 11.5 us; bfloat16 192x192x144: 706 us,
+// 138 us), against 0.12 ms to write 717 MB.
+
+struct Split3 {          // K, or K / T
+    float a, b, c;
+};
+struct BuildConst {
+    Split3 K;
+    float rh[3][2], rl[3][2];   // 1 / (2 h) and 1 / h per axis in two terms
+    float rm[3][2];             // upper bounds of both, times 2^-51
+};
+
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+// K / T to 2^-66 relative; NaN in the second term where a remainder could leave float32's range.
+__device__ __forceinline__ Split3 divide3(const Split3& K, float T) {
+    const float y = __frcp_rn(T);
+    Split3 q;
+    q.a = __fdiv_rn(K.a, T);
+    float r = fmaf(-q.a, T, K.a), e;             // exact for a correctly rounded quotient
+    two_sum(r, K.b, r, e);
+    q.b = __fmul_rn(r, y);
+    r = __fadd_rn(fmaf(-q.b, T, r), __fadd_rn(e, K.c));
+    q.c = __fmul_rn(r, y);
+    const float m = fabsf(q.a);
+    if (!(fabsf(T) > 1.0e-15f && fabsf(T) < 1.0e15f && m > 1.0e-12f && m < 1.0e12f))
+        q.b = __int_as_float(0x7fc00000);
+    return q;
+}
+
+// f = RN(p + e), |e| << |p|; true where a value within E of p + e rounds to f as well.
+__device__ __forceinline__ bool rounds_to(float p, float e, float E, float& f) {
+    f = __fadd_rn(p, e);
+    const float rho = __fsub_rn(e, __fsub_rn(f, p));
+    const uint32_t b = __float_as_uint(f);
+    // half an ulp; a power of two has half of that below it, and tiny results are left out
+    const float half = __uint_as_float((b & 0x7f800000u) - (24u << 23));
+    return (b & 0x7fffffu) != 0u && (b & 0x7f800000u) > (64u << 23) && fabsf(rho) + E < half;
+}
+__device__ __forceinline__ bool rounds_to(float p, float e, float E, uint16_t& h) {
+    float f;
+    if (!rounds_to(p, e, E, f)) return false;
+    h = __bfloat16_as_ushort(__float2bfloat16_rn(f));
+    return (__float_as_uint(f) & 0xffffu) != 0x8000u;   // halfway: the rest decides
+}
+
+__device__ __forceinline__ void round_exact(double v, float& f) { f = __double2float_rn(v); }
+__device__ __forceinline__ void round_exact(double v, uint16_t& h) { h = __bfloat16_as_ushort(__double2bfloat16(v)); }
+
+__device__ __forceinline__ float4 make_record(const float v[4]) { return make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ uint2 make_record(const uint16_t v[4]) {
+    return make_uint2((uint32_t)v[0] | ((uint32_t)v[1] << 16), (uint32_t)v[2] | ((uint32_t)v[3] << 16));
+}
+
+// One block per brick, as build_store_kernel; V = float or uint16_t (bfloat16 bits).
+template <class R, class V>
+__global__ void __launch_bounds__(256) build_split_kernel(GridDev g, BuildConst bc, const float* __restrict__ T,
+                                                          typename StoreElem<R>::type* __restrict__ store) {
+    constexpr int kCells = kHalo * kHalo * kHalo;
+    __shared__ float qa[kCells], qb[kCells], qc[kCells];
+    __shared__ __align__(32) R rec[kBrickCells];
+    const uint32_t b = blockIdx.x, nbx = (uint32_t)g.nb[0], nby = (uint32_t)g.nb[1];
+    const int bx = (int)(b % nbx), by = (int)((b / nbx) % nby), bz = (int)(b / (nbx * nby));
+    const int ox = bx * kBrick - 1, oy = by * kBrick - 1, oz = bz * kBrick - 1;
+    for (int t = threadIdx.x; t < kCells; t += 256) {
+        const int hx = t % kHalo, hy = (t / kHalo) % kHalo, hz = t / (kHalo * kHalo);
+        const int i = min(max(ox + hx, 0), g.n[0] - 1), j = min(max(oy + hy, 0), g.n[1] - 1),
+                  k = min(max(oz + hz, 0), g.n[2] - 1);
+        const Split3 q = divide3(bc.K, __ldg(T + ((size_t)k * g.n[1] + j) * g.n[0] + i));
+        qa[t] = q.a, qb[t] = q.b, qc[t] = q.c;
+    }
+    __syncthreads();
+    for (int local = threadIdx.x; local < kBrickCells; local += 256) {
+        const int lx = local % kBrickSide, ly = (local / kBrickSide) % kBrickSide, lz = local / (kBrickSide * kBrickSide);
+        const int c[3] = {min(bx * kBrick + lx, g.n[0] - 1), min(by * kBrick + ly, g.n[1] - 1),
+                          min(bz * kBrick + lz, g.n[2] - 1)};
+        const int at = ((c[2] - oz) * kHalo + (c[1] - oy)) * kHalo + (c[0] - ox);
+        const int step[3] = {1, kHalo, kHalo * kHalo};
+        const float de = qa[at];
+        V v[4];
+        bool sure[4];
+        sure[0] = rounds_to(de, __fadd_rn(qb[at], qc[at]), fabsf(de) * 1.4210855e-14f, v[0]);   // 2^-46
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int lo = c[a] > 0 ? at - step[a] : at, hi = c[a] < g.n[a] - 1 ? at + step[a] : at;
+            // (selected, not indexed: a per-lane index into the parameters takes the constant-load
+            // unit a cycle per thread, which bounded this kernel at 734 us)
+            const bool one = c[a] == 0 || c[a] == g.n[a] - 1;   // one-sided
+            const float rh = one ? bc.rh[a][1] : bc.rh[a][0], rl = one ? bc.rl[a][1] : bc.rl[a][0],
+                        rm = one ? bc.rm[a][1] : bc.rm[a][0];
+            const float s0 = __fsub_rn(qa[hi], qa[lo]);        // exact for values within a factor of two
+            float s1, e1, p, e;
+            two_sum(qb[hi], -qb[lo], s1, e1);
+            e1 = __fadd_rn(e1, __fsub_rn(qc[hi], qc[lo]));
+            two_sum(s0, s1, p, e);
+            e = __fadd_rn(e, e1);
+            two_sum(p, e, p, e);                               // difference = p + e
+            const float w = __fmul_rn(p, rh);
+            const float we = fmaf(p, rl, fmaf(e, rh, fmaf(p, rh, -w)));
+            const float big = fmaxf(fabsf(qa[hi]), fabsf(qa[lo]));
+            const bool near = big <= 2.0f * fminf(fabsf(qa[hi]), fabsf(qa[lo])) && __fmul_rn(qa[hi], qa[lo]) > 0.0f;
+            sure[1 + a] = near && rounds_to(w, we, fmaf(fabsf(w), 5.6843419e-14f, big * rm), v[1 + a]);   // 2^-44
+            if (p == 0.0f && e == 0.0f && near) {              // equal temperatures
+                v[1 + a] = V(0);
+                sure[1 + a] = true;
+            }
+        }
+        if (!(sure[0] && sure[1] && sure[2] && sure[3])) {
+            if (!sure[0]) round_exact(deta_at(g, T, c[0], c[1], c[2]), v[0]);
+            for (int a = 0; a < 3; ++a) {
+                if (sure[1 + a]) continue;
+                int lo[3] = {c[0], c[1], c[2]}, hi[3] = {c[0], c[1], c[2]};
+                lo[a] = max(c[a] - 1, 0);
+                hi[a] = min(c[a] + 1, g.n[a] - 1);
+                const double den = hi[a] - lo[a] == 2 ? dmul(2.0, g.h[a]) : g.h[a];
+                round_exact(ddiv(dsub(deta_at(g, T, hi[0], hi[1], hi[2]), deta_at(g, T, lo[0], lo[1], lo[2])), den),
+                            v[1 + a]);
+            }
+        }
+        rec[local] = make_record(v);
     }
     __syncthreads();
     const uint32_t slot = morton3((uint32_t)bx, (uint32_t)by, (uint32_t)bz);
-    for (int local = threadIdx.x; local < kBrickCells; local += blockDim.x)
+    for (int local = threadIdx.x; local < kBrickCells; local += 256)
         write_elem(store + (size_t)slot * kBrickCells + local, rec, local, local % kBrickSide < kBrickSide - 1);
 }
 
@@ -744,11 +862,23 @@ cudaError_t launch_probe_read(const void* buf, long long bytes, int repeats, flo
 
 cudaError_t launch_build_store(const GridDev& g, const float* T, void* store, cudaStream_t st) {
     const unsigned blocks = (unsigned)g.nb[0] * g.nb[1] * g.nb[2];
-    switch (g.prec) {
-        case 0: build_store_kernel<D4><<<blocks, 256, 0, st>>>(g, T, (D4*)store); break;
-        case 3: build_store_kernel<uint2><<<blocks, 256, 0, st>>>(g, T, (B4P*)store); break;
-        default: build_store_kernel<float4><<<blocks, 256, 0, st>>>(g, T, (F4P*)store); break;
+    if (g.prec == 0) {
+        build_store_kernel<<<blocks, 256, 0, st>>>(g, T, (D4*)store);
+        return cudaGetLastError();
     }
+    BuildConst bc;
+    bc.K.a = (float)g.K;
+    bc.K.b = (float)(g.K - (double)bc.K.a);
+    bc.K.c = (float)((g.K - (double)bc.K.a) - (double)bc.K.b);
+    for (int a = 0; a < 3; ++a)
+        for (int one = 0; one < 2; ++one) {
+            const double r = 1.0 / (one ? g.h[a] : 2.0 * g.h[a]);
+            bc.rh[a][one] = (float)r;
+            bc.rl[a][one] = (float)(r - (double)bc.rh[a][one]);
+            bc.rm[a][one] = (float)(r * 4.4408920985006262e-16 * 1.001);   // 2^-51
+        }
+    if (g.prec == 3) build_split_kernel<uint2, uint16_t><<<blocks, 256, 0, st>>>(g, bc, T, (B4P*)store);
+    else build_split_kernel<float4, float><<<blocks, 256, 0, st>>>(g, bc, T, (F4P*)store);
     return cudaGetLastError();
 }
 
