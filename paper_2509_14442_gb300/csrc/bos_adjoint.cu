@@ -1584,37 +1584,72 @@ __global__ void __launch_bounds__(kAdjWarps * 32) adjoint_fp64_kernel(SceneDev S
 }
 
 // dL/dT per node: transpose of the difference stencil of grad eta, plus d L/d deta, times
-// d deta/dT = -K / T^2.
-__device__ __forceinline__ double acc_channel(const float4* acc, long long m, int ch) {
-    const float4 v = acc[m];
-    return (double)(ch == 0 ? v.x : ch == 1 ? v.y : ch == 2 ? v.z : v.w);
-}
-__device__ __forceinline__ double acc_channel(const double* acc, long long m, int ch) { return acc[m * 4 + ch]; }
-
-template <class A, class O = float>
-__global__ void gradient_kernel(GridDev g, const A* __restrict__ acc, const float* __restrict__ T,
-                                O* __restrict__ dLdT) {
-    const long long n = (long long)g.n[0] * g.n[1] * g.n[2];
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const int idx[3] = {(int)(c % g.n[0]), (int)((c / g.n[0]) % g.n[1]), (int)(c / ((long long)g.n[0] * g.n[1]))};
-        const long long stride[3] = {1, g.n[0], (long long)g.n[0] * g.n[1]};
-        double tot = acc_channel(acc, c, 0);
-        for (int a = 0; a < 3; ++a) {
-            const int i = idx[a], na = g.n[a];
-            const double ih = g.inv_h[a], ih2 = 0.5 * g.inv_h[a];
-            if (i - 1 >= 0) tot += acc_channel(acc, c - stride[a], 1 + a) * (i - 1 == 0 ? ih : ih2);        // node i-1 reads i as hi
-            if (i + 1 <= na - 1) tot -= acc_channel(acc, c + stride[a], 1 + a) * (i + 1 == na - 1 ? ih : ih2);  // node i+1 reads i as lo
-            if (i == 0) tot -= acc_channel(acc, c, 1 + a) * ih;                                             // one-sided at the faces
-            if (i == na - 1) tot += acc_channel(acc, c, 1 + a) * ih;
-        }
-        if constexpr (sizeof(A) == 8) {
-            const double Tc = (double)T[c];
-            dLdT[c] = (O)(tot * (-g.K / (Tc * Tc)));
-        } else {
-            const float Tc = T[c];
-            dLdT[c] = (float)tot * (-(float)g.K / (Tc * Tc));
-        }
+// d deta/dT = -K / T^2.  Float64 accumulators (A = double) are summed in float64.
+template <class O>
+__global__ void gradient_fp64_kernel(GridDev g, const double* __restrict__ acc, const float* __restrict__ T,
+                                     O* __restrict__ dLdT) {
+    const uint32_t n = (uint32_t)g.n[0] * g.n[1] * g.n[2], c = blockIdx.x * 256u + threadIdx.x;
+    if (c >= n) return;
+    const uint32_t stride[3] = {1u, (uint32_t)g.n[0], (uint32_t)g.n[0] * (uint32_t)g.n[1]};
+    const int idx[3] = {(int)(c % stride[1]), (int)(c / stride[1] % (uint32_t)g.n[1]), (int)(c / stride[2])};
+    double tot = acc[(size_t)c * 4];
+    for (int a = 0; a < 3; ++a) {
+        const int i = idx[a], na = g.n[a];
+        const double ih = g.inv_h[a], ih2 = 0.5 * g.inv_h[a];
+        const double* p = acc + 1 + a;
+        if (i - 1 >= 0) tot += p[(size_t)(c - stride[a]) * 4] * (i - 1 == 0 ? ih : ih2);        // node i-1 reads i as hi
+        if (i + 1 <= na - 1) tot -= p[(size_t)(c + stride[a]) * 4] * (i + 1 == na - 1 ? ih : ih2);  // node i+1 reads i as lo
+        if (i == 0) tot -= p[(size_t)c * 4] * ih;                                               // one-sided at the faces
+        if (i == na - 1) tot += p[(size_t)c * 4] * ih;
     }
+    const double Tc = (double)T[c];
+    dLdT[c] = (O)(tot * (-g.K / (Tc * Tc)));
+}
+
+// The same for float32 accumulators.  The sum is carried in two float32 terms (products and
+// sums with their rounding errors, Knuth's two-sum), which keeps ~2^-46 of its largest term:
+// the float64 sum it replaces held the 12.6 M cells of a 256x256x192 grid for 611 us on the
+// float64 pipe and in 64-bit index divisions; this takes 121 us, against 45 us to read the
+// accumulators and T and write dL/dT (five rows of accumulators pass through L2 per row).
+struct GradConst {
+    float hi[3][2], lo[3][2];   // 1 / (2 h), 1 / h in two terms
+    float K;
+};
+
+__device__ __forceinline__ void add_term(float& s, float& e, float a, float kh, float kl) {
+    const float p = __fmul_rn(a, kh);
+    e = __fadd_rn(e, fmaf(a, kl, fmaf(a, kh, -p)));
+    const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z)));
+    s = t;
+}
+
+__global__ void __launch_bounds__(256) gradient_kernel(GridDev g, GradConst k, const float4* __restrict__ acc4,
+                                                       const float* __restrict__ T, float* __restrict__ dLdT) {
+    const uint32_t n = (uint32_t)g.n[0] * g.n[1] * g.n[2], c = blockIdx.x * 256u + threadIdx.x;
+    if (c >= n) return;
+    const uint32_t nx = (uint32_t)g.n[0], nxy = nx * (uint32_t)g.n[1];
+    const uint32_t z = c / nxy, r = c - z * nxy, y = r / nx;
+    const uint32_t idx[3] = {r - y * nx, y, z}, stride[3] = {1u, nx, nxy};
+    const float* acc = reinterpret_cast<const float*>(acc4) + (size_t)c * 4;
+    float s = acc[0], e = 0.0f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const uint32_t i = idx[a], last = (uint32_t)g.n[a] - 1u;
+        const float* p = acc + 1 + a;
+        if (i > 0u) {                                    // node i-1 reads i as hi
+            const bool one = i == 1u;                    // (selected: see build_split_kernel)
+            add_term(s, e, p[-(ptrdiff_t)stride[a] * 4], one ? k.hi[a][1] : k.hi[a][0], one ? k.lo[a][1] : k.lo[a][0]);
+        }
+        if (i < last) {                                  // node i+1 reads i as lo
+            const bool one = i + 1u == last;
+            add_term(s, e, -p[(size_t)stride[a] * 4], one ? k.hi[a][1] : k.hi[a][0], one ? k.lo[a][1] : k.lo[a][0]);
+        }
+        if (i == 0u) add_term(s, e, -p[0], k.hi[a][1], k.lo[a][1]);      // one-sided at the faces
+        if (i == last) add_term(s, e, p[0], k.hi[a][1], k.lo[a][1]);
+    }
+    const float Tc = T[c];
+    dLdT[c] = __fadd_rn(s, e) * (-k.K / (Tc * Tc));
 }
 
 // Batched adjoints (the request server): one launch covers warp tiles of several jobs,
@@ -1722,9 +1757,20 @@ cudaError_t launch_adjoint_batch(int mode, int integ, const BatchJob* jobs, int 
     return cudaErrorNotSupported;
 }
 
-cudaError_t launch_gradient(const GridDev& g, const float4* acc, const float* T, float* dLdT, int num_sms,
-                            cudaStream_t st) {
-    gradient_kernel<float4><<<num_sms * 8, 256, 0, st>>>(g, acc, T, dLdT);
+static unsigned cell_blocks(const GridDev& g) {
+    return (unsigned)(((long long)g.n[0] * g.n[1] * g.n[2] + 255) / 256);
+}
+
+cudaError_t launch_gradient(const GridDev& g, const float4* acc, const float* T, float* dLdT, cudaStream_t st) {
+    GradConst k;
+    k.K = (float)g.K;
+    for (int a = 0; a < 3; ++a)
+        for (int one = 0; one < 2; ++one) {
+            const double v = one ? g.inv_h[a] : 0.5 * g.inv_h[a];
+            k.hi[a][one] = (float)v;
+            k.lo[a][one] = (float)(v - (double)k.hi[a][one]);
+        }
+    gradient_kernel<<<cell_blocks(g), 256, 0, st>>>(g, k, acc, T, dLdT);
     return cudaGetLastError();
 }
 
@@ -1797,8 +1843,8 @@ cudaError_t launch_backward_fp64(const SceneDev& S, const CkptDev& ck, const Adj
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const double* acc = reinterpret_cast<const double*>(adj.acc);
-    if (f64) gradient_kernel<double, double><<<num_sms * 8, 256, 0, st>>>(S.g, acc, T, static_cast<double*>(dLdT));
-    else gradient_kernel<double, float><<<num_sms * 8, 256, 0, st>>>(S.g, acc, T, static_cast<float*>(dLdT));
+    if (f64) gradient_fp64_kernel<<<cell_blocks(S.g), 256, 0, st>>>(S.g, acc, T, static_cast<double*>(dLdT));
+    else gradient_fp64_kernel<<<cell_blocks(S.g), 256, 0, st>>>(S.g, acc, T, static_cast<float*>(dLdT));
     return cudaGetLastError();
 }
 
@@ -1813,9 +1859,7 @@ cudaError_t launch_backward(int mode, const SceneDev& S, const CkptDev& ck, cons
     else if (mode == 2) e = quasi ? launch_adjoint_quasi_t<B4P>(S, ck, adj, w, num_sms, st)
                                   : launch_adjoint_t<B4P>(S, ck, adj, w, num_sms, st);
     else return cudaErrorNotSupported;
-    if (e != cudaSuccess) return e;
-    gradient_kernel<float4><<<num_sms * 8, 256, 0, st>>>(S.g, adj.acc, T, dLdT);
-    return cudaGetLastError();
+    return e == cudaSuccess ? launch_gradient(S.g, adj.acc, T, dLdT, st) : e;
 }
 
 }  // namespace bos

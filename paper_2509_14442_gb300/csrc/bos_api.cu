@@ -768,7 +768,7 @@ bos_status_t ctx_batch_backward(bos_ctx* c, const float* dLdI, cudaStream_t st, 
 
 bos_status_t ctx_gradient(bos_ctx* c, float* dLdT, cudaStream_t st) {
     DeviceGuard dg(c->device);
-    cudaError_t e = launch_gradient(c->g, c->acc, c->T, dLdT, c->num_sms, st);
+    cudaError_t e = launch_gradient(c->g, c->acc, c->T, dLdT, st);
     return e == cudaSuccess ? BOS_OK : cuda_fail(e, "bos_backward: gradient");
 }
 

@@ -133,8 +133,7 @@ cudaError_t launch_render_batch(int mode, int integ, const BatchJob* jobs, int n
                                 int num_sms, cudaStream_t st);
 cudaError_t launch_adjoint_batch(int mode, int integ, const BatchJob* jobs, int njobs, int total, int* counter,
                                  float* seg_base, int k_max, int num_sms, cudaStream_t st);
-cudaError_t launch_gradient(const GridDev& g, const float4* acc, const float* T, float* dLdT, int num_sms,
-                            cudaStream_t st);
+cudaError_t launch_gradient(const GridDev& g, const float4* acc, const float* T, float* dLdT, cudaStream_t st);
 cudaError_t launch_ray_steps(const SceneDev& S, int32_t* nsteps, int num_sms, cudaStream_t st);
 cudaError_t launch_export_nodes(const GridDev& g, void* out, int num_sms, cudaStream_t st);
 cudaError_t launch_loss_l2(const float* I, const float* target, long long n, double* loss, float* dLdI, int num_sms,
