@@ -25,12 +25,6 @@ constexpr int kAdjWarps = kAdjWarpsPerBlock;   // warps per block
 #ifndef BOS_ADJ_MIN_BLOCKS
 #define BOS_ADJ_MIN_BLOCKS 5              // resident blocks per SM the register budget is cut for
 #endif
-#ifndef BOS_ADJ_QUASI_MIN_BLOCKS
-#define BOS_ADJ_QUASI_MIN_BLOCKS 7        // the same for the quasi-linear adjoint (128 registers, 16 warps/SM),
-#endif                                    // used when there are more than 12 warp tiles per SM
-#ifndef BOS_ADJ_QUASI_SMALL_MIN_BLOCKS
-#define BOS_ADJ_QUASI_SMALL_MIN_BLOCKS 1  // the quasi-linear adjoint for few tiles (no register cap)
-#endif
 constexpr int kRow = 36;              // floats per lane row of the cell accumulators (16-byte aligned rows)
 constexpr int kConnDoubles = 20;      // per-lane shared doubles of the refracted connection's adjoint
 constexpr uint32_t kNoKey = 0xffffffffu;
@@ -178,41 +172,6 @@ __device__ __forceinline__ void accumulate(float* rows, bool act, uint32_t cell,
             const f32x2 ww = pack2(w, w);
             float4 r = row[c];
             f32x2 lo = fma2(ww, qlo, pack2(r.x, r.y)), hi = fma2(ww, qhi, pack2(r.z, r.w));
-            unpack2(lo, r.x, r.y);
-            unpack2(hi, r.z, r.w);
-            row[c] = r;
-        }
-    }
-}
-
-// Warp-collective: add w_c(cf) Q and, where `dual`, then w_c(cf2) Q2 (a second sample in
-// the same cell) to the lane's cell row: the same two FMAs per value, in the same order, as
-// two calls of `accumulate`, with one read and one write of the row.
-__device__ __forceinline__ void accumulate_dual(float* rows, bool act, uint32_t cell, const float cf[3], float4 Q,
-                                                bool dual, const float cf2[3], float4 Q2, CellAcc& ca, float* acc,
-                                                int nx, int nxy) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t key = act ? cell : kNoKey;
-    flush_rows(rows, act && ca.key != kNoKey && ca.key != key, ca, acc, nx, nxy);
-    if (act) {
-        ca.key = key;
-        float4* row = reinterpret_cast<float4*>(rows + lane * kRow);
-        const float g0 = 1.0f - cf[0], g1 = 1.0f - cf[1], g2 = 1.0f - cf[2];
-        const float h0 = 1.0f - cf2[0], h1 = 1.0f - cf2[1], h2 = 1.0f - cf2[2];
-        const f32x2 qlo = pack2(Q.x, Q.y), qhi = pack2(Q.z, Q.w);
-        const f32x2 q2lo = pack2(Q2.x, Q2.y), q2hi = pack2(Q2.z, Q2.w);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const float w = ((c & 1) ? cf[0] : g0) * ((c & 2) ? cf[1] : g1) * ((c & 4) ? cf[2] : g2);
-            const f32x2 ww = pack2(w, w);
-            float4 r = row[c];
-            f32x2 lo = fma2(ww, qlo, pack2(r.x, r.y)), hi = fma2(ww, qhi, pack2(r.z, r.w));
-            if (dual) {
-                const float v = ((c & 1) ? cf2[0] : h0) * ((c & 2) ? cf2[1] : h1) * ((c & 4) ? cf2[2] : h2);
-                const f32x2 vv = pack2(v, v);
-                lo = fma2(vv, q2lo, lo);
-                hi = fma2(vv, q2hi, hi);
-            }
             unpack2(lo, r.x, r.y);
             unpack2(hi, r.z, r.w);
             row[c] = r;
@@ -516,6 +475,27 @@ __device__ __forceinline__ PolyGrad poly_grad(const CellPoly& p, const Frac3& f)
     return g;
 }
 
+template <bool VALUE_ONLY>
+__device__ __forceinline__ PolyGrad poly_point(const CellPoly& p, const Frac3& f) {
+    if constexpr (!VALUE_ONLY) return poly_grad(p, f);
+    PolyGrad g = {};
+    g.v = poly_value(p, splat2(f.x), splat2(f.y), splat2(f.z));
+    return g;
+}
+
+// The marcher's line of a ray with step 0 at its step `origin`.
+template <class E>
+__device__ __forceinline__ void set_line(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
+                                         int origin, MarchLine& L, MarchCell& m) {
+    const double half = 0.5 * (R.ell / (double)R.N);
+    double u0[3], du[3];
+    for (int a = 0; a < 3; ++a) {
+        du[a] = half * R.d[a] * S.g.inv_h[a];
+        u0[a] = (rs[a] + R.t_in * R.d[a] - S.g.origin[a]) * S.g.inv_h[a] - 0.5 + 2.0 * (double)origin * du[a];
+    }
+    march_line(F.inv_h, u0, du, L, m);
+}
+
 // (dD/d record)^T w: the record adjoint Q that the corners share.
 __device__ __forceinline__ Cell2 record_adjoint(const PolyGrad& g, float eta, P3 w) {
     const f32x2 t = mul2(w.yz, g.v.hi);
@@ -544,8 +524,11 @@ __device__ __forceinline__ bool tile_needs_stages(const CkptDev& ck, const TileS
     return __any_sync(0xffffffffu, strong);
 }
 
-// One warp tile of the Sharma adjoint by reversal.  Rows are empty on entry and on return.
-template <class E, bool CONN>
+// One warp tile of the adjoint by reversal.  Rows are empty on entry and on return.  QUASI: the
+// quasi-linear tracer, whose points lie on the straight line: the same recurrences for V and
+// the adjoints without the point adjoints (its outputs are linear in the sampled values), for
+// every ray.
+template <class E, bool CONN, bool QUASI = false>
 __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& ck, const AdjDev& adj,
                                              const CompField<E>& F, const TileShape& ts, int t, int lane, float* rows,
                                              float* acc, uint32_t ncells, int* err, int* deferred, double* xlum) {
@@ -558,7 +541,7 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
     double* const tpb = xlum + 15;
     double* const nqp = xlum + 18;
     const TilePix tp = tile_pixel(S, ts, t, lane);
-    if (tile_needs_stages(ck, ts, t, lane, tp.valid)) {
+    if (!QUASI && tile_needs_stages(ck, ts, t, lane, tp.valid)) {
         if (lane == 0) atomicAdd(deferred, 1);
         return;
     }
@@ -597,13 +580,9 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
             bool far_off = false;
             if (act) {
                 const double sl = RR.ell / (double)RR.N;
-                double u0[3], du[3], rin[3];
-                for (int a = 0; a < 3; ++a) {
-                    rin[a] = rs[a] + RR.t_in * RR.d[a];
-                    u0[a] = (rin[a] - S.g.origin[a]) * S.g.inv_h[a] - 0.5;
-                    du[a] = (0.5 * sl) * RR.d[a] * S.g.inv_h[a];
-                }
-                march_line(F.inv_h, u0, du, L, m);
+                double rin[3];
+                for (int a = 0; a < 3; ++a) rin[a] = rs[a] + RR.t_in * RR.d[a];
+                set_line(S, F, rs, RR, 0, L, m);
                 Frac3 f;
                 march_point<true>(F, L, m, 0ull, dr, f);
                 key = march_key(m, (uint32_t)nx, (uint32_t)nxy);
@@ -612,8 +591,12 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                 dt = kept((float)dtd);
                 sc = kept((float)(dtd * dtd * (1.0 / 6.0)));
                 dS = p3(kept((float)(sl * RR.d[0])), kept((float)(sl * RR.d[1])), kept((float)(sl * RR.d[2])));
-                const float4 s0 = cstate[slot], s1 = cstate[ck.nrays + slot], s2 = cstate[2 * ck.nrays + slot];
-                const float er[3] = {s0.x - s0.w, s0.y - s1.w, s0.z - s2.w};
+                const float4 s0 = cstate[slot], s1 = cstate[ck.nrays + slot];
+                float4 s2 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (!QUASI) s2 = cstate[2 * ck.nrays + slot];
+                // (quasi-linear tracing keeps its end state uncompensated, with the path excess)
+                const float er[3] = {s0.x - (QUASI ? 0.0f : s0.w), s0.y - (QUASI ? 0.0f : s1.w),
+                                     s0.z - s2.w};
                 const float ev[3] = {s1.x - s2.x, s1.y - s2.y, s1.z - s2.z};
                 double rN[3], vN[3], drb[3], dvb[3], lb = 0.0;
                 for (int a = 0; a < 3; ++a) {
@@ -628,7 +611,7 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                         tpb[a] = 0.0;
                     }
                 } else {
-                    const double len_before = R.t_in + R.ell + (double)ck.excess[slot];
+                    const double len_before = R.t_in + R.ell + (double)(QUASI ? s0.w : ck.excess[slot]);
                     wall_adjoint(S, rN, vN, len_before, Ib, drb, dvb, lb, CONN ? xlum : nullptr, CONN ? xlb : nullptr);
                 }
                 lenb = kept((float)lb) * sc;
@@ -642,7 +625,8 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                 const float si = sc * idt;
                 Vb = p3(kept((float)dvb[0] * si), kept((float)dvb[1] * si), kept((float)dvb[2] * si));
                 sih = mul3(sc, L.ih);
-                far_off = !(maxabs3(P3{dr.x * L.ih.x, mul2(dr.yz, L.ih.yz)}) <= 0.0625f);
+                if (QUASI) dr = P3{0.0f, 0ull};
+                far_off = !QUASI && !(maxabs3(P3{dr.x * L.ih.x, mul2(dr.yz, L.ih.yz)}) <= 0.0625f);
             }
             // A ray that ends more than a sixteenth of a cell off its line takes its state from
             // the checkpoints where there is one: its deviation's rounding, 2^-29 of a cell and
@@ -654,14 +638,24 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
             rows_clear(row);
             P3 ab = {0.0f, 0ull};             // a_ of the later step, waiting for its point
             float work = 0.0f;                // sum of a_.a + b_.b + c_.c
+            const P3 VbN = Vb;
+            P3 ulen = {0.0f, 0ull};           // quasi-linear: lenb times the unit directions so far
+            float back = 0.0f;                // and the steps reversed so far
             float tps[3] = {0.0f, 0.0f, 0.0f};
             P3 rseg = rb;
             int seg0 = n_max - to_ckpt;       // first node of the segment (the refracted sums)
-            f32x2 h = splat2(2.0f * (float)n_max);
+            int origin = n_max / kLineSteps * kLineSteps;   // the step that the line is set up from
+            if (origin > 0 && act) set_line(S, F, rs, RR, origin, L, m);
+            f32x2 h = splat2(2.0f * (float)(n_max - origin));
             bool used = false;                // the rows hold something
             bool later = false;               // a later step of this ray has been reversed
             for (int n = n_max;; --n, --to_ckpt) {
                 const bool on = n <= N;
+                if (n < origin) {   // (the next point finds its cell again)
+                    origin -= kLineSteps;
+                    if (act) set_line(S, F, rs, RR, origin, L, m);
+                    h = splat2(2.0f * (float)(n - origin));
+                }
                 // ---- the point between steps n - 1 and n
                 P3 c = {0.0f, 0ull}, q3 = c;
                 Frac3 f;
@@ -685,19 +679,22 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                     if (moved) key = march_key(m, (uint32_t)nx, (uint32_t)nxy);
                 }
                 if (on) {
-                    const PolyGrad g = poly_grad(m.p, f);
+                    const PolyGrad g = poly_point<QUASI>(m.p, f);
                     const float eta = 1.0f + lo2(g.v.lo);
                     c = march_accel(g.v, sc);
                     if (later) V = kept_state ? Vk : sub3(V, c);
                     P3 w = ab;
                     if (n > 0) {
                         w = add3(w, Vb);
-                        q3 = point_adjoint(g, record_adjoint(g, eta, Vb), sih);
+                        if (!QUASI) q3 = point_adjoint(g, record_adjoint(g, eta, Vb), sih);
                     }
                     Cell2 Q = record_adjoint(g, eta, w);
-                    const P3 q = point_adjoint(g, Q, sih);
                     work = fmaf(eta, lo2(Q.lo), work);
-                    rb = add3(rb, sub3(q, q3));
+                    P3 q = {0.0f, 0ull};
+                    if (!QUASI) {
+                        q = point_adjoint(g, Q, sih);
+                        rb = add3(rb, sub3(q, q3));
+                    }
                     if constexpr (CONN) {
                         const float tn = (float)(n - seg0);
                         const P3 q1 = sub3(q, q3);
@@ -731,29 +728,43 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                 // ---- the middle of step n - 1
                 h = add2(h, splat2(-1.0f));
                 moved = false;
-                if (on) moved = march_point<false>(F, L, m, h, fma3(0.75f, c, fma3(-0.5f, V, dr)), f);
+                if (on) moved = march_point<false>(F, L, m, h, QUASI ? dr : fma3(0.75f, c, fma3(-0.5f, V, dr)), f);
                 if (__any_sync(0xffffffffu, moved)) {
                     rows_flush(rows, moved && used, key, row, acc, nx, nxy, ncells, err);
                     if (moved) key = march_key(m, (uint32_t)nx, (uint32_t)nxy);
                 }
                 if (on) {
-                    const PolyGrad g = poly_grad(m.p, f);
+                    const PolyGrad g = poly_point<QUASI>(m.p, f);
                     const float eta = 1.0f + lo2(g.v.lo);
                     const P3 b = march_accel(g.v, sc);
                     const P3 inc = sub3(V, fma3(2.0f, b, c));          // r' - r
-                    dr = sub3(dr, inc);
+                    if (!QUASI) dr = sub3(dr, inc);
                     V = sub3(V, fma3(4.0f, b, c));                     // less a, at the next point
                     const P3 step = add3(dS, inc);
                     const float ln = lenb * rsqrtf(dot3(step, step));
                     const P3 sg = fma3(ln, step, rb);                  // r_ with the path length's share
-                    const P3 bb = fma3(2.0f, sg, fma3(4.0f, Vb, mul3(3.0f, q3)));
+                    P3 bb = mul3(4.0f, Vb), q2 = {0.0f, 0ull};
+                    if (!QUASI) bb = fma3(3.0f, q3, bb);
+                    bb = fma3(2.0f, sg, bb);
                     const Cell2 Q = record_adjoint(g, eta, bb);
-                    const P3 q2 = point_adjoint(g, Q, sih);
                     work = fmaf(eta, lo2(Q.lo), work);
                     rows_add(row, f, Q);
-                    rb = add3(rb, add3(q3, q2));
-                    ab = fma3(0.75f, q2, add3(sg, Vb));
-                    Vb = add3(Vb, fma3(0.5f, q2, add3(sg, q3)));
+                    ab = add3(sg, Vb);
+                    if (QUASI) {
+                        // r_ is constant: V_ from its closed form, whose float32 error does not
+                        // build up over the steps
+                        back += 1.0f;
+                        ulen = fma3(ln, step, ulen);
+                        Vb = add3(fma3(back, rb, VbN), ulen);
+                    } else {
+                        Vb = add3(Vb, sg);
+                    }
+                    if (!QUASI) {
+                        q2 = point_adjoint(g, Q, sih);
+                        rb = add3(rb, add3(q3, q2));
+                        ab = fma3(0.75f, q2, ab);
+                        Vb = add3(Vb, fma3(0.5f, q2, q3));
+                    }
                     later = true;
                     if constexpr (CONN) {
                         const P3 t = fma3((float)(n - seg0), q3, mul3((float)(n - seg0) - 0.5f, q2));
@@ -1080,8 +1091,8 @@ __device__ __forceinline__ void adjoint_tile(const SceneDev& S, const CkptDev& c
 // recompute (relative L2 2e-7 .. 7e-7).  128 registers and 16 warps beat 168 and 12 by 2 to 3 %;
 // with the connection, whose spills then reach the loop, 168 are 7 % faster.  Summing the rows
 // of a whole warp one cell at a time, with branches around the row reads, took 62.7 ms.
-template <class E, bool CONN>
-__global__ void __launch_bounds__(kAdjWarps * 32, CONN ? BOS_REV_CONN_MIN_BLOCKS : BOS_REV_MIN_BLOCKS)
+template <class E, bool CONN, bool QUASI, bool FEW>
+__global__ void __launch_bounds__(kAdjWarps * 32, FEW ? 1 : CONN ? BOS_REV_CONN_MIN_BLOCKS : BOS_REV_MIN_BLOCKS)
     reverse_kernel(SceneDev S, CkptDev ck, AdjDev adj, WorkDev wk) {
     extern __shared__ float4 smem4[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1097,7 +1108,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, CONN ? BOS_REV_CONN_MIN_BLOCKS
         if (lane == 0) t = atomicAdd(wk.tile_counter, 1);
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= ntiles) break;
-        reverse_tile<E, CONN>(S, ck, adj, F, ts, t, lane, rows, reinterpret_cast<float*>(adj.acc), ncells, S.g.err,
+        reverse_tile<E, CONN, QUASI>(S, ck, adj, F, ts, t, lane, rows, reinterpret_cast<float*>(adj.acc), ncells, S.g.err,
                               wk.tile_counter + 1, xlum);
     }
 }
@@ -1137,197 +1148,6 @@ __global__ void __launch_bounds__(kAdjWarps * 32, BOS_ADJ_MIN_BLOCKS) adjoint_ke
         if (t >= ntiles) break;
         if (!tile_needs_stages(ck, ts, t, lane, tile_pixel(S, ts, t, lane).valid)) continue;
         adjoint_tile<E, CONN>(S, ck, adj, F, ts, t, lane, rows, st_buf, acc, ca, xlum);
-    }
-    flush_rows(rows, ca.key != kNoKey, ca, acc, S.g.n[0], S.g.n[0] * S.g.n[1]);
-}
-
-// Adjoint of quasi-linear tracing (Sec. 2.2).  The stage points lie on the straight
-// line, so the outputs are linear in the sampled D values and no position adjoint flows
-// back through them.  Reversing a step leaves the position adjoint unchanged and adds
-// dt (r_bar + len_bar u_n) to the velocity adjoint (u_n the unit direction of step n), so
-//   v_bar_{n+1} = v_bar_N + dt (N - n - 1) r_bar + dt len_bar sum_{m > n} u_m
-// is known from the final state and a running prefix of u: one sweep in forward order
-// recomputes the samples and scatters every stage's sensitivity (the end sample of a
-// step and the start sample of the next are one point and one scatter).
-// A quasi-linear line sample: its cell and the field value only (the samples sit on the
-// straight line, so no position adjoint and hence no field gradient is needed).
-struct LineSample {
-    uint32_t key;
-    float cf[3];
-    float4 v;   // (deta, grad eta)
-};
-
-template <class E>
-__device__ __forceinline__ void line_sample(const CompField<E>& F, const long long U[3], BrickCache& bc,
-                                            LineSample& p) {
-    const float zero[3] = {0.0f, 0.0f, 0.0f};
-    int ci[3];
-    comp_cell(F, U, zero, ci, p.cf);
-    p.key = cell_key_of(F, ci);
-    p.v = trilinear2(F.store, comp_offset(F, bc, ci), p.cf[0], p.cf[1], p.cf[2]);
-}
-
-// Corner record of D = (1 + deta) grad at a line sample for the adjoint Db of D.
-__device__ __forceinline__ float4 line_corner_record(const float4 v, const float Db[3]) {
-    const float eta = 1.0f + v.x;
-    return make_float4(Db[0] * v.y + Db[1] * v.z + Db[2] * v.w, eta * Db[0], eta * Db[1], eta * Db[2]);
-}
-
-// One warp tile of the quasi-linear adjoint (one forward-order sweep per ray).
-template <class E>
-__device__ __forceinline__ void adjoint_quasi_tile(const SceneDev& S, const CkptDev& ck, const AdjDev& adj,
-                                                   const CompField<E>& F, const TileShape& ts, int t, int lane,
-                                                   float* rows, float* acc, CellAcc& ca) {
-    const int nx = S.g.n[0], nxy = S.g.n[0] * S.g.n[1];
-    const int spp = S.cam.spp;
-    const float zero[3] = {0.0f, 0.0f, 0.0f};
-    const int sl = lane % ts.G;
-    const TilePix tp = tile_pixel(S, ts, t, lane);
-    const int px = tp.px, py = tp.py;
-    const bool valid = tp.valid;
-    for (int qs = 0; qs < ts.samples_per_lane; ++qs) {
-        const int s = ts.samples_per_lane == 1 ? sl : qs;
-        const long long slot = ((long long)t * 32 + lane) * ts.samples_per_lane + qs;
-        bool act = valid;
-        Ray R;
-        R.N = 0;
-        R.wall = false;
-        double Ib = 0.0;
-        if (act) {
-            R = ray_setup(S, px, py, s);
-            Ib = (double)adj.dLdI[(size_t)tp.out] / spp;
-        }
-        act = act && R.wall && R.N > 0 && Ib != 0.0;
-        CompState st;
-        CompConst k;
-        double eta_in = 1.0, rin[3] = {0, 0, 0};
-        float rb[3] = {0, 0, 0}, vbN[3] = {0, 0, 0}, lenb = 0.0f, usum[3] = {0, 0, 0};
-        double etab = 0.0;
-        if (act) {
-            comp_setup(S, F, S.cam.pos, R, st, k, eta_in, rin);
-            const float4 s0 = ck.state[0 * ck.nrays + slot];
-            const float4 s1 = ck.state[1 * ck.nrays + slot];
-            const float4 s2 = ck.state[2 * ck.nrays + slot];
-            usum[0] = s1.w;
-            usum[1] = s2.x;
-            usum[2] = s2.y;
-            double rN[3], vN[3], drb[3], dvb[3], lb;
-            const float drN[3] = {s0.x, s0.y, s0.z}, dvN[3] = {s1.x, s1.y, s1.z};
-            for (int a = 0; a < 3; ++a) {
-                rN[a] = rin[a] + R.ell * R.d[a] + (double)drN[a];
-                vN[a] = eta_in * R.d[a] + (double)dvN[a];
-            }
-            wall_adjoint(S, rN, vN, R.t_in + R.ell + (double)s0.w, Ib, drb, dvb, lb);
-            for (int a = 0; a < 3; ++a) {
-                rb[a] = (float)drb[a];
-                vbN[a] = (float)dvb[a];
-            }
-            lenb = (float)lb;
-            etab = dvb[0] * R.d[0] + dvb[1] * R.d[1] + dvb[2] * R.d[2];
-        }
-        const int N = act ? R.N : 0;
-        const int n_max = __reduce_max_sync(0xffffffffu, (unsigned)N);
-        const float dt = act ? k.dt : 0.0f;
-        BrickCache bc = {kNoKey, 0u};
-        // the start sample of step 0
-        LineSample p0 = {};
-        float A[3] = {0, 0, 0}, dv[3] = {0, 0, 0}, prefix[3] = {0, 0, 0}, carry[3] = {0, 0, 0}, dtb = 0.0f;
-        if (act) {
-            line_sample(F, st.U, bc, p0);
-            float D[3];
-            rhs_of(p0.v, D);
-            for (int a = 0; a < 3; ++a) A[a] = dt * D[a];
-        }
-        for (int n = 0; n < n_max; ++n) {
-            const bool a_ = act && n < N;
-            LineSample pm = {}, pe = {};
-            float B[3] = {0, 0, 0}, C[3] = {0, 0, 0}, u[3] = {0, 0, 0}, Dm[3] = {0, 0, 0}, De[3] = {0, 0, 0};
-            float Db0[3] = {0, 0, 0}, Dbm[3] = {0, 0, 0};
-            if (a_) {
-                long long U2[3], U3[3];
-                for (int a = 0; a < 3; ++a) {
-                    U2[a] = st.U[a] + (long long)n * k.dU[a] + k.dUh[a];
-                    U3[a] = st.U[a] + (long long)(n + 1) * k.dU[a];
-                }
-                line_sample(F, U2, bc, pm);
-                rhs_of(pm.v, Dm);
-                line_sample(F, U3, bc, pe);
-                rhs_of(pe.v, De);
-                float inc[3], nn = 0.0f;
-                for (int a = 0; a < 3; ++a) {
-                    B[a] = dt * Dm[a];
-                    C[a] = dt * De[a];
-                    inc[a] = dt * (dv[a] + (A[a] + 2.0f * B[a]) * (1.0f / 6.0f));
-                    const float w = k.dS[a] + inc[a];
-                    u[a] = w;
-                    nn += w * w;
-                }
-                const float rn = rsqrtf(nn);
-                const float rem = (float)(N - n - 1);
-                for (int a = 0; a < 3; ++a) {
-                    u[a] *= rn;
-                    prefix[a] += u[a];
-                    const float rbp = rb[a] + lenb * u[a];                       // adjoint of r_{n+1}
-                    const float vb1 = vbN[a] + dt * rem * rb[a] + dt * lenb * (usum[a] - prefix[a]);
-                    const float Ab = (dt * (1.0f / 6.0f)) * rbp + vb1 * (1.0f / 6.0f);
-                    const float Bb = (dt * (1.0f / 3.0f)) * rbp + vb1 * (4.0f / 6.0f);
-                    const float Cb = vb1 * (1.0f / 6.0f);
-                    dtb += rbp * (dv[a] + (A[a] + 2.0f * B[a]) * (1.0f / 6.0f)) + Ab * (A[a] / dt) + Bb * Dm[a] +
-                           Cb * De[a];
-                    Db0[a] = carry[a] + dt * Ab;      // start sample: this step's A and the previous C
-                    Dbm[a] = dt * Bb;
-                    carry[a] = dt * Cb;
-                    dv[a] += (A[a] + 4.0f * B[a] + C[a]) * (1.0f / 6.0f);
-                    A[a] = C[a];
-                }
-            }
-            float4 Q = make_float4(0, 0, 0, 0), Qm = make_float4(0, 0, 0, 0);
-            if (a_) {
-                Q = line_corner_record(p0.v, Db0);
-                Qm = line_corner_record(pm.v, Dbm);
-            }
-            // the step's two samples share a cell more often than not: one row update
-            const bool same = a_ && pm.key == p0.key;
-            accumulate_dual(rows, a_, p0.key, p0.cf, Q, same, pm.cf, Qm, ca, acc, nx, nxy);
-            accumulate(rows, a_ && !same, pm.key, pm.cf, Qm, ca, acc, nx, nxy);
-            if (a_) p0 = pe;
-        }
-        // the end sample of the last step, then eta_in = 1 + deta(r_in)
-        float4 Q = make_float4(0, 0, 0, 0);
-        if (act) Q = line_corner_record(p0.v, carry);
-        accumulate(rows, act, p0.key, p0.cf, Q, ca, acc, nx, nxy);
-        int ci[3] = {0, 0, 0};
-        float cf[3] = {0, 0, 0};
-        if (act) {
-            etab -= (double)dtb * (double)dt / eta_in;
-            comp_cell(F, st.U, zero, ci, cf);
-        }
-        accumulate(rows, act, cell_key_of(F, ci), cf, make_float4((float)etab, 0.0f, 0.0f, 0.0f), ca, acc, nx, nxy);
-    }
-}
-
-template <class E, int MINB>
-__global__ void __launch_bounds__(kAdjWarps * 32, MINB)
-    adjoint_quasi_kernel(SceneDev S, CkptDev ck, AdjDev adj, WorkDev wk) {
-    extern __shared__ float4 smem4[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * 32 * kRow;
-    {
-        float4* row = reinterpret_cast<float4*>(rows + lane * kRow);
-        for (int c = 0; c < 8; ++c) row[c] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    }
-    __syncwarp();
-    const CompField<E> F = comp_field<E>(S.g);
-    const TileShape ts = tile_shape(S.cam.width, S.cam.height, S.cam.spp);
-    const int ntiles = tile_count(S, ts);
-    float* acc = reinterpret_cast<float*>(adj.acc);
-    CellAcc ca = {kNoKey, (uint32_t)S.g.n[0] * S.g.n[1] * S.g.n[2], S.g.err};
-    for (;;) {
-        int t = 0;
-        if (lane == 0) t = atomicAdd(wk.tile_counter, 1);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= ntiles) break;
-        adjoint_quasi_tile<E>(S, ck, adj, F, ts, t, lane, rows, acc, ca);
     }
     flush_rows(rows, ca.key != kNoKey, ca, acc, S.g.n[0], S.g.n[0] * S.g.n[1]);
 }
@@ -1653,17 +1473,35 @@ __global__ void __launch_bounds__(256) gradient_kernel(GridDev g, GradConst k, c
 }
 
 // Batched adjoints (the request server): one launch covers warp tiles of several jobs,
-// indexed as in render_batch_kernel.  The lane rows belong to one job's accumulators at a
-// time, so they are flushed whenever a warp moves on to another job's tile.  The Sharma
-// form's segment slices come from seg_base with room for k_max steps.
+// indexed as in render_batch_kernel.  counter: queue, tiles left to adjoint_batch_kernel, its
+// queue.
 template <class E, bool QUASI>
-__global__ void __launch_bounds__(kAdjWarps * 32, QUASI ? BOS_ADJ_QUASI_MIN_BLOCKS : BOS_ADJ_MIN_BLOCKS)
+__global__ void __launch_bounds__(kAdjWarps * 32, BOS_REV_MIN_BLOCKS)
+    reverse_batch_kernel(const BatchJob* __restrict__ jobs, int njobs, int total, int* counter) {
+    extern __shared__ float4 smem4[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * 32 * kRow;
+    for (;;) {
+        int g = 0;
+        if (lane == 0) g = atomicAdd(counter, 1);
+        g = __shfl_sync(0xffffffffu, g, 0);
+        if (g >= total) break;
+        const BatchJob& J = jobs[batch_job_of(jobs, njobs, g)];
+        reverse_tile<E, false, QUASI>(J.S, J.ck, J.adj, comp_field<E>(J.S.g),
+                                      tile_shape(J.S.cam.width, J.S.cam.height, J.S.cam.spp), J.tile0 + (g - J.first),
+                                      lane, rows, reinterpret_cast<float*>(J.adj.acc),
+                                      (uint32_t)J.S.g.n[0] * J.S.g.n[1] * J.S.g.n[2], J.S.g.err, counter + 1, nullptr);
+    }
+}
+
+// The Sharma tiles that reverse_batch_kernel left.  The lane rows belong to one job's
+// accumulators at a time, so they are flushed whenever a warp moves on to another job's tile.
+// The segment slices come from seg_base with room for k_max steps.
+template <class E>
+__global__ void __launch_bounds__(kAdjWarps * 32, BOS_ADJ_MIN_BLOCKS)
     adjoint_batch_kernel(const BatchJob* __restrict__ jobs, int njobs, int total, int* counter, float* seg_base,
                          int k_max) {
-    if (!QUASI) {   // the tiles that reverse_batch_kernel left
-        if (counter[1] == 0) return;
-        counter += 2;
-    }
+    if (counter[1] == 0) return;
     extern __shared__ float4 smem4[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * 32 * kRow;
@@ -1677,7 +1515,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, QUASI ? BOS_ADJ_QUASI_MIN_BLOC
     int cur = -1;                      // job whose accumulators the rows belong to
     for (;;) {
         int g = 0;
-        if (lane == 0) g = atomicAdd(counter, 1);
+        if (lane == 0) g = atomicAdd(counter + 2, 1);
         g = __shfl_sync(0xffffffffu, g, 0);
         if (g >= total) break;
         const int j = batch_job_of(jobs, njobs, g);
@@ -1692,37 +1530,14 @@ __global__ void __launch_bounds__(kAdjWarps * 32, QUASI ? BOS_ADJ_QUASI_MIN_BLOC
         ca.err = J.S.g.err;
         const CompField<E> F = comp_field<E>(J.S.g);
         const TileShape ts = tile_shape(J.S.cam.width, J.S.cam.height, J.S.cam.spp);
-        float* acc = reinterpret_cast<float*>(J.adj.acc);
-        if constexpr (QUASI)
-            adjoint_quasi_tile<E>(J.S, J.ck, J.adj, F, ts, J.tile0 + (g - J.first), lane, rows, acc, ca);
-        else if (tile_needs_stages(J.ck, ts, J.tile0 + (g - J.first), lane,
-                                   tile_pixel(J.S, ts, J.tile0 + (g - J.first), lane).valid))
-            adjoint_tile<E, false>(J.S, J.ck, J.adj, F, ts, J.tile0 + (g - J.first), lane, rows, st_buf, acc, ca,
-                                   nullptr);
+        const int t = J.tile0 + (g - J.first);
+        if (tile_needs_stages(J.ck, ts, t, lane, tile_pixel(J.S, ts, t, lane).valid))
+            adjoint_tile<E, false>(J.S, J.ck, J.adj, F, ts, t, lane, rows, st_buf,
+                                   reinterpret_cast<float*>(J.adj.acc), ca, nullptr);
     }
     if (cur >= 0) {
         const BatchJob& P = jobs[cur];
         flush_rows(rows, ca.key != kNoKey, ca, reinterpret_cast<float*>(P.adj.acc), P.S.g.n[0], P.S.g.n[0] * P.S.g.n[1]);
-    }
-}
-
-// reverse_kernel over several jobs' tiles; counter: queue, tiles left, queue of the rest.
-template <class E>
-__global__ void __launch_bounds__(kAdjWarps * 32, BOS_REV_MIN_BLOCKS)
-    reverse_batch_kernel(const BatchJob* __restrict__ jobs, int njobs, int total, int* counter) {
-    extern __shared__ float4 smem4[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * 32 * kRow;
-    for (;;) {
-        int g = 0;
-        if (lane == 0) g = atomicAdd(counter, 1);
-        g = __shfl_sync(0xffffffffu, g, 0);
-        if (g >= total) break;
-        const BatchJob& J = jobs[batch_job_of(jobs, njobs, g)];
-        reverse_tile<E, false>(J.S, J.ck, J.adj, comp_field<E>(J.S.g),
-                               tile_shape(J.S.cam.width, J.S.cam.height, J.S.cam.spp), J.tile0 + (g - J.first), lane, rows,
-                               reinterpret_cast<float*>(J.adj.acc), (uint32_t)J.S.g.n[0] * J.S.g.n[1] * J.S.g.n[2],
-                               J.S.g.err, counter + 1, nullptr);
     }
 }
 
@@ -1731,19 +1546,16 @@ static cudaError_t launch_adjoint_batch_c(const BatchJob* jobs, int njobs, int t
                                           int k_max, int num_sms, cudaStream_t st) {
     const size_t smem = (size_t)kAdjWarps * 32 * kRow * sizeof(float);
     int per_sm = 0;
-    cudaError_t e;
-    if constexpr (!QUASI) {
-        e = occupancy_prefer_l1(reverse_batch_kernel<E>, kAdjWarps * 32, smem, per_sm);
-        if (e != cudaSuccess) return e;
-        if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        reverse_batch_kernel<E><<<num_sms * per_sm, kAdjWarps * 32, smem, st>>>(jobs, njobs, total, counter);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    e = occupancy_prefer_l1(adjoint_batch_kernel<E, QUASI>, kAdjWarps * 32, smem, per_sm);
+    cudaError_t e = occupancy_prefer_l1(reverse_batch_kernel<E, QUASI>, kAdjWarps * 32, smem, per_sm);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    reverse_batch_kernel<E, QUASI><<<num_sms * per_sm, kAdjWarps * 32, smem, st>>>(jobs, njobs, total, counter);
+    if ((e = cudaGetLastError()) != cudaSuccess || QUASI) return e;
+    e = occupancy_prefer_l1(adjoint_batch_kernel<E>, kAdjWarps * 32, smem, per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const int blocks = num_sms * per_sm < kAdjMaxBlocks ? num_sms * per_sm : kAdjMaxBlocks;
-    adjoint_batch_kernel<E, QUASI><<<blocks, kAdjWarps * 32, smem, st>>>(jobs, njobs, total, counter, seg_base, k_max);
+    adjoint_batch_kernel<E><<<blocks, kAdjWarps * 32, smem, st>>>(jobs, njobs, total, counter, seg_base, k_max);
     return cudaGetLastError();
 }
 
@@ -1774,6 +1586,29 @@ cudaError_t launch_gradient(const GridDev& g, const float4* acc, const float* T,
     return cudaGetLastError();
 }
 
+template <class E, bool CONN, bool QUASI, bool FEW>
+static cudaError_t launch_reverse_f(const SceneDev& S, const CkptDev& ck, const AdjDev& adj, const WorkDev& w,
+                                    int num_sms, cudaStream_t st) {
+    const size_t smem = (size_t)kAdjWarps * 32 * kRow * sizeof(float);
+    int per_sm = 0;
+    cudaError_t e = occupancy_prefer_l1(reverse_kernel<E, CONN, QUASI, FEW>, kAdjWarps * 32, smem, per_sm);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    reverse_kernel<E, CONN, QUASI, FEW><<<num_sms * per_sm, kAdjWarps * 32, smem, st>>>(S, ck, adj, w);
+    return cudaGetLastError();
+}
+
+// Launches of at most kFewTiles warp tiles per SM take the form without a register cap (~230
+// registers, which leaves 8 warps per SM resident): the GPU is not full either way and each
+// ray finishes sooner without spills.
+template <class E, bool CONN, bool QUASI>
+static cudaError_t launch_reverse(const SceneDev& S, const CkptDev& ck, const AdjDev& adj, const WorkDev& w, int num_sms,
+                                  cudaStream_t st) {
+    if (QUASI && tile_count(S, tile_shape(S.cam.width, S.cam.height, S.cam.spp)) <= num_sms * kFewTiles)
+        return launch_reverse_f<E, CONN, QUASI, QUASI>(S, ck, adj, w, num_sms, st);
+    return launch_reverse_f<E, CONN, QUASI, false>(S, ck, adj, w, num_sms, st);
+}
+
 template <class E, bool CONN>
 static cudaError_t launch_adjoint_c(const SceneDev& S, const CkptDev& ck, const AdjDev& adj, const WorkDev& w,
                                     int num_sms, cudaStream_t st) {
@@ -1785,12 +1620,8 @@ static cudaError_t launch_adjoint_c(const SceneDev& S, const CkptDev& ck, const 
     e = occupancy_prefer_l1(adjoint_kernel<E, CONN>, kAdjWarps * 32, smem, per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1 || adj.seg == nullptr) return cudaErrorInvalidConfiguration;
-    int rev_per_sm = 0;
-    e = occupancy_prefer_l1(reverse_kernel<E, CONN>, kAdjWarps * 32, smem, rev_per_sm);
+    e = launch_reverse<E, CONN, false>(S, ck, adj, w, num_sms, st);
     if (e != cudaSuccess) return e;
-    if (rev_per_sm < 1) return cudaErrorInvalidConfiguration;
-    reverse_kernel<E, CONN><<<num_sms * rev_per_sm, kAdjWarps * 32, smem, st>>>(S, ck, adj, w);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int blocks = num_sms * per_sm < kAdjMaxBlocks ? num_sms * per_sm : kAdjMaxBlocks;
     adjoint_kernel<E, CONN><<<blocks, kAdjWarps * 32, smem, st>>>(S, ck, adj, w);
     return cudaGetLastError();
@@ -1806,30 +1637,6 @@ static cudaError_t launch_adjoint_t(const SceneDev& S, const CkptDev& ck, const 
         return launch_adjoint_c<E, true>(S, ck, adj, w, num_sms, st);
     }
     return launch_adjoint_c<E, false>(S, ck, adj, w, num_sms, st);
-}
-
-template <class E, int MINB>
-static cudaError_t launch_adjoint_quasi_b(const SceneDev& S, const CkptDev& ck, const AdjDev& adj, const WorkDev& w,
-                                          int num_sms, cudaStream_t st) {
-    size_t smem = (size_t)kAdjWarps * 32 * kRow * sizeof(float);
-    int per_sm = 0;
-    cudaError_t e = occupancy_prefer_l1(adjoint_quasi_kernel<E, MINB>, kAdjWarps * 32, smem, per_sm);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    adjoint_quasi_kernel<E, MINB><<<num_sms * per_sm, kAdjWarps * 32, smem, st>>>(S, ck, adj, w);
-    return cudaGetLastError();
-}
-
-// Two register budgets of the quasi-linear adjoint: with more than 12 warp tiles per SM,
-// the 128-register form's 16 resident warps per SM hide more latency; with fewer (a
-// 5000-pixel minibatch is ~300 tiles) the GPU is not full either way, and the form without
-// a register cap (180-200 registers, no spills) finishes each ray sooner.
-template <class E>
-static cudaError_t launch_adjoint_quasi_t(const SceneDev& S, const CkptDev& ck, const AdjDev& adj, const WorkDev& w,
-                                          int num_sms, cudaStream_t st) {
-    const int ntiles = tile_count(S, tile_shape(S.cam.width, S.cam.height, S.cam.spp));
-    if (ntiles > num_sms * 12) return launch_adjoint_quasi_b<E, BOS_ADJ_QUASI_MIN_BLOCKS>(S, ck, adj, w, num_sms, st);
-    return launch_adjoint_quasi_b<E, BOS_ADJ_QUASI_SMALL_MIN_BLOCKS>(S, ck, adj, w, num_sms, st);
 }
 
 // Float64 store and tracer: Sharma RKN, float64 accumulators; seed and dL/dT in float32 or
@@ -1854,9 +1661,9 @@ cudaError_t launch_backward(int mode, const SceneDev& S, const CkptDev& ck, cons
     if (!quasi && ck.every > 64) return cudaErrorNotSupported;
     cudaError_t e;
     if (mode == 4) return launch_backward_fp64(S, ck, adj, w, T, dLdT, false, num_sms, st);
-    if (mode == 1) e = quasi ? launch_adjoint_quasi_t<F4P>(S, ck, adj, w, num_sms, st)
+    if (mode == 1) e = quasi ? launch_reverse<F4P, false, true>(S, ck, adj, w, num_sms, st)
                              : launch_adjoint_t<F4P>(S, ck, adj, w, num_sms, st);
-    else if (mode == 2) e = quasi ? launch_adjoint_quasi_t<B4P>(S, ck, adj, w, num_sms, st)
+    else if (mode == 2) e = quasi ? launch_reverse<B4P, false, true>(S, ck, adj, w, num_sms, st)
                                   : launch_adjoint_t<B4P>(S, ck, adj, w, num_sms, st);
     else return cudaErrorNotSupported;
     return e == cudaSuccess ? launch_gradient(S.g, adj.acc, T, dLdT, st) : e;

@@ -355,7 +355,6 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
         const float zero[3] = {0.0f, 0.0f, 0.0f};
         int ci[3];
         float cf[3], A[3], B[3], C[3], D[3];
-        float usum[3] = {0.0f, 0.0f, 0.0f};
         const float dt = k.dt;
         rhs_of(comp_eval(F, st.U, zero, bc, ci, cf), D);
         for (int a = 0; a < 3; ++a) A[a] = dt * D[a];
@@ -381,11 +380,6 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
             float ii = inc_r[0] * inc_r[0] + inc_r[1] * inc_r[1] + inc_r[2] * inc_r[2];
             float di = k.dhat[0] * inc_r[0] + k.dhat[1] * inc_r[1] + k.dhat[2] * inc_r[2];
             st.excess += __fdividef(2.0f * si + ii, 2.0f * k.step_len + di);
-            if (state != nullptr) {          // sum of the unit step directions, for the adjoint
-                float w[3] = {k.dS[0] + inc_r[0], k.dS[1] + inc_r[1], k.dS[2] + inc_r[2]};
-                float rn = rsqrtf(w[0] * w[0] + w[1] * w[1] + w[2] * w[2]);
-                for (int a = 0; a < 3; ++a) usum[a] += w[a] * rn;
-            }
             for (int a = 0; a < 3; ++a) {
                 kahan_add(st.dr[a], st.cr[a], inc_r[a]);
                 kahan_add(st.dv[a], st.cv[a], inc_v[a]);
@@ -393,12 +387,11 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
                 A[a] = C[a];
             }
         }
-        if (state != nullptr) {   // the final state, for the one-sweep adjoint
+        if (state != nullptr) {   // the end state, from which the adjoint reverses the ray
             state[0 * ck.nrays + ray] = make_float4(st.dr[0] - st.cr[0], st.dr[1] - st.cr[1], st.dr[2] - st.cr[2],
                                                        st.excess);
             state[1 * ck.nrays + ray] = make_float4(st.dv[0] - st.cv[0], st.dv[1] - st.cv[1], st.dv[2] - st.cv[2],
-                                                       usum[0]);
-            state[2 * ck.nrays + ray] = make_float4(usum[1], usum[2], 0.0f, 0.0f);
+                                                       0.0f);
         }
     } else if constexpr (INTEG == 0 && BOS_FWD_PIPELINE) {
         // Sharma steps, software-pipelined: the next step's first stage needs only the new
@@ -475,7 +468,7 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
             // steps that the adjoint can reverse without their stage terms: dt |A - B| / 6 within
             // kSameReverse cells (not so: NaN, too)
             const float ih = fmaxf(F.inv_h[0], fmaxf(F.inv_h[1], F.inv_h[2]));
-            *apart_cells = R.N > kLineSteps ? __int_as_float(0x7f800000) : apart * dt * (ih * (1.0f / 6.0f));
+            *apart_cells = apart * dt * (ih * (1.0f / 6.0f));
         }
     } else {
         for (int n = 0; n < R.N; ++n) {

@@ -49,6 +49,10 @@ struct RenderOut {
     double* hit;
 };
 
+// Warp tiles per SM up to which a launch takes a tracer's form without a register cap: what
+// such a form (180 to 240 registers) keeps resident.
+constexpr int kFewTiles = 8;
+
 constexpr size_t kTileCounterBytes = 3 * sizeof(int);
 
 struct WorkDev {

@@ -75,6 +75,13 @@ def test_reversed_adjoint_matches_oracle(bos, orc, name):
     assert gradient_error(bos, orc, smooth(ALL[name]()), bos.BOS_PREC_FP32_COMP) <= GRAD_REL_L2
 
 
+@pytest.mark.parametrize("name", ["steep", "diagonal", "two_cells", "uneven_cells", "three_samples", "bent_K16"])
+def test_reversed_quasi_linear_adjoint_matches_oracle(bos, orc, name):
+    sc = smooth(ALL[name]())
+    sc = sc.replace(integ=dataclasses.replace(sc.integ, integrator=2))
+    assert gradient_error(bos, orc, sc, bos.BOS_PREC_FP32_COMP) <= GRAD_REL_L2
+
+
 @pytest.mark.parametrize("name", ["partly_steep", "uneven_cells", "three_samples"])
 def test_reversed_refracted_adjoint_matches_oracle(bos, orc, name):
     sc = smooth(ALL[name]())
