@@ -1604,8 +1604,8 @@ static cudaError_t launch_reverse_f(const SceneDev& S, const CkptDev& ck, const 
 template <class E, bool CONN, bool QUASI>
 static cudaError_t launch_reverse(const SceneDev& S, const CkptDev& ck, const AdjDev& adj, const WorkDev& w, int num_sms,
                                   cudaStream_t st) {
-    if (QUASI && tile_count(S, tile_shape(S.cam.width, S.cam.height, S.cam.spp)) <= num_sms * kFewTiles)
-        return launch_reverse_f<E, CONN, QUASI, QUASI>(S, ck, adj, w, num_sms, st);
+    if (tile_count(S, tile_shape(S.cam.width, S.cam.height, S.cam.spp)) <= num_sms * kFewTiles)
+        return launch_reverse_f<E, CONN, QUASI, true>(S, ck, adj, w, num_sms, st);
     return launch_reverse_f<E, CONN, QUASI, false>(S, ck, adj, w, num_sms, st);
 }
 

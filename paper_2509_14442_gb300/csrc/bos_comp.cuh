@@ -332,9 +332,13 @@ __device__ __forceinline__ WallRel comp_wall(const SceneDev& S, const Ray& R, do
     const float cd = df[0] * nf[0] + df[1] * nf[1] + df[2] * nf[2];
     const float Lrem = (float)(R.tw - R.t_in - R.ell);
     const float e = (float)eta_in;
-    const float ndr = nf[0] * dr[0] + nf[1] * dr[1] + nf[2] * dr[2];
-    const float ndv = nf[0] * dv[0] + nf[1] * dv[1] + nf[2] * dv[2];
-    const float den = e * cd + ndv;                       // <n, v_N>
+    // Explicitly rounded: left to the assembler, a product and a sum are fused or not depending
+    // on the kernel's register budget, and an image must not depend on which form rendered it.
+    auto dot = [](const float x[3], const float y[3]) {
+        return fmaf(x[2], y[2], fmaf(x[1], y[1], __fmul_rn(x[0], y[0])));
+    };
+    const float ndr = dot(nf, dr), ndv = dot(nf, dv);
+    const float den = fmaf(e, cd, ndv);                       // <n, v_N>
     h.valid = den > 0.0f;
     if (!h.valid) {
         h.dx[0] = h.dx[1] = h.dx[2] = 0.0f;
@@ -342,12 +346,12 @@ __device__ __forceinline__ WallRel comp_wall(const SceneDev& S, const Ray& R, do
         return h;
     }
     const float iden = 1.0f / den;
-    const float ts = (Lrem * cd - ndr) * iden;
-    const float kk = -(e * ndr + Lrem * ndv) * iden;
-    for (int a = 0; a < 3; ++a) h.dx[a] = dr[a] + ts * dv[a] + kk * df[a];
-    const float ddv = df[0] * dv[0] + df[1] * dv[1] + df[2] * dv[2];
-    const float vl = sqrtf(e * e + 2.0f * e * ddv + (dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2]));
-    h.len = (float)(R.t_in + R.ell) + (excess + ts * vl);   // signed continuation t* |v|
+    const float ts = __fmul_rn(fmaf(Lrem, cd, -ndr), iden);
+    const float kk = -__fmul_rn(fmaf(Lrem, ndv, __fmul_rn(e, ndr)), iden);
+    for (int a = 0; a < 3; ++a) h.dx[a] = fmaf(kk, df[a], fmaf(ts, dv[a], dr[a]));
+    const float ddv = dot(df, dv);
+    const float vl = sqrtf(__fadd_rn(fmaf(e, e, __fmul_rn(__fmul_rn(2.0f, e), ddv)), dot(dv, dv)));
+    h.len = __fadd_rn((float)(R.t_in + R.ell), fmaf(ts, vl, excess));   // signed continuation t* |v|
     h.cosw = den / vl;
     return h;
 }

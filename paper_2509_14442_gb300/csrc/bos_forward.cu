@@ -413,28 +413,32 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
                 state[(c * 3 + 1) * ck.nrays + ray] = make_float4(st.dv[0], st.dv[1], st.dv[2], st.cr[1]);
                 state[(c * 3 + 2) * ck.nrays + ray] = make_float4(st.cv[0], st.cv[1], st.cv[2], st.cr[2]);
             }
-            float B[3], C[3], q[3], inc_r[3], inc_v[3];
+            // Every operation is explicitly rounded: left to the assembler, a product and a sum are
+            // fused or not depending on the kernel's register budget.
+            float B[3], q[3], inc_r[3];
             long long U2[3], U3[3];
             for (int a = 0; a < 3; ++a) {
-                q[a] = st.dr[a] + (0.5f * dt) * st.dv[a] + (0.125f * dt) * A[a];
+                q[a] = fmaf(__fmul_rn(0.125f, dt), A[a], fmaf(__fmul_rn(0.5f, dt), st.dv[a], st.dr[a]));
                 U2[a] = st.U[a] + k.dUh[a];
                 U3[a] = st.U[a] + k.dU[a];
             }
             --left;
             rhs_of(eval(U2, q, bc, ci, cf), D);
             for (int a = 0; a < 3; ++a) {
-                B[a] = dt * D[a];
+                B[a] = __fmul_rn(dt, D[a]);
                 apart = fmaxf(apart, fabsf(A[a] - B[a]));
             }
+            float X[3];
             for (int a = 0; a < 3; ++a) {
-                q[a] = st.dr[a] + dt * st.dv[a] + (0.5f * dt) * B[a];
-                inc_r[a] = dt * (st.dv[a] + (A[a] + 2.0f * B[a]) * (1.0f / 6.0f));
+                q[a] = fmaf(__fmul_rn(0.5f, dt), B[a], fmaf(dt, st.dv[a], st.dr[a]));
+                X[a] = fmaf(fmaf(2.0f, B[a], A[a]), 1.0f / 6.0f, st.dv[a]);
+                inc_r[a] = __fmul_rn(dt, X[a]);
             }
             float dr1[3], cr1[3];
             for (int a = 0; a < 3; ++a) {
-                dr1[a] = st.dr[a];
-                cr1[a] = st.cr[a];
-                kahan_add(dr1[a], cr1[a], inc_r[a]);
+                const float y = fmaf(dt, X[a], -st.cr[a]);
+                dr1[a] = __fadd_rn(st.dr[a], y);
+                cr1[a] = __fsub_rn(__fsub_rn(dr1[a], st.dr[a]), y);
             }
             // independent: stage 3 of this step and stage 1 of the next
             float D1[3] = {0.0f, 0.0f, 0.0f};
@@ -444,10 +448,6 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
                 float cf1[3];
                 rhs_of(eval(U3, dr1, bc1, ci1, cf1), D1);
             }
-            for (int a = 0; a < 3; ++a) {
-                C[a] = dt * D[a];
-                inc_v[a] = (A[a] + 4.0f * B[a] + C[a]) * (1.0f / 6.0f);
-            }
             float si = k.dS[0] * inc_r[0] + k.dS[1] * inc_r[1] + k.dS[2] * inc_r[2];
             float ii = inc_r[0] * inc_r[0] + inc_r[1] * inc_r[1] + inc_r[2] * inc_r[2];
             float di = k.dhat[0] * inc_r[0] + k.dhat[1] * inc_r[1] + k.dhat[2] * inc_r[2];
@@ -455,9 +455,14 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
             for (int a = 0; a < 3; ++a) {
                 st.dr[a] = dr1[a];
                 st.cr[a] = cr1[a];
-                kahan_add(st.dv[a], st.cv[a], inc_v[a]);
+                const float s4 = fmaf(4.0f, B[a], A[a]);
+                const float sv = fmaf(dt, D[a], s4);
+                const float y = fmaf(sv, 1.0f / 6.0f, -st.cv[a]);
+                const float v1 = __fadd_rn(st.dv[a], y);
+                st.cv[a] = __fsub_rn(__fsub_rn(v1, st.dv[a]), y);
+                st.dv[a] = v1;
                 st.U[a] = U3[a];
-                A[a] = dt * D1[a];
+                A[a] = __fmul_rn(dt, D1[a]);
             }
         }
         if (state != nullptr) {
@@ -892,18 +897,19 @@ template <int MODE, int INTEG>
 static cudaError_t launch_render_t(const SceneDev& S, const RenderOut& o, const WorkDev& w, const CkptDev& ck,
                                    int num_sms, cudaStream_t st) {
     if constexpr (MODE == 1 || MODE == 2) {
+        const bool few = tile_count(S, tile_shape(S.cam.width, S.cam.height, S.cam.spp)) <= num_sms * kFewTiles;
         // Sharma without checkpoints marches from cell to cell; with them the image, which seeds
         // a gradient, keeps the stage-by-stage arithmetic that the adjoint's recompute repeats
         if constexpr (INTEG == 0) {
             if (ck.state == nullptr)
                 return S.L.mode == 2 ? launch_render_c<MODE, INTEG, true, false, false>(S, o, w, ck, num_sms, st)
-                                     : launch_render_c<MODE, INTEG, false, false, false>(S, o, w, ck, num_sms, st);
+                       : few ? launch_render_c<MODE, INTEG, false, true, false>(S, o, w, ck, num_sms, st)
+                             : launch_render_c<MODE, INTEG, false, false, false>(S, o, w, ck, num_sms, st);
         }
         if (S.L.mode == 2) return launch_render_c<MODE, INTEG, true>(S, o, w, ck, num_sms, st);
-        // quasi-linear tracing of a few tiles (up to 8 warps per SM): the uncapped form
-        if constexpr (INTEG == 2) {
-            if (tile_count(S, tile_shape(S.cam.width, S.cam.height, S.cam.spp)) <= num_sms * 8)
-                return launch_render_c<MODE, INTEG, false, true>(S, o, w, ck, num_sms, st);
+        // a few tiles (up to 8 warps per SM): the uncapped form
+        if constexpr (INTEG != 1) {
+            if (few) return launch_render_c<MODE, INTEG, false, true>(S, o, w, ck, num_sms, st);
         }
     }
     return launch_render_c<MODE, INTEG, false>(S, o, w, ck, num_sms, st);
