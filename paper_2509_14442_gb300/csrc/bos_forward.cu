@@ -248,6 +248,28 @@ struct Sums {
     double I, du, dv, hu, hv;
 };
 
+// A ray's float64 set-up values wait in shared memory while it is traced.  Kept in registers
+// they cost 12, and the assembler then repeats conversions of them to float32 inside the loop
+// to save others: three per step, which held the float64 pipe at 47 % of a render.
+constexpr int kRenderThreads = 128;
+template <int SLOT>
+__device__ __forceinline__ volatile double* ray_park() {
+    __shared__ double buf[6 * kRenderThreads];
+    return buf + threadIdx.x;
+}
+__device__ __forceinline__ void park_ray(volatile double* p, const Ray& R) {
+    for (int a = 0; a < 3; ++a) p[a * kRenderThreads] = R.d[a];
+    p[3 * kRenderThreads] = R.tw;
+    p[4 * kRenderThreads] = R.t_in;
+    p[5 * kRenderThreads] = R.ell;
+}
+__device__ __forceinline__ void unpark_ray(volatile double* p, Ray& R) {
+    for (int a = 0; a < 3; ++a) R.d[a] = p[a * kRenderThreads];
+    R.tw = p[3 * kRenderThreads];
+    R.t_in = p[4 * kRenderThreads];
+    R.ell = p[5 * kRenderThreads];
+}
+
 // Sharma steps of one ray through the cell marcher, in the scaled variables V = dt dv and
 // a = (dt^2 / 6) D (metres per step), so that
 //   p2 = S(n+1/2) + dr + V/2 + 3a/4,   p3 = S(n+1) + dr + V + 3b
@@ -261,7 +283,8 @@ struct Sums {
 // the first term is the end deviation, so only the small second one is summed.
 template <class E>
 __device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
-                                          float dr_end[3], float dv_end[3], float& excess_end, double& eta_in) {
+                                          volatile double* park, float dr_end[3], float dv_end[3], float& excess_end,
+                                          float& eta_out) {
     MarchLine L;
     MarchCell m;
     const double sl = R.ell / (double)R.N;
@@ -278,7 +301,8 @@ __device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>&
     float excess = 0.0f;
     f32x2 h = 0ull;   // half step, in both halves
     const Cell2 v0 = march_value<true>(F, L, m, h, dr);
-    eta_in = 1.0 + (double)lo2(v0.lo);
+    const double eta_in = 1.0 + (double)lo2(v0.lo);
+    eta_out = __fadd_rn(1.0f, lo2(v0.lo));
     // dt = (ell / N) / eta_in; dt^2 / 6 scales every acceleration of the ray, so it is rounded
     // once, from float64 (one Newton step on the float32 reciprocal)
     const double ie0 = (double)(1.0f / (float)eta_in), dt = sl * (ie0 * (2.0 - eta_in * ie0));
@@ -287,10 +311,11 @@ __device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>&
     int n = 0;
     while (n < R.N) {
         if (lo2(h) >= 2.0f * kLineSteps) {
+            Ray Q;
+            unpark_ray(park, Q);
             for (int q = 0; q < 3; ++q) {
-                u0[q] = (rs[q] + R.t_in * R.d[q] - S.g.origin[q]) * S.g.inv_h[q] - 0.5 +
-                        2.0 * n * ((0.5 * sl) * R.d[q] * S.g.inv_h[q]);
-                du[q] = (0.5 * sl) * R.d[q] * S.g.inv_h[q];
+                du[q] = (0.5 * (Q.ell / (double)R.N)) * Q.d[q] * S.g.inv_h[q];
+                u0[q] = (rs[q] + Q.t_in * Q.d[q] - S.g.origin[q]) * S.g.inv_h[q] - 0.5 + 2.0 * n * du[q];
             }
             march_line(F.inv_h, u0, du, L, m);   // the cell is found again: back to cell 0 first
             h = 0ull;
@@ -326,11 +351,147 @@ __device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>&
     excess_end = excess + dot3(d, e);
 }
 
+// Sharma steps of one ray with checkpoints, stage by stage on the 32.32 fixed-point line: the
+// arithmetic whose result seeds a gradient and which adjoint_kernel repeats.  Every operation
+// is explicitly rounded (left to the assembler, a product and a sum are fused or not depending
+// on the register budget), in packed pairs where three components do the same.  The next
+// step's first stage needs only the new position, not C, so it is evaluated beside this
+// step's third stage.
+//
+// The ray keeps its last cell's four paired records and that cell's indices: a point whose line
+// position is in the same cell and whose fractions are in [0, 1) takes the records as they
+// are, without an address.
+//
+// What bounds it: instruction issue (58 %) and the FMA pipe (48 %) at 16 warps per SM.  256x256x192
+// cells, 2048^2 rays with checkpoints: 28.7 ms with an address per point and scalar updates,
+// 21.8 ms so (27.1 ms with the address kept and explicit rounding only, 25.6 without the
+// address, 23.9 with the equal-fractions test, 21.8 with the ray parked); 96 registers and 20
+// warps 24.1 ms, 168 and 12 23.3 ms.  Same bits.  With the refracted connection 168 registers are
+// best (1.79 ms; 128: 2.08; 96: 2.85; before: 2.11, 128x128x96 cells at 512^2).
+struct StageCell {
+    int c[3];
+    BrickCache bc;
+    Cell2 v[4], d[4];      // pairs at o, o + 9, o + 81, o + 90: records and x differences
+};
+
+// Fraction of a line position's low words.
+__device__ __forceinline__ P3 line_frac(const long long U[3]) {
+    auto fr = [](long long u) { return __fsub_rn(__uint_as_float(((uint32_t)u >> 9) | 0x3f800000u), 1.0f); };   // see comp_cell
+    return p3(fr(U[0]), fr(U[1]), fr(U[2]));
+}
+
+// D = (1 + deta) grad eta at line position U (fractions fr) plus deviation q.
+template <class E>
+__device__ __forceinline__ P3 stage_rhs(const CompField<E>& F, const long long U[3], P3 fr, P3 ih, P3 q, StageCell& m) {
+    const P3 u = P3{fmaf(q.x, ih.x, fr.x), fma2(q.yz, ih.yz, fr.yz)};
+    float f[3] = {u.x, lo2(u.yz), hi2(u.yz)};
+    const int c0 = (int)(U[0] >> 32), c1 = (int)(U[1] >> 32), c2 = (int)(U[2] >> 32);
+    const uint32_t top = max(__float_as_uint(f[0]), max(__float_as_uint(f[1]), __float_as_uint(f[2])));
+    if (top >= 0x3f800000u || ((c0 ^ m.c[0]) | (c1 ^ m.c[1]) | (c2 ^ m.c[2])) != 0) {
+        int ci[3] = {c0, c1, c2};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {   // comp_cell's clamping (a no-op inside the grid)
+            const float fl = floorf(f[a]);
+            const int I = ci[a] + (int)fl;
+            ci[a] = min(max(I, 0), F.n[a] - 2);
+            f[a] = __fadd_rn(__fsub_rn(f[a], fl), (float)(I - ci[a]));
+        }
+        if (((ci[0] ^ m.c[0]) | (ci[1] ^ m.c[1]) | (ci[2] ^ m.c[2])) != 0) {
+            m.c[0] = ci[0], m.c[1] = ci[1], m.c[2] = ci[2];
+            const uint32_t o = comp_offset(F, m.bc, ci);
+            load_rec(F.store, o, m.v[0], m.d[0]);
+            load_rec(F.store, o + 9, m.v[1], m.d[1]);
+            load_rec(F.store, o + 81, m.v[2], m.d[2]);
+            load_rec(F.store, o + 90, m.v[3], m.d[3]);
+        }
+    }
+    const f32x2 t0 = splat2(f[0]), t1 = splat2(f[1]), t2 = splat2(f[2]);
+    Cell2 a[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] = Cell2{fma2(t0, m.d[i].lo, m.v[i].lo), fma2(t0, m.d[i].hi, m.v[i].hi)};
+    const Cell2 r = lerpc(lerpc(a[0], a[1], t1), lerpc(a[2], a[3], t1), t2);
+    const float eta = __fadd_rn(1.0f, lo2(r.lo));
+    return P3{__fmul_rn(eta, hi2(r.lo)), mul2(splat2(eta), r.hi)};
+}
+
+template <class E>
+__device__ __forceinline__ void stage_run(const CompField<E>& F, const Ray& R, const CompConst& k, const CkptDev& ck,
+                                          float4* state, long long ray, CompState& st, float* apart_cells) {
+    const P3 ih = p3(F.inv_h[0], F.inv_h[1], F.inv_h[2]);
+    const P3 d = p3(kept(k.dhat[0]), kept(k.dhat[1]), kept(k.dhat[2]));
+    const float dt = kept(k.dt), len2 = kept(2.0f * k.step_len);
+    const float h1 = __fmul_rn(0.5f, dt), e1 = __fmul_rn(0.125f, dt);
+    long long U[3], dU[3];
+    for (int a = 0; a < 3; ++a) {
+        U[a] = st.U[a];
+        dU[a] = k.dU[a];
+        asm volatile("" : "+l"(U[a]), "+l"(dU[a]));   // see kept()
+    }
+    StageCell m;
+    m.c[0] = m.c[1] = m.c[2] = -2;   // no cell
+    m.bc = {0xffffffffu, 0u};
+    P3 dr = {0.0f, 0ull}, cr = dr, dv = dr, cv = dr;
+    float excess = 0.0f, apart = 0.0f;   // apart: largest |A - B| of the steps
+    P3 A = mul3(dt, stage_rhs(F, U, line_frac(U), ih, dr, m));
+    const int K = ck.every;
+    int left = K;                        // steps before the next checkpoint
+    for (int n = 0; n < R.N; ++n) {
+        if (state != nullptr && left == 0) {
+            left = K;
+            const size_t c = bounded((size_t)(n / K), (size_t)ck.max_ckpt, ck.err);
+            state[(c * 3 + 0) * ck.nrays + ray] = make_float4(dr.x, lo2(dr.yz), hi2(dr.yz), cr.x);
+            state[(c * 3 + 1) * ck.nrays + ray] = make_float4(dv.x, lo2(dv.yz), hi2(dv.yz), lo2(cr.yz));
+            state[(c * 3 + 2) * ck.nrays + ray] = make_float4(cv.x, lo2(cv.yz), hi2(cv.yz), hi2(cr.yz));
+        }
+        --left;
+        long long U2[3];
+        for (int a = 0; a < 3; ++a) {
+            U2[a] = U[a] + (dU[a] >> 1);
+            U[a] += dU[a];
+        }
+        const P3 B = mul3(dt, stage_rhs(F, U2, line_frac(U2), ih, fma3(e1, A, fma3(h1, dv, dr)), m));
+        apart = fmaxf(apart, maxabs3(sub3(A, B)));
+        const P3 q = fma3(h1, B, fma3(dt, dv, dr));
+        const P3 X = fma3(1.0f / 6.0f, fma3(2.0f, B, A), dv);
+        const P3 inc = mul3(dt, X);
+        const P3 y = P3{fmaf(dt, X.x, -cr.x), fma2(splat2(dt), X.yz, neg2(cr.yz))};
+        const P3 fr = line_frac(U);
+        const P3 D = stage_rhs(F, U, fr, ih, q, m);
+        kahan3(dr, cr, y);
+        // the third stage's point and the new position differ by second order in the step: where
+        // their fractions round to the same bits, so does D there
+        P3 A1 = {0.0f, 0ull};
+        const P3 u1 = P3{fmaf(q.x, ih.x, fr.x), fma2(q.yz, ih.yz, fr.yz)};
+        const P3 u2 = P3{fmaf(dr.x, ih.x, fr.x), fma2(dr.yz, ih.yz, fr.yz)};
+        if (u1.yz == u2.yz && __float_as_uint(u1.x) == __float_as_uint(u2.x)) A1 = mul3(dt, D);
+        else if (n + 1 < R.N) A1 = mul3(dt, stage_rhs(F, U, fr, ih, dr, m));
+        const P3 s = fma3(dt, D, fma3(4.0f, B, A));
+        kahan3(dv, cv, P3{fmaf(s.x, 1.0f / 6.0f, -cv.x), fma2(s.yz, splat2(1.0f / 6.0f), neg2(cv.yz))});
+        A = A1;
+        // |dS + inc| - |dS|, dS = L d:  d.inc (summed as the end deviation) plus the rest
+        const float di = dot3(d, inc);
+        excess = fmaf(fmaf(-di, di, dot3(inc, inc)), rcp_approx(__fadd_rn(len2, di)), excess);
+    }
+    st.dr[0] = dr.x, st.dr[1] = lo2(dr.yz), st.dr[2] = hi2(dr.yz);
+    st.cr[0] = cr.x, st.cr[1] = lo2(cr.yz), st.cr[2] = hi2(cr.yz);
+    st.dv[0] = dv.x, st.dv[1] = lo2(dv.yz), st.dv[2] = hi2(dv.yz);
+    st.cv[0] = cv.x, st.cv[1] = lo2(cv.yz), st.cv[2] = hi2(cv.yz);
+    st.excess = __fadd_rn(excess, dot3(d, sub3(dr, cr)));
+    if (state != nullptr) {
+        // the first checkpoint is the entry state, which is zero: its slot holds the end state
+        state[0 * ck.nrays + ray] = make_float4(st.dr[0], st.dr[1], st.dr[2], st.cr[0]);
+        state[1 * ck.nrays + ray] = make_float4(st.dv[0], st.dv[1], st.dv[2], st.cr[1]);
+        state[2 * ck.nrays + ray] = make_float4(st.cv[0], st.cv[1], st.cv[2], st.cr[2]);
+        // steps that the adjoint can reverse without their stage terms: dt |A - B| / 6 within
+        // kSameReverse cells (not so: NaN, too)
+        const float ihm = fmaxf(F.inv_h[0], fmaxf(F.inv_h[1], F.inv_h[2]));
+        *apart_cells = apart * dt * (ihm * (1.0f / 6.0f));
+    }
+}
+
 // Integrate one ray of the comp path (N > 0) from the pinhole rs; optionally store its
-// checkpoints every K steps in `state` (slot `ray`).  Leaves the end state in st.  CACHE:
-// the Sharma stages go through the ray's cell cache (the refracted connection's kernels,
-// which hold a second ray's state, go without: at 96 registers they spill).
-template <class E, int INTEG, bool CACHE>
+// checkpoints every K steps in `state` (slot `ray`).  Leaves the end state in st.
+template <class E, int INTEG>
 __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
                                          const CkptDev& ck, float4* state, long long ray, CompState& st,
                                          double& eta_in, float* apart_cells) {
@@ -338,16 +499,7 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
     double rin[3];
     comp_setup(S, F, rs, R, st, k, eta_in, rin);
     BrickCache bc = {0xffffffffu, 0u};
-    CellRecs cr;
-    cr.o = 0xffffffffu;
-    auto eval = [&](const long long U[3], const float q[3], BrickCache& b, int ci[3], float cf[3]) {
-        if constexpr (CACHE) return comp_eval_c(F, U, q, b, cr, ci, cf);
-        else return comp_eval(F, U, q, b, ci, cf);
-    };
     const int K = ck.every;
-#ifndef BOS_FWD_PIPELINE
-#define BOS_FWD_PIPELINE 1
-#endif
     if constexpr (INTEG == 2) {
         // Quasi-linear tracing (Sec. 2.2): the field is sampled on the straight line at the
         // start, middle and end of every step (Sharma's weights); the end sample is the next
@@ -393,88 +545,8 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
             state[1 * ck.nrays + ray] = make_float4(st.dv[0] - st.cv[0], st.dv[1] - st.cv[1], st.dv[2] - st.cv[2],
                                                        0.0f);
         }
-    } else if constexpr (INTEG == 0 && BOS_FWD_PIPELINE) {
-        // Sharma steps, software-pipelined: the next step's first stage needs only the new
-        // position r' = r + dt (v + (A + 2B)/6), not C, so it is evaluated together with this
-        // step's third stage.  Same operations as comp_step, in a different order in time.
-        BrickCache bc1 = {0xffffffffu, 0u};
-        int ci[3];
-        float cf[3], A[3], D[3];
-        rhs_of(eval(st.U, st.dr, bc1, ci, cf), D);
-        const float dt = k.dt;
-        for (int a = 0; a < 3; ++a) A[a] = dt * D[a];
-        float apart = 0.0f;   // largest |A - B| of the steps
-        int left = K;         // steps before the next checkpoint
-        for (int n = 0; n < R.N; ++n) {
-            if (state != nullptr && left == 0) {
-                left = K;
-                const size_t c = bounded((size_t)(n / K), (size_t)ck.max_ckpt, ck.err);
-                state[(c * 3 + 0) * ck.nrays + ray] = make_float4(st.dr[0], st.dr[1], st.dr[2], st.cr[0]);
-                state[(c * 3 + 1) * ck.nrays + ray] = make_float4(st.dv[0], st.dv[1], st.dv[2], st.cr[1]);
-                state[(c * 3 + 2) * ck.nrays + ray] = make_float4(st.cv[0], st.cv[1], st.cv[2], st.cr[2]);
-            }
-            // Every operation is explicitly rounded: left to the assembler, a product and a sum are
-            // fused or not depending on the kernel's register budget.
-            float B[3], q[3], inc_r[3];
-            long long U2[3], U3[3];
-            for (int a = 0; a < 3; ++a) {
-                q[a] = fmaf(__fmul_rn(0.125f, dt), A[a], fmaf(__fmul_rn(0.5f, dt), st.dv[a], st.dr[a]));
-                U2[a] = st.U[a] + k.dUh[a];
-                U3[a] = st.U[a] + k.dU[a];
-            }
-            --left;
-            rhs_of(eval(U2, q, bc, ci, cf), D);
-            for (int a = 0; a < 3; ++a) {
-                B[a] = __fmul_rn(dt, D[a]);
-                apart = fmaxf(apart, fabsf(A[a] - B[a]));
-            }
-            float X[3];
-            for (int a = 0; a < 3; ++a) {
-                q[a] = fmaf(__fmul_rn(0.5f, dt), B[a], fmaf(dt, st.dv[a], st.dr[a]));
-                X[a] = fmaf(fmaf(2.0f, B[a], A[a]), 1.0f / 6.0f, st.dv[a]);
-                inc_r[a] = __fmul_rn(dt, X[a]);
-            }
-            float dr1[3], cr1[3];
-            for (int a = 0; a < 3; ++a) {
-                const float y = fmaf(dt, X[a], -st.cr[a]);
-                dr1[a] = __fadd_rn(st.dr[a], y);
-                cr1[a] = __fsub_rn(__fsub_rn(dr1[a], st.dr[a]), y);
-            }
-            // independent: stage 3 of this step and stage 1 of the next
-            float D1[3] = {0.0f, 0.0f, 0.0f};
-            rhs_of(eval(U3, q, bc, ci, cf), D);
-            if (n + 1 < R.N) {
-                int ci1[3];
-                float cf1[3];
-                rhs_of(eval(U3, dr1, bc1, ci1, cf1), D1);
-            }
-            float si = k.dS[0] * inc_r[0] + k.dS[1] * inc_r[1] + k.dS[2] * inc_r[2];
-            float ii = inc_r[0] * inc_r[0] + inc_r[1] * inc_r[1] + inc_r[2] * inc_r[2];
-            float di = k.dhat[0] * inc_r[0] + k.dhat[1] * inc_r[1] + k.dhat[2] * inc_r[2];
-            st.excess += __fdividef(2.0f * si + ii, 2.0f * k.step_len + di);
-            for (int a = 0; a < 3; ++a) {
-                st.dr[a] = dr1[a];
-                st.cr[a] = cr1[a];
-                const float s4 = fmaf(4.0f, B[a], A[a]);
-                const float sv = fmaf(dt, D[a], s4);
-                const float y = fmaf(sv, 1.0f / 6.0f, -st.cv[a]);
-                const float v1 = __fadd_rn(st.dv[a], y);
-                st.cv[a] = __fsub_rn(__fsub_rn(v1, st.dv[a]), y);
-                st.dv[a] = v1;
-                st.U[a] = U3[a];
-                A[a] = __fmul_rn(dt, D1[a]);
-            }
-        }
-        if (state != nullptr) {
-            // the first checkpoint is the entry state, which is zero: its slot holds the end state
-            state[0 * ck.nrays + ray] = make_float4(st.dr[0], st.dr[1], st.dr[2], st.cr[0]);
-            state[1 * ck.nrays + ray] = make_float4(st.dv[0], st.dv[1], st.dv[2], st.cr[1]);
-            state[2 * ck.nrays + ray] = make_float4(st.cv[0], st.cv[1], st.cv[2], st.cr[2]);
-            // steps that the adjoint can reverse without their stage terms: dt |A - B| / 6 within
-            // kSameReverse cells (not so: NaN, too)
-            const float ih = fmaxf(F.inv_h[0], fmaxf(F.inv_h[1], F.inv_h[2]));
-            *apart_cells = apart * dt * (ih * (1.0f / 6.0f));
-        }
+    } else if constexpr (INTEG == 0) {
+        stage_run(F, R, k, ck, state, ray, st, apart_cells);
     } else {
         for (int n = 0; n < R.N; ++n) {
             if (state != nullptr && n % K == 0) {
@@ -498,17 +570,22 @@ __device__ __forceinline__ void comp_end(const CompState& st, float dr[3], float
 // End deviation, path excess and entry index of a ray: Sharma without checkpoints marches from
 // cell to cell, everything else goes stage by stage.
 template <class E, int INTEG, bool CONN, bool SAVE>
-__device__ __forceinline__ void trace_end(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
+__device__ __forceinline__ void trace_end(const SceneDev& S, const CompField<E>& F, const double rs[3], Ray& R,
+                                          volatile double* park,
                                           const CkptDev& ck, float4* state, long long ray, float dr[3], float dv[3],
-                                          float& excess, double& eta_in, float* apart) {
+                                          float& excess, float& eta, float* apart) {
+    if constexpr (INTEG == 0) park_ray(park, R);   // (the other tracers have registers to spare)
     if constexpr (INTEG == 0 && !SAVE) {
-        march_run(S, F, rs, R, dr, dv, excess, eta_in);
+        march_run(S, F, rs, R, park, dr, dv, excess, eta);
     } else {
         CompState st;
-        comp_run<E, INTEG, !CONN>(S, F, rs, R, ck, state, ray, st, eta_in, apart);
+        double eta_in;
+        comp_run<E, INTEG>(S, F, rs, R, ck, state, ray, st, eta_in, apart);
+        eta = (float)eta_in;
         comp_end(st, dr, dv);
         excess = st.excess;
     }
+    if constexpr (INTEG == 0) unpark_ray(park, R);
 }
 
 // Trace one camera ray of the comp path (checkpoints every K steps when ck.state is set).
@@ -517,14 +594,14 @@ __device__ __forceinline__ void trace_end(const SceneDev& S, const CompField<E>&
 // wall hit of the projector ray aimed at a (traced like a camera ray), so that
 // a = x_ref + e with e <- dx - (y(a) - (P + t_w d_p)) - ((P + t_w d_p) - a).
 template <class E, int INTEG, bool CONN, bool SAVE>
-__device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, const Ray& R, const CkptDev& ck,
+__device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, Ray R, const CkptDev& ck,
                                 long long ray, bool want_hit, unsigned long long& steps) {
     WallRel h;
     float path = 0.0f, apart = 0.0f;   // path excess; largest stage distance of a step (cells)
     if (R.N > 0) {
         float dr[3], dv[3], excess;
-        double eta_in;
-        trace_end<E, INTEG, CONN, SAVE>(S, F, S.cam.pos, R, ck, ck.state, ray, dr, dv, excess, eta_in, &apart);
+        float eta_in;
+        trace_end<E, INTEG, CONN, SAVE>(S, F, S.cam.pos, R, ray_park<0>(), ck, ck.state, ray, dr, dv, excess, eta_in, &apart);
         path = excess;
         steps += (unsigned long long)R.N;
         h = comp_wall(S, R, eta_in, dr, dv, excess);
@@ -540,13 +617,14 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, const 
             double xref[3];
             for (int a = 0; a < 3; ++a) xref[a] = S.cam.pos[a] + R.tw * R.d[a];
             const double* P = S.L.proj.pos;
+            if constexpr (INTEG == 0) park_ray(ray_park<0>(), R);
             for (int m = 0; m < S.L.connect_iters; ++m) {
-                const Ray Rp = projector_setup(S, xref, e);
+                Ray Rp = projector_setup(S, xref, e);
                 float yrel[3] = {0.0f, 0.0f, 0.0f};
                 if (Rp.wall && Rp.N > 0) {
-                    double eta_p;
+                    float eta_p;
                     float pr[3], pv[3], pexcess, papart = 0.0f;
-                    trace_end<E, INTEG, CONN, SAVE>(S, F, P, Rp, ck, m == 0 ? ck.pstate : nullptr, ray, pr, pv, pexcess,
+                    trace_end<E, INTEG, CONN, SAVE>(S, F, P, Rp, ray_park<1>(), ck, m == 0 ? ck.pstate : nullptr, ray, pr, pv, pexcess,
                                                     eta_p, &papart);
                     if (!(papart <= apart)) apart = papart;
                     steps += (unsigned long long)Rp.N;
@@ -554,12 +632,18 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, const 
                     if (hp.valid)
                         for (int a = 0; a < 3; ++a) yrel[a] = hp.dx[a];
                 }
+                if constexpr (INTEG == 0) {
+                    unpark_ray(ray_park<0>(), R);
+                    for (int a = 0; a < 3; ++a) xref[a] = S.cam.pos[a] + R.tw * R.d[a];
+                }
                 for (int a = 0; a < 3; ++a) {
                     const double eps = (xref[a] + (double)e[a]) - (P[a] + Rp.tw * Rp.d[a]);
                     e[a] = (h.dx[a] - yrel[a]) + (float)eps;
                 }
             }
         }
+        if constexpr (INTEG == 0)
+            if (h.valid) unpark_ray(ray_park<0>(), R);
         if (ck.conn != nullptr) {   // (a zero cosine factor marks a ray that misses the wall)
             ck.conn[2 * ray] = make_float4(h.dx[0], h.dx[1], h.dx[2], h.valid ? h.cosw / h.len : 0.0f);
             ck.conn[2 * ray + 1] = make_float4(h.dx[0] - e[0], h.dx[1] - e[1], h.dx[2] - e[2], 0.0f);
@@ -659,8 +743,11 @@ __device__ __forceinline__ RayResult trace_ray(const SceneDev& S, const Ray& R, 
 #ifndef BOS_FWD_MARCH_MIN_BLOCKS
 #define BOS_FWD_MARCH_MIN_BLOCKS 4        // Sharma through the cell marcher (32 polynomial values per ray)
 #endif
-#ifndef BOS_FWD_CACHED_MIN_BLOCKS
-#define BOS_FWD_CACHED_MIN_BLOCKS 5       // Sharma with checkpoints, whose cell cache holds 32 values per ray
+#ifndef BOS_FWD_STAGE_MIN_BLOCKS
+#define BOS_FWD_STAGE_MIN_BLOCKS 4        // Sharma with checkpoints (32 values of the last cell per ray)
+#endif
+#ifndef BOS_FWD_STAGE_CONN_MIN_BLOCKS
+#define BOS_FWD_STAGE_CONN_MIN_BLOCKS 3   // the same with the refracted connection
 #endif
 #ifndef BOS_FWD_QUASI_MIN_BLOCKS
 #define BOS_FWD_QUASI_MIN_BLOCKS 3        // quasi-linear tracing (more registers, more overlap)
@@ -668,8 +755,7 @@ __device__ __forceinline__ RayResult trace_ray(const SceneDev& S, const Ray& R, 
 constexpr int render_min_blocks(int mode, int integ, bool conn, bool save) {
     return integ == 2 ? BOS_FWD_QUASI_MIN_BLOCKS
            : (mode != 1 && mode != 2) || integ != 0 ? BOS_FWD_MIN_BLOCKS
-           : !save ? BOS_FWD_MARCH_MIN_BLOCKS
-           : !conn && BOS_FWD_PIPELINE ? BOS_FWD_CACHED_MIN_BLOCKS : BOS_FWD_MIN_BLOCKS;
+           : save ? (conn ? BOS_FWD_STAGE_CONN_MIN_BLOCKS : BOS_FWD_STAGE_MIN_BLOCKS) : BOS_FWD_MARCH_MIN_BLOCKS;
 }
 // One warp tile of a render: the rays of its (up to) 32 lanes, averaged per pixel, written
 // to the outputs; adds the traced ray-steps to my_steps.
@@ -763,7 +849,7 @@ __global__ void __launch_bounds__(128, FEW ? 1 : render_min_blocks(MODE, INTEG, 
 // jobs[j + 1].first and is that job's tile jobs[j].tile0 + (g - jobs[j].first).  Warps
 // pull items in order, so the jobs' tiles are interleaved as they are listed.
 template <int MODE, int INTEG>
-__global__ void __launch_bounds__(128, render_min_blocks(MODE, INTEG, false, true))
+__global__ void __launch_bounds__(128, render_min_blocks(MODE, INTEG, false, false))
     render_batch_kernel(const BatchJob* __restrict__ jobs, int njobs, int total, int* counter) {
     const int lane = threadIdx.x & 31;
     for (;;) {

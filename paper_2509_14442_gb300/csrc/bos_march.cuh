@@ -33,6 +33,7 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
 __device__ __forceinline__ f32x2 splat2(float a) { return pack2(a, a); }
 __device__ __forceinline__ float lo2(f32x2 v) {
     float a, b;
