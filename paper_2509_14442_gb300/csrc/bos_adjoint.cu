@@ -672,7 +672,7 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                         Vk = mul3(dt, p3(s1.x - s2.x, s1.y - s2.y, s1.z - s2.z));
                         kept_state = true;
                     }
-                    moved = march_point<false>(F, L, m, h, dr, f);
+                    moved = march_point<false, QUASI>(F, L, m, h, dr, f);
                 }
                 if (__any_sync(0xffffffffu, moved)) {
                     rows_flush(rows, moved && used, key, row, acc, nx, nxy, ncells, err);
@@ -728,7 +728,7 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                 // ---- the middle of step n - 1
                 h = add2(h, splat2(-1.0f));
                 moved = false;
-                if (on) moved = march_point<false>(F, L, m, h, QUASI ? dr : fma3(0.75f, c, fma3(-0.5f, V, dr)), f);
+                if (on) moved = march_point<false, QUASI>(F, L, m, h, QUASI ? dr : fma3(0.75f, c, fma3(-0.5f, V, dr)), f);
                 if (__any_sync(0xffffffffu, moved)) {
                     rows_flush(rows, moved && used, key, row, acc, nx, nxy, ncells, err);
                     if (moved) key = march_key(m, (uint32_t)nx, (uint32_t)nxy);

@@ -270,7 +270,7 @@ __device__ __forceinline__ void unpark_ray(volatile double* p, Ray& R) {
     R.ell = p[5 * kRenderThreads];
 }
 
-// Sharma steps of one ray through the cell marcher, in the scaled variables V = dt dv and
+// Steps of one ray through the cell marcher (QUASI: quasi-linear, else Sharma's), in the scaled variables V = dt dv and
 // a = (dt^2 / 6) D (metres per step), so that
 //   p2 = S(n+1/2) + dr + V/2 + 3a/4,   p3 = S(n+1) + dr + V + 3b
 //   dr += V + a + 2b,                  V += a + 4b + c
@@ -281,7 +281,11 @@ __device__ __forceinline__ void unpark_ray(volatile double* p, Ray& R) {
 // coarse step through a steep field), that lane evaluates a' at its own point.  The path
 // excess sum |dS + inc| - |dS| is d.(sum of inc) + sum (|inc|^2 - (d.inc)^2) / (2L + d.inc):
 // the first term is the end deviation, so only the small second one is summed.
-template <class E>
+// Quasi-linear tracing (Sec. 2.2) takes the same weights at the start, middle and end of each
+// step on the straight line: the end sample is the next step's start sample.  Render and adjoint
+// of 256x256x192 cells at 1024 x 768 rays: 14.21 ms with four gathers per step pair through the
+// 64-bit line position, 12.82 ms so.
+template <class E, bool QUASI>
 __device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
                                           volatile double* park, float dr_end[3], float dv_end[3], float& excess_end,
                                           float& eta_out) {
@@ -325,6 +329,19 @@ __device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>&
         const int n1 = min(R.N, n + kLineSteps);
         for (; n < n1; ++n) {
             h = add2(h, splat2(1.0f));
+            if constexpr (QUASI) {
+                const P3 b = march_accel(march_value<false, true>(F, L, m, h, dr), s);
+                h = add2(h, splat2(1.0f));
+                const P3 c = march_accel(march_value<false, true>(F, L, m, h, dr), s);
+                const P3 t = fma3(2.0f, b, a);
+                const P3 y = add3(t, sub3(V, cr));
+                kahan3(dr, cr, y);
+                kahan3(V, cv, sub3(add3(fma3(2.0f, b, t), c), cv));
+                const float di = dot3(d, y);
+                excess = fmaf(fmaf(-di, di, dot3(y, y)), rcp_approx(__fadd_rn(len2, di)), excess);
+                a = c;
+                continue;
+            }
             const P3 b = march_accel(march_value(F, L, m, h, fma3(0.75f, a, fma3(0.5f, V, dr))), s);
             h = add2(h, splat2(1.0f));
             P3 p = fma3(3.0f, b, add3(dr, V));
@@ -498,56 +515,11 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
     CompConst k;
     double rin[3];
     comp_setup(S, F, rs, R, st, k, eta_in, rin);
-    BrickCache bc = {0xffffffffu, 0u};
-    const int K = ck.every;
-    if constexpr (INTEG == 2) {
-        // Quasi-linear tracing (Sec. 2.2): the field is sampled on the straight line at the
-        // start, middle and end of every step (Sharma's weights); the end sample is the next
-        // step's start sample, so each step gathers twice, with no dependence on the ray.
-        const float zero[3] = {0.0f, 0.0f, 0.0f};
-        int ci[3];
-        float cf[3], A[3], B[3], C[3], D[3];
-        const float dt = k.dt;
-        rhs_of(comp_eval(F, st.U, zero, bc, ci, cf), D);
-        for (int a = 0; a < 3; ++a) A[a] = dt * D[a];
-        // two steps per iteration: their four line samples do not depend on one another,
-        // so their gathers overlap (the quasi-linear kernel gets a larger register budget for this)
-#pragma unroll 2
-        for (int n = 0; n < R.N; ++n) {
-            long long U2[3], U3[3];
-            for (int a = 0; a < 3; ++a) {
-                U2[a] = st.U[a] + k.dUh[a];
-                U3[a] = st.U[a] + k.dU[a];
-            }
-            rhs_of(comp_eval(F, U2, zero, bc, ci, cf), D);
-            for (int a = 0; a < 3; ++a) B[a] = dt * D[a];
-            rhs_of(comp_eval(F, U3, zero, bc, ci, cf), D);
-            float inc_r[3], inc_v[3];
-            for (int a = 0; a < 3; ++a) {
-                C[a] = dt * D[a];
-                inc_r[a] = dt * (st.dv[a] + (A[a] + 2.0f * B[a]) * (1.0f / 6.0f));
-                inc_v[a] = (A[a] + 4.0f * B[a] + C[a]) * (1.0f / 6.0f);
-            }
-            float si = k.dS[0] * inc_r[0] + k.dS[1] * inc_r[1] + k.dS[2] * inc_r[2];
-            float ii = inc_r[0] * inc_r[0] + inc_r[1] * inc_r[1] + inc_r[2] * inc_r[2];
-            float di = k.dhat[0] * inc_r[0] + k.dhat[1] * inc_r[1] + k.dhat[2] * inc_r[2];
-            st.excess += __fdividef(2.0f * si + ii, 2.0f * k.step_len + di);
-            for (int a = 0; a < 3; ++a) {
-                kahan_add(st.dr[a], st.cr[a], inc_r[a]);
-                kahan_add(st.dv[a], st.cv[a], inc_v[a]);
-                st.U[a] = U3[a];
-                A[a] = C[a];
-            }
-        }
-        if (state != nullptr) {   // the end state, from which the adjoint reverses the ray
-            state[0 * ck.nrays + ray] = make_float4(st.dr[0] - st.cr[0], st.dr[1] - st.cr[1], st.dr[2] - st.cr[2],
-                                                       st.excess);
-            state[1 * ck.nrays + ray] = make_float4(st.dv[0] - st.cv[0], st.dv[1] - st.cv[1], st.dv[2] - st.cv[2],
-                                                       0.0f);
-        }
-    } else if constexpr (INTEG == 0) {
+    if constexpr (INTEG == 0) {
         stage_run(F, R, k, ck, state, ray, st, apart_cells);
     } else {
+        BrickCache bc = {0xffffffffu, 0u};
+        const int K = ck.every;
         for (int n = 0; n < R.N; ++n) {
             if (state != nullptr && n % K == 0) {
                 const size_t c = bounded((size_t)(n / K), (size_t)ck.max_ckpt, ck.err);
@@ -567,16 +539,20 @@ __device__ __forceinline__ void comp_end(const CompState& st, float dr[3], float
     }
 }
 
-// End deviation, path excess and entry index of a ray: Sharma without checkpoints marches from
-// cell to cell, everything else goes stage by stage.
+// End deviation, path excess and entry index of a ray: Sharma without checkpoints and the
+// quasi-linear tracer march from cell to cell, everything else goes stage by stage.
 template <class E, int INTEG, bool CONN, bool SAVE>
 __device__ __forceinline__ void trace_end(const SceneDev& S, const CompField<E>& F, const double rs[3], Ray& R,
                                           volatile double* park,
                                           const CkptDev& ck, float4* state, long long ray, float dr[3], float dv[3],
                                           float& excess, float& eta, float* apart) {
-    if constexpr (INTEG == 0) park_ray(park, R);   // (the other tracers have registers to spare)
-    if constexpr (INTEG == 0 && !SAVE) {
-        march_run(S, F, rs, R, park, dr, dv, excess, eta);
+    if constexpr (INTEG != 1) park_ray(park, R);   // (classical steps have registers to spare)
+    if constexpr (INTEG == 2 || (INTEG == 0 && !SAVE)) {
+        march_run<E, INTEG == 2>(S, F, rs, R, park, dr, dv, excess, eta);
+        if (INTEG == 2 && state != nullptr) {   // the end state, from which the adjoint reverses the ray
+            state[0 * ck.nrays + ray] = make_float4(dr[0], dr[1], dr[2], excess);
+            state[1 * ck.nrays + ray] = make_float4(dv[0], dv[1], dv[2], 0.0f);
+        }
     } else {
         CompState st;
         double eta_in;
@@ -585,7 +561,7 @@ __device__ __forceinline__ void trace_end(const SceneDev& S, const CompField<E>&
         comp_end(st, dr, dv);
         excess = st.excess;
     }
-    if constexpr (INTEG == 0) unpark_ray(park, R);
+    if constexpr (INTEG != 1) unpark_ray(park, R);
 }
 
 // Trace one camera ray of the comp path (checkpoints every K steps when ck.state is set).
@@ -617,7 +593,7 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, Ray R,
             double xref[3];
             for (int a = 0; a < 3; ++a) xref[a] = S.cam.pos[a] + R.tw * R.d[a];
             const double* P = S.L.proj.pos;
-            if constexpr (INTEG == 0) park_ray(ray_park<0>(), R);
+            if constexpr (INTEG != 1) park_ray(ray_park<0>(), R);
             for (int m = 0; m < S.L.connect_iters; ++m) {
                 Ray Rp = projector_setup(S, xref, e);
                 float yrel[3] = {0.0f, 0.0f, 0.0f};
@@ -632,7 +608,7 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, Ray R,
                     if (hp.valid)
                         for (int a = 0; a < 3; ++a) yrel[a] = hp.dx[a];
                 }
-                if constexpr (INTEG == 0) {
+                if constexpr (INTEG != 1) {
                     unpark_ray(ray_park<0>(), R);
                     for (int a = 0; a < 3; ++a) xref[a] = S.cam.pos[a] + R.tw * R.d[a];
                 }
@@ -642,7 +618,7 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, Ray R,
                 }
             }
         }
-        if constexpr (INTEG == 0)
+        if constexpr (INTEG != 1)
             if (h.valid) unpark_ray(ray_park<0>(), R);
         if (ck.conn != nullptr) {   // (a zero cosine factor marks a ray that misses the wall)
             ck.conn[2 * ray] = make_float4(h.dx[0], h.dx[1], h.dx[2], h.valid ? h.cosw / h.len : 0.0f);
@@ -750,7 +726,7 @@ __device__ __forceinline__ RayResult trace_ray(const SceneDev& S, const Ray& R, 
 #define BOS_FWD_STAGE_CONN_MIN_BLOCKS 3   // the same with the refracted connection
 #endif
 #ifndef BOS_FWD_QUASI_MIN_BLOCKS
-#define BOS_FWD_QUASI_MIN_BLOCKS 3        // quasi-linear tracing (more registers, more overlap)
+#define BOS_FWD_QUASI_MIN_BLOCKS 4        // quasi-linear tracing through the cell marcher (3 blocks: 3 % slower a step)
 #endif
 constexpr int render_min_blocks(int mode, int integ, bool conn, bool save) {
     return integ == 2 ? BOS_FWD_QUASI_MIN_BLOCKS

@@ -157,9 +157,12 @@ __device__ __forceinline__ void march_line(const float inv_h[3], const double u0
     m.ci = P3{kCellBias, splat2(kCellBias)};
 }
 
+// LINE: the point on the line itself (q is not looked at).
+template <bool LINE>
 __device__ __forceinline__ P3 march_frac(const MarchLine& L, const MarchCell& m, f32x2 h, P3 q) {
-    return add3(P3{fmaf(lo2(h), L.dh.x, m.base.x), fma2(h, L.dh.yz, m.base.yz)},
-                P3{fmaf(q.x, L.ih.x, m.corr.x), fma2(q.yz, L.ih.yz, m.corr.yz)});
+    const P3 u = P3{fmaf(lo2(h), L.dh.x, m.base.x), fma2(h, L.dh.yz, m.base.yz)};
+    if constexpr (LINE) return add3(u, m.corr);
+    return add3(u, P3{fmaf(q.x, L.ih.x, m.corr.x), fma2(q.yz, L.ih.yz, m.corr.yz)});
 }
 
 struct Frac3 {
@@ -170,10 +173,10 @@ struct Frac3 {
 // fall outside the cell the ray is moved to the cell of the point (clamped to the grid: the
 // edge cells extrapolate) and that cell's polynomial is loaded.  FIRST: no cell is loaded yet.
 // Returns true where the cell changed.
-template <bool FIRST, class E>
+template <bool FIRST, bool LINE = false, class E>
 __device__ __forceinline__ bool march_point(const CompField<E>& F, const MarchLine& L, MarchCell& m, f32x2 h, P3 q,
                                             Frac3& f) {
-    P3 u = march_frac(L, m, h, q);
+    P3 u = march_frac<LINE>(L, m, h, q);
     f = Frac3{u.x, lo2(u.yz), hi2(u.yz)};
     // 0 <= f < 1 exactly when the bit pattern is below that of 1.0f
     const uint32_t top = max(__float_as_uint(f.x), max(__float_as_uint(f.y), __float_as_uint(f.z)));
@@ -193,7 +196,7 @@ __device__ __forceinline__ bool march_point(const CompField<E>& F, const MarchLi
     m.ci = p3(ci[0], ci[1], ci[2]);
     m.base = add3(m.base, p3(back[0], back[1], back[2]));
     m.corr = P3{fmaf(lo2(h), L.dlo.x, L.ulo.x), fma2(h, L.dlo.yz, L.ulo.yz)};
-    u = march_frac(L, m, h, q);
+    u = march_frac<LINE>(L, m, h, q);
     f = Frac3{u.x, lo2(u.yz), hi2(u.yz)};
     if (FIRST || (moved >> 3) != 0u)
         m.brick = morton3((c[0] & 0x7fffffu) >> 3, (c[1] & 0x7fffffu) >> 3, (c[2] & 0x7fffffu) >> 3) *
@@ -208,10 +211,10 @@ __device__ __forceinline__ bool march_point(const CompField<E>& F, const MarchLi
 }
 
 // (deta, grad eta) at a point.
-template <bool FIRST = false, class E>
+template <bool FIRST = false, bool LINE = false, class E>
 __device__ __forceinline__ Cell2 march_value(const CompField<E>& F, const MarchLine& L, MarchCell& m, f32x2 h, P3 q) {
     Frac3 f;
-    march_point<FIRST>(F, L, m, h, q, f);
+    march_point<FIRST, LINE>(F, L, m, h, q, f);
     return poly_value(m.p, splat2(f.x), splat2(f.y), splat2(f.z));
 }
 
