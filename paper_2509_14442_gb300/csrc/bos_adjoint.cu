@@ -1165,27 +1165,15 @@ struct D4Grad {
     D4 v, d0, d1, d2;   // value and derivatives with respect to the three fractions
 };
 
-__device__ __forceinline__ D4 dsub4(D4 a, D4 b) {
-    D4 r;
-    r.x = a.x - b.x;
-    r.y = a.y - b.y;
-    r.z = a.z - b.z;
-    r.w = a.w - b.w;
-    return r;
-}
-
-// Value (the operations of trilinear_d, so bit-identical) and fraction derivatives.
-__device__ __forceinline__ D4Grad trilinear_grad_d(const D4* s, uint32_t o, double f0, double f1, double f2) {
-    const D4 c000 = load_d4(s, o), c100 = load_d4(s, o + 1), c010 = load_d4(s, o + 9), c110 = load_d4(s, o + 10);
-    const D4 c001 = load_d4(s, o + 81), c101 = load_d4(s, o + 82), c011 = load_d4(s, o + 90), c111 = load_d4(s, o + 91);
-    const D4 a0 = dlerp(c000, c100, f0), a1 = dlerp(c010, c110, f0), a2 = dlerp(c001, c101, f0),
-             a3 = dlerp(c011, c111, f0);
-    const D4 b0 = dlerp(a0, a1, f1), b1 = dlerp(a2, a3, f1);
+// Value (dcell_value's operations, so bit-identical) and fraction derivatives.
+__device__ __forceinline__ D4Grad dcell_grad(const DCell& m, const double f[3]) {
+    const D4 e0 = dfma4(f[0], m.c[1], m.c[0]), e1 = dfma4(f[0], m.c[3], m.c[2]);
+    const D4 e2 = dfma4(f[0], m.c[5], m.c[4]), e3 = dfma4(f[0], m.c[7], m.c[6]);
     D4Grad r;
-    r.v = dlerp(b0, b1, f2);
-    r.d2 = dsub4(b1, b0);
-    r.d1 = dlerp(dsub4(a1, a0), dsub4(a3, a2), f2);
-    r.d0 = dlerp(dlerp(dsub4(c100, c000), dsub4(c110, c010), f1), dlerp(dsub4(c101, c001), dsub4(c111, c011), f1), f2);
+    r.d2 = dfma4(f[1], e3, e2);
+    r.v = dfma4(f[2], r.d2, dfma4(f[1], e1, e0));
+    r.d1 = dfma4(f[2], e3, e1);
+    r.d0 = dfma4(f[2], dfma4(f[1], m.c[7], m.c[5]), dfma4(f[1], m.c[3], m.c[1]));
     return r;
 }
 
@@ -1195,15 +1183,11 @@ struct DStage {
     D4Grad g;
 };
 
-// Field value and gradient at absolute position x: the cell and fractions of field_at.
-__device__ __forceinline__ void dstage_eval(const GridDev& g, const double x[3], DStage& s) {
-    for (int a = 0; a < 3; ++a) {
-        const double u = (x[a] - g.origin[a]) / g.h[a] - 0.5;
-        split_coord(u, g.n[a], s.i[a], s.f[a]);
-    }
-    uint32_t o = bounded(brick_offset(s.i[0], s.i[1], s.i[2]) + 91u, g.store_elems, g.err);
-    o = o ? o - 91u : 0u;
-    s.g = trilinear_grad_d(static_cast<const D4*>(g.store), o, s.f[0], s.f[1], s.f[2]);
+// Field value and gradient at absolute position x.
+__device__ __forceinline__ void dstage_eval(const GridDev& g, const double x[3], DCell& m, DStage& s) {
+    dcell_point(g, x, m, s.f);
+    for (int a = 0; a < 3; ++a) s.i[a] = m.i[a];
+    s.g = dcell_grad(m, s.f);
 }
 
 __device__ __forceinline__ void drhs(const DStage& s, double D[3]) {
@@ -1213,25 +1197,62 @@ __device__ __forceinline__ void drhs(const DStage& s, double D[3]) {
     D[2] = eta * s.g.v.w;
 }
 
-// Adjoint of D = (1 + deta) grad at a stage for Db: the position adjoint pb, and the
-// record adjoint Q scattered to the 8 corners with the trilinear weights.
-__device__ __forceinline__ void drhs_adjoint_scatter(const GridDev& g, const DStage& s, const double Db[3], double pb[3],
-                                                     double* acc, bool act) {
+// Adjoint of D = (1 + deta) grad at a stage for Db: the position adjoint pb and the record
+// adjoint Q that the corners share.
+__device__ __forceinline__ void drhs_adjoint(const GridDev& g, const DStage& s, const double Db[3], double pb[3],
+                                             double Q[4]) {
     const double eta = 1.0 + s.g.v.x;
     const double Dg = Db[0] * s.g.v.y + Db[1] * s.g.v.z + Db[2] * s.g.v.w;
     const D4 dv[3] = {s.g.d0, s.g.d1, s.g.d2};
-    for (int a = 0; a < 3; ++a)
-        pb[a] = g.inv_h[a] * (dv[a].x * Dg + eta * (Db[0] * dv[a].y + Db[1] * dv[a].z + Db[2] * dv[a].w));
+    Q[0] = Dg;
+    for (int a = 0; a < 3; ++a) Q[1 + a] = eta * Db[a];
+    for (int a = 0; a < 3; ++a) pb[a] = g.inv_h[a] * (dv[a].x * Q[0] + dv[a].y * Q[1] + dv[a].z * Q[2] + dv[a].w * Q[3]);
+}
+
+// Corner sensitivities of a lane's current cell in float64, a row of shared memory per lane
+// (value 4 c + channel; odd row stride: neither a lane's own accesses nor a warp's read of one
+// row conflict).  A ray stays in a cell for six to twelve stage points, and neighbouring rays
+// share cells: summed per lane and then over the warp's lanes of a cell, a tile sends a few
+// hundred node additions where every point sent 32 per lane.
+constexpr int kRowD = 33;
+
+__device__ __forceinline__ void flush_rows_d(double* rows, bool flag, uint32_t& key, double* acc, const GridDev& g) {
+    unsigned pend = __ballot_sync(0xffffffffu, flag);
+    if (!pend) return;
+    __syncwarp();
+    const int lane = threadIdx.x & 31, corner = lane >> 2;
+    const uint32_t nx = (uint32_t)g.n[0], nxy = nx * (uint32_t)g.n[1];
+    const uint32_t off = (uint32_t)(corner & 1) + (uint32_t)((corner >> 1) & 1) * nx + (uint32_t)(corner >> 2) * nxy;
+    const uint32_t mykey = flag ? key : kNoKey;
+    while (pend) {
+        const uint32_t lk = __shfl_sync(0xffffffffu, mykey, __ffs(pend) - 1);
+        unsigned grp = __ballot_sync(0xffffffffu, mykey == lk);
+        pend &= ~grp;
+        double sum = 0.0;
+        for (; grp; grp &= grp - 1) sum += rows[(__ffs(grp) - 1) * kRowD + lane];
+        atomicAdd(acc + (size_t)bounded(lk + off, nxy * (uint32_t)g.n[2], g.err) * 4 + (lane & 3), sum);
+    }
+    __syncwarp();
+    if (flag) {
+        for (int c = 0; c < 32; ++c) rows[lane * kRowD + c] = 0.0;
+        key = kNoKey;
+    }
+    __syncwarp();
+}
+
+// Warp-collective: add w_c(f) Q to the lane's row (flushed first where the cell changes).
+__device__ __forceinline__ void accumulate_d(double* rows, bool act, const int i[3], const double f[3], const double Q[4],
+                                             uint32_t& key, double* acc, const GridDev& g) {
+    const uint32_t cell = (uint32_t)i[0] + (uint32_t)g.n[0] * ((uint32_t)i[1] + (uint32_t)g.n[1] * (uint32_t)i[2]);
+    flush_rows_d(rows, act && key != kNoKey && key != cell, key, acc, g);
     if (!act) return;
-    const double Q[4] = {Dg, eta * Db[0], eta * Db[1], eta * Db[2]};
-    const size_t nx = (size_t)g.n[0], nxy = (size_t)g.n[0] * g.n[1];
-    const size_t base = (size_t)s.i[0] + (size_t)s.i[1] * nx + (size_t)s.i[2] * nxy;
+    key = cell;
+    double* row = rows + (threadIdx.x & 31) * kRowD;
+#pragma unroll
     for (int c = 0; c < 8; ++c) {
-        const double w = ((c & 1) ? s.f[0] : 1.0 - s.f[0]) * ((c & 2) ? s.f[1] : 1.0 - s.f[1]) *
-                         ((c & 4) ? s.f[2] : 1.0 - s.f[2]);
-        const size_t node = base + (size_t)(c & 1) + (size_t)((c >> 1) & 1) * nx + (size_t)(c >> 2) * nxy;
-        const size_t nd = bounded(node, (size_t)g.n[0] * g.n[1] * g.n[2], g.err);
-        for (int ch = 0; ch < 4; ++ch) atomicAdd(acc + nd * 4 + ch, w * Q[ch]);
+        const double w = ((c & 1) ? f[0] : 1.0 - f[0]) * ((c & 2) ? f[1] : 1.0 - f[1]) * ((c & 4) ? f[2] : 1.0 - f[2]);
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) row[4 * c + ch] = fma(w, Q[ch], row[4 * c + ch]);
     }
 }
 
@@ -1246,6 +1267,10 @@ __global__ void __launch_bounds__(kAdjWarps * 32) adjoint_fp64_kernel(SceneDev S
     double* acc = reinterpret_cast<double*>(adj.acc);
     const GridDev& g = S.g;
     const FullField<double> F = {S.g};
+    __shared__ double rows_sh[kAdjWarps * 32 * kRowD];
+    double* const rows = rows_sh + (size_t)warp * 32 * kRowD;
+    for (int c = 0; c < 32; ++c) rows[lane * kRowD + c] = 0.0;
+    uint32_t key = kNoKey;                // cell of the lane's row
     const int W = S.cam.width, H = S.cam.height, spp = S.cam.spp;
     const TileShape ts = tile_shape(W, H, spp);
     const int ntiles = tile_count(S, ts);
@@ -1279,6 +1304,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) adjoint_fp64_kernel(SceneDev S
             const int nseg = (N + K - 1) / K;
             const int nseg_max = __reduce_max_sync(0xffffffffu, (unsigned)nseg);
             double rb[3] = {0, 0, 0}, vb[3] = {0, 0, 0}, dtb = 0.0, lenb = 0.0;
+            const double dt6 = sixth(dt);
             for (int c = nseg_max - 1; c >= 0; --c) {
                 const int n0 = c * K, n1 = min(n0 + K, N);
                 const bool seg = act && n0 < N;
@@ -1310,95 +1336,95 @@ __global__ void __launch_bounds__(kAdjWarps * 32) adjoint_fp64_kernel(SceneDev S
                 const int n_hi = __reduce_max_sync(0xffffffffu, (unsigned)(seg ? n1 : 0));
                 for (int n = n_hi - 1; n >= n0; --n) {
                     const bool a_ = seg && n < n1;
-                    if (!a_) continue;
-                    const double* p = buf + (size_t)(n - n0) * 6 * 32 + lane;
-                    double r[3], v[3], A[3], B[3], D1[3], D2[3], D3[3], q[3];
-                    for (int a = 0; a < 3; ++a) {
-                        r[a] = p[32 * a];
-                        v[a] = p[32 * (3 + a)];
-                    }
                     DStage s1, s2, s3;
-                    dstage_eval(g, r, s1);
-                    drhs(s1, D1);
-                    for (int a = 0; a < 3; ++a) A[a] = dt * D1[a];
-                    for (int a = 0; a < 3; ++a) q[a] = r[a] + (dt * 0.5) * v[a] + (dt * 0.125) * A[a];
-                    dstage_eval(g, q, s2);
-                    drhs(s2, D2);
-                    for (int a = 0; a < 3; ++a) B[a] = dt * D2[a];
-                    for (int a = 0; a < 3; ++a) q[a] = r[a] + dt * v[a] + (dt * 0.5) * B[a];
-                    dstage_eval(g, q, s3);
-                    drhs(s3, D3);
-                    // r' = r + dt (v + (A + 2B)/6), |r' - r| enters the path length
-                    double inc[3], nn = 0.0, u[3];
-                    for (int a = 0; a < 3; ++a) {
-                        inc[a] = dt * (v[a] + (A[a] + 2.0 * B[a]) / 6.0);
-                        nn += inc[a] * inc[a];
+                    double Q1[4], Q2[4], Q3[4];
+                    if (a_) {
+                        const double* p = buf + (size_t)(n - n0) * 6 * 32 + lane;
+                        double r[3], v[3], A[3], B[3], D1[3], D2[3], D3[3], q[3];
+                        for (int a = 0; a < 3; ++a) {
+                            r[a] = p[32 * a];
+                            v[a] = p[32 * (3 + a)];
+                        }
+                        dstage_eval(g, r, F.m, s1);
+                        drhs(s1, D1);
+                        for (int a = 0; a < 3; ++a) A[a] = dt * D1[a];
+                        for (int a = 0; a < 3; ++a) q[a] = r[a] + (dt * 0.5) * v[a] + (dt * 0.125) * A[a];
+                        dstage_eval(g, q, F.m, s2);
+                        drhs(s2, D2);
+                        for (int a = 0; a < 3; ++a) B[a] = dt * D2[a];
+                        for (int a = 0; a < 3; ++a) q[a] = r[a] + dt * v[a] + (dt * 0.5) * B[a];
+                        dstage_eval(g, q, F.m, s3);
+                        drhs(s3, D3);
+                        // r' = r + dt (v + (A + 2B)/6), |r' - r| enters the path length
+                        double inc[3], nn = 0.0, u[3];
+                        for (int a = 0; a < 3; ++a) {
+                            inc[a] = dt * (v[a] + sixth(A[a] + 2.0 * B[a]));
+                            nn += inc[a] * inc[a];
+                        }
+                        const double rn = rsqrt(nn);
+                        double rbs[3], Ab[3], Bb[3], Cb[3], rn_[3], vn_[3], Db[3], pb[3];
+                        for (int a = 0; a < 3; ++a) {
+                            u[a] = inc[a] * rn;
+                            rbs[a] = rb[a] + lenb * u[a];
+                        }
+                        for (int a = 0; a < 3; ++a) {
+                            Cb[a] = sixth(vb[a]);
+                            Ab[a] = dt6 * rbs[a] + Cb[a];
+                            Bb[a] = 2.0 * (dt6 * rbs[a]) + vb[a] * (4.0 / 6.0);
+                            rn_[a] = rbs[a];
+                            vn_[a] = vb[a] + dt * rbs[a];
+                            dtb += rbs[a] * (v[a] + sixth(A[a] + 2.0 * B[a]));
+                        }
+                        // C = dt D(p3), p3 = r + dt v + dt/2 B
+                        for (int a = 0; a < 3; ++a) {
+                            dtb += Cb[a] * D3[a];
+                            Db[a] = dt * Cb[a];
+                        }
+                        drhs_adjoint(g, s3, Db, pb, Q3);
+                        for (int a = 0; a < 3; ++a) {
+                            rn_[a] += pb[a];
+                            vn_[a] += dt * pb[a];
+                            Bb[a] += (0.5 * dt) * pb[a];
+                            dtb += pb[a] * (v[a] + 0.5 * B[a]);
+                        }
+                        // B = dt D(p2), p2 = r + dt/2 v + dt/8 A
+                        for (int a = 0; a < 3; ++a) {
+                            dtb += Bb[a] * D2[a];
+                            Db[a] = dt * Bb[a];
+                        }
+                        drhs_adjoint(g, s2, Db, pb, Q2);
+                        for (int a = 0; a < 3; ++a) {
+                            rn_[a] += pb[a];
+                            vn_[a] += (0.5 * dt) * pb[a];
+                            Ab[a] += (0.125 * dt) * pb[a];
+                            dtb += pb[a] * (0.5 * v[a] + 0.125 * A[a]);
+                        }
+                        // A = dt D(p1), p1 = r
+                        for (int a = 0; a < 3; ++a) {
+                            dtb += Ab[a] * D1[a];
+                            Db[a] = dt * Ab[a];
+                        }
+                        drhs_adjoint(g, s1, Db, pb, Q1);
+                        for (int a = 0; a < 3; ++a) {
+                            rb[a] = rn_[a] + pb[a] - lenb * u[a];
+                            vb[a] = vn_[a];
+                        }
                     }
-                    const double rn = 1.0 / sqrt(nn);
-                    double rbs[3], Ab[3], Bb[3], Cb[3], rn_[3], vn_[3], Db[3], pb[3];
-                    for (int a = 0; a < 3; ++a) {
-                        u[a] = inc[a] * rn;
-                        rbs[a] = rb[a] + lenb * u[a];
-                    }
-                    for (int a = 0; a < 3; ++a) {
-                        Ab[a] = (dt / 6.0) * rbs[a] + vb[a] / 6.0;
-                        Bb[a] = (dt / 3.0) * rbs[a] + vb[a] * (4.0 / 6.0);
-                        Cb[a] = vb[a] / 6.0;
-                        rn_[a] = rbs[a];
-                        vn_[a] = vb[a] + dt * rbs[a];
-                        dtb += rbs[a] * (v[a] + (A[a] + 2.0 * B[a]) / 6.0);
-                    }
-                    // C = dt D(p3), p3 = r + dt v + dt/2 B
-                    for (int a = 0; a < 3; ++a) {
-                        dtb += Cb[a] * D3[a];
-                        Db[a] = dt * Cb[a];
-                    }
-                    drhs_adjoint_scatter(g, s3, Db, pb, acc, true);
-                    for (int a = 0; a < 3; ++a) {
-                        rn_[a] += pb[a];
-                        vn_[a] += dt * pb[a];
-                        Bb[a] += (0.5 * dt) * pb[a];
-                        dtb += pb[a] * (v[a] + 0.5 * B[a]);
-                    }
-                    // B = dt D(p2), p2 = r + dt/2 v + dt/8 A
-                    for (int a = 0; a < 3; ++a) {
-                        dtb += Bb[a] * D2[a];
-                        Db[a] = dt * Bb[a];
-                    }
-                    drhs_adjoint_scatter(g, s2, Db, pb, acc, true);
-                    for (int a = 0; a < 3; ++a) {
-                        rn_[a] += pb[a];
-                        vn_[a] += (0.5 * dt) * pb[a];
-                        Ab[a] += (0.125 * dt) * pb[a];
-                        dtb += pb[a] * (0.5 * v[a] + 0.125 * A[a]);
-                    }
-                    // A = dt D(p1), p1 = r
-                    for (int a = 0; a < 3; ++a) {
-                        dtb += Ab[a] * D1[a];
-                        Db[a] = dt * Ab[a];
-                    }
-                    drhs_adjoint_scatter(g, s1, Db, pb, acc, true);
-                    for (int a = 0; a < 3; ++a) {
-                        rb[a] = rn_[a] + pb[a] - lenb * u[a];
-                        vb[a] = vn_[a];
-                    }
+                    accumulate_d(rows, a_, s3.i, s3.f, Q3, key, acc, g);
+                    accumulate_d(rows, a_, s2.i, s2.f, Q2, key, acc, g);
+                    accumulate_d(rows, a_, s1.i, s1.f, Q1, key, acc, g);
                 }
                 __syncwarp();
             }
             // ---- entry: v0 = eta_in d, dt = ell / (N eta_in), eta_in = 1 + deta(r_in)
+            DStage se;
+            double Qe[4] = {0.0, 0.0, 0.0, 0.0};
             if (act) {
-                const double etab = vb[0] * R.d[0] + vb[1] * R.d[1] + vb[2] * R.d[2] - dtb * dt / eta_in;
-                DStage se;
-                dstage_eval(g, rin, se);
-                const size_t nx = (size_t)g.n[0], nxy = (size_t)g.n[0] * g.n[1];
-                const size_t base = (size_t)se.i[0] + (size_t)se.i[1] * nx + (size_t)se.i[2] * nxy;
-                for (int c = 0; c < 8; ++c) {
-                    const double w = ((c & 1) ? se.f[0] : 1.0 - se.f[0]) * ((c & 2) ? se.f[1] : 1.0 - se.f[1]) *
-                                     ((c & 4) ? se.f[2] : 1.0 - se.f[2]);
-                    const size_t node = base + (size_t)(c & 1) + (size_t)((c >> 1) & 1) * nx + (size_t)(c >> 2) * nxy;
-                    atomicAdd(acc + bounded(node, (size_t)g.n[0] * g.n[1] * g.n[2], g.err) * 4, w * etab);
-                }
+                Qe[0] = vb[0] * R.d[0] + vb[1] * R.d[1] + vb[2] * R.d[2] - dtb * dt / eta_in;
+                split_point(g, rin, se.i, se.f);
             }
+            accumulate_d(rows, act, se.i, se.f, Qe, key, acc, g);
+            flush_rows_d(rows, key != kNoKey, key, acc, g);
         }
     }
 }

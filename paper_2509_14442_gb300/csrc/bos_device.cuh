@@ -308,15 +308,6 @@ __device__ __forceinline__ float4 trilinear(const F4P* s, uint32_t o, float f0, 
     return lerp4(b0, b1, f2);
 }
 
-__device__ __forceinline__ D4 dlerp(D4 a, D4 b, double t) {
-    D4 r;
-    r.x = a.x + t * (b.x - a.x);
-    r.y = a.y + t * (b.y - a.y);
-    r.z = a.z + t * (b.z - a.z);
-    r.w = a.w + t * (b.w - a.w);
-    return r;
-}
-
 __device__ __forceinline__ D4 load_d4(const D4* s, uint32_t o) {
     const double2* p = reinterpret_cast<const double2*>(s + o);
     double2 a = __ldg(p), b = __ldg(p + 1);
@@ -326,14 +317,6 @@ __device__ __forceinline__ D4 load_d4(const D4* s, uint32_t o) {
     r.z = b.x;
     r.w = b.y;
     return r;
-}
-
-__device__ __forceinline__ D4 trilinear_d(const D4* s, uint32_t o, double f0, double f1, double f2) {
-    D4 a0 = dlerp(load_d4(s, o), load_d4(s, o + 1), f0);
-    D4 a1 = dlerp(load_d4(s, o + 9), load_d4(s, o + 10), f0);
-    D4 a2 = dlerp(load_d4(s, o + 81), load_d4(s, o + 82), f0);
-    D4 a3 = dlerp(load_d4(s, o + 90), load_d4(s, o + 91), f0);
-    return dlerp(dlerp(a0, a1, f1), dlerp(a2, a3, f1), f2);
 }
 
 // Cell coordinates of a point given in grid units u = (x - o)/h - 1/2 (any type):
@@ -346,23 +329,6 @@ __device__ __forceinline__ void split_coord(T u, int n, int& i, T& f) {
     fl = fl > T(n - 2) ? T(n - 2) : fl;
     i = (int)fl;
     f = u - fl;
-}
-
-// Field at an absolute position, in T arithmetic (the FP64 and plain-FP32 paths).
-__device__ __forceinline__ void field_at(const GridDev& g, const double x[3], double& eta, double grad[3]) {
-    int i[3];
-    double f[3];
-    for (int a = 0; a < 3; ++a) {
-        double u = (x[a] - g.origin[a]) / g.h[a] - 0.5;
-        split_coord(u, g.n[a], i[a], f[a]);
-    }
-    uint32_t o = bounded(brick_offset(i[0], i[1], i[2]) + 91u, g.store_elems, g.err);
-    o = o ? o - 91u : 0u;
-    D4 v = trilinear_d(static_cast<const D4*>(g.store), o, f[0], f[1], f[2]);
-    eta = 1.0 + v.x;
-    grad[0] = v.y;
-    grad[1] = v.z;
-    grad[2] = v.w;
 }
 
 // ------------------------------------------------------------------ sampling (Sec. 2.3)

@@ -672,8 +672,8 @@ __device__ RayResult trace_full(const SceneDev& S, const FullField<T>& F, const 
             F.rhs(p, D);
             for (int a = 0; a < 3; ++a) C[a] = dt * D[a];
             for (int a = 0; a < 3; ++a) {
-                r[a] = r[a] + dt * (v[a] + (A[a] + T(2) * B[a]) / T(6));
-                v[a] = v[a] + (A[a] + T(4) * B[a] + C[a]) / T(6);
+                r[a] = r[a] + dt * (v[a] + sixth(A[a] + T(2) * B[a]));
+                v[a] = v[a] + sixth(A[a] + T(4) * B[a] + C[a]);
             }
         } else {
             full_step<T, INTEG>(F, r, v, dt);
@@ -728,8 +728,11 @@ __device__ __forceinline__ RayResult trace_ray(const SceneDev& S, const Ray& R, 
 #ifndef BOS_FWD_QUASI_MIN_BLOCKS
 #define BOS_FWD_QUASI_MIN_BLOCKS 4        // quasi-linear tracing through the cell marcher (3 blocks: 3 % slower a step)
 #endif
+#ifndef BOS_FWD_FP64_MIN_BLOCKS
+#define BOS_FWD_FP64_MIN_BLOCKS 3         // float64: its pipe is full with a few warps, the cell's polynomial is 64 registers
+#endif
 constexpr int render_min_blocks(int mode, int integ, bool conn, bool save) {
-    return integ == 2 ? BOS_FWD_QUASI_MIN_BLOCKS
+    return mode == 4 ? BOS_FWD_FP64_MIN_BLOCKS : integ == 2 ? BOS_FWD_QUASI_MIN_BLOCKS
            : (mode != 1 && mode != 2) || integ != 0 ? BOS_FWD_MIN_BLOCKS
            : save ? (conn ? BOS_FWD_STAGE_CONN_MIN_BLOCKS : BOS_FWD_STAGE_MIN_BLOCKS) : BOS_FWD_MARCH_MIN_BLOCKS;
 }
