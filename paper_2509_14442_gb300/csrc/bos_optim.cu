@@ -86,47 +86,120 @@ __device__ __forceinline__ uint32_t morton2(uint32_t x, uint32_t y) {
     return spread(x) | (spread(y) << 1);
 }
 
-// One block sorts a pixel list (n <= kSortMax) by the Morton key of (px, py), bitonic
-// sort in shared memory; entries past n are padded with the largest key.
+// One block sorts a pixel list (n <= kSortMax) by the Morton key of (px, py): a least-significant
+// digit radix sort, eight bits per pass, as many passes as the largest key has digits (two for
+// a 100 x 100 image).  Warp w owns elements [32 w R, 32 (w + 1) R) in R rounds of a lane each; the
+// lanes of a round that share a digit find one another with match.any, so ranks are stable and
+// need no atomics.  Elements wait in registers while the block scatters them through shared
+// memory.  What bounds it: the latency of its dependent steps on the one SM.  A reconstruction
+// iteration of 5000 pixels (64^3 cells, 2 rays each): 528 us with the bitonic sort that stood
+// here, whose 91 passes took 107 us, 436 us so.
+// A warp's counters are a row of 257: counting (any digit) and the scan (8 digits x 4 groups of
+// warps per warp) both spread over the banks.
 constexpr int kSortMax = 16384;
 constexpr int kSortThreads = 1024;
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kSortRow = 257;
 
-__global__ void __launch_bounds__(kSortThreads) sort_pixels_kernel(int32_t* __restrict__ pix, int n, int width,
-                                                                   int m) {
+constexpr size_t sort_smem_bytes(int n) { return (2 * (size_t)n + kSortWarps * kSortRow) * sizeof(uint32_t); }
+
+template <int ROUNDS>
+__global__ void __launch_bounds__(kSortThreads) sort_pixels_kernel(int32_t* __restrict__ pix, int n, int width) {
     extern __shared__ uint32_t sh[];
-    uint32_t* key = sh;
-    uint32_t* val = sh + m;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        if (i < n) {
-            const uint32_t p = (uint32_t)pix[i];
-            key[i] = morton2(p % (uint32_t)width, p / (uint32_t)width);
-            val[i] = p;
-        } else {
-            key[i] = 0xffffffffu;
-            val[i] = 0xffffffffu;
-        }
-    }
+    uint32_t* const keys = sh;
+    uint32_t* const vals = sh + n;
+    uint32_t* const hist = sh + 2 * n;
+    __shared__ uint32_t wsum[kSortWarps], all_bits;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int R = (n + kSortThreads - 1) / kSortThreads;      // <= ROUNDS
+    const int first = w * 32 * R + lane;
+    uint32_t* const mine = hist + w * kSortRow;
+    uint32_t key[ROUNDS], val[ROUNDS], rank[ROUNDS], bits = 0;
+    if (threadIdx.x == 0) all_bits = 0;
     __syncthreads();
-    for (int k = 2; k <= m; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < m; i += blockDim.x) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const bool up = (i & k) == 0;
-                    const uint32_t a = key[i], b = key[l];
-                    if ((a > b) == up) {
-                        key[i] = b;
-                        key[l] = a;
-                        const uint32_t t = val[i];
-                        val[i] = val[l];
-                        val[l] = t;
-                    }
-                }
-            }
-            __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const int e = first + 32 * r;
+        key[r] = val[r] = rank[r] = 0;
+        if (r < R && e < n) {
+            val[r] = (uint32_t)pix[e];
+            key[r] = morton2(val[r] % (uint32_t)width, val[r] / (uint32_t)width);
+            bits |= key[r];
         }
     }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) pix[i] = (int32_t)val[i];
+    bits = __reduce_or_sync(0xffffffffu, bits);
+    if (lane == 0) atomicOr(&all_bits, bits);
+    __syncthreads();
+    bits = all_bits;
+    for (int shift = 0; shift < 32 && (bits >> shift) != 0; shift += 8) {
+        for (int i = threadIdx.x; i < kSortWarps * kSortRow; i += kSortThreads) hist[i] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < ROUNDS; ++r) {
+            const bool on = r < R && first + 32 * r < n;
+            const unsigned act = __ballot_sync(0xffffffffu, on);
+            if (on) {
+                const uint32_t d = (key[r] >> shift) & 255u;
+                const unsigned peers = __match_any_sync(act, d);
+                const uint32_t before = mine[d];
+                rank[r] = before + __popc(peers & ((1u << lane) - 1u));
+                __syncwarp(act);
+                if (lane == __ffs(peers) - 1) mine[d] = before + __popc(peers);
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+        // exclusive prefix sums over (digit, warp): thread t takes digit t / 4 of warps 8 (t % 4) ..
+        uint32_t c[8], sum = 0;
+        uint32_t* const col = hist + (threadIdx.x & 3) * 8 * kSortRow + (threadIdx.x >> 2);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            c[k] = col[k * kSortRow];
+            sum += c[k];
+        }
+        uint32_t incl = sum;
+#pragma unroll
+        for (int m = 1; m < 32; m <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xffffffffu, incl, m);
+            if (lane >= m) incl += o;
+        }
+        if (lane == 31) wsum[w] = incl;
+        __syncthreads();
+        uint32_t base = lane < w ? wsum[lane] : 0u;
+        base = __reduce_add_sync(0xffffffffu, base) + incl - sum;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            col[k * kSortRow] = base;
+            base += c[k];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < ROUNDS; ++r)
+            if (r < R && first + 32 * r < n) {
+                const uint32_t at = mine[(key[r] >> shift) & 255u] + rank[r];
+                keys[at] = key[r];
+                vals[at] = val[r];
+            }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < ROUNDS; ++r)
+            if (r < R && first + 32 * r < n) {
+                key[r] = keys[first + 32 * r];
+                val[r] = vals[first + 32 * r];
+            }
+    }
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r)
+        if (r < R && first + 32 * r < n) pix[first + 32 * r] = (int32_t)val[r];
+}
+
+template <int ROUNDS>
+static cudaError_t launch_sort_pixels(int32_t* pix, int n, int width, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(sort_pixels_kernel<ROUNDS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sort_smem_bytes(ROUNDS * kSortThreads));
+    if (e != cudaSuccess) return e;
+    sort_pixels_kernel<ROUNDS><<<1, kSortThreads, sort_smem_bytes(n), st>>>(pix, n, width);
+    return cudaGetLastError();
 }
 
 }  // namespace bos
@@ -186,14 +259,12 @@ bos_status_t bos_sort_pixels(int32_t* pix_dev, int64_t npix, int width, int heig
         bos::set_last_error("bos_sort_pixels: need 1 <= npix <= 16384 and an image of at most 65535 x 65535");
         return BOS_ERR_INVALID_ARG;
     }
-    int m = 1;
-    while (m < npix) m <<= 1;
-    const size_t smem = 2 * (size_t)m * sizeof(uint32_t);
-    cudaError_t e = cudaFuncSetAttribute(bos::sort_pixels_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(2 * bos::kSortMax * sizeof(uint32_t)));
-    if (e != cudaSuccess) return BOS_ERR_CUDA;
-    bos::sort_pixels_kernel<<<1, bos::kSortThreads, smem, (cudaStream_t)stream>>>(pix_dev, (int)npix, width, m);
-    return cudaGetLastError() == cudaSuccess ? BOS_OK : BOS_ERR_CUDA;
+    const int n = (int)npix;
+    const cudaStream_t st = (cudaStream_t)stream;
+    const cudaError_t e = n <= 2 * bos::kSortThreads   ? bos::launch_sort_pixels<2>(pix_dev, n, width, st)
+                          : n <= 8 * bos::kSortThreads ? bos::launch_sort_pixels<8>(pix_dev, n, width, st)
+                                                       : bos::launch_sort_pixels<16>(pix_dev, n, width, st);
+    return e == cudaSuccess ? BOS_OK : BOS_ERR_CUDA;
 }
 
 bos_status_t bos_counter_add(uint64_t* counter_dev, uint64_t inc, void* stream) {
