@@ -459,6 +459,39 @@ __device__ __forceinline__ void rows_flush(float* rows, bool flag, uint32_t key,
     __syncwarp();
 }
 
+// The same where neighbouring rays share few cells: every flagged lane adds its own rows, eight
+// 16-byte atomics that nothing waits for.  Then a quarter's lanes are in several cells, and
+// rows_flush takes a pass of dependent shared loads and sums for each.
+__device__ __forceinline__ void rows_scatter(bool flag, uint32_t key, CellRows& r, float* acc, int nx, int nxy,
+                                             uint32_t ncells, int* err) {
+    if (!flag) return;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const uint32_t off = (uint32_t)(c & 1) + (uint32_t)((c >> 1) & 1) * (uint32_t)nx + (uint32_t)(c >> 2) * (uint32_t)nxy;
+        atomicAdd(reinterpret_cast<float4*>(acc) + bounded(key + off, ncells, err), to4(r.c[c]));
+    }
+    rows_clear(r);
+}
+
+template <bool SCATTER>
+__device__ __forceinline__ void rows_out(float* rows, bool flag, uint32_t key, CellRows& r, float* acc, int nx, int nxy,
+                                         uint32_t ncells, int* err) {
+    if constexpr (SCATTER) rows_scatter(flag, key, r, acc, nx, nxy, ncells, err);
+    else rows_flush(rows, flag, key, r, acc, nx, nxy, ncells, err);
+}
+
+// Whether a launch's lanes are sparse enough for that: per cell of the grid's smallest cross
+// section at most 12, with the refracted connection (whose two rays visit other cells) at most
+// 24.  Whole steps at n lanes per cell, rows_flush -> rows_scatter: 200x200x150 cells, n = 0.7: 1306 ->
+// 1075 us; 64x64x48 cells, n = 7: 357 -> 335; a 64^3 minibatch, n = 2.4: 437 -> 390; 128x128x96 cells with
+// the connection, n = 21: 6.37 -> 5.70 ms; even at n = 12; 200x200x150 cells, n = 19: 9.6 -> 10.0 ms, 40: 19.0 ->
+// 20.7 ms; 24x24x18 cells, n = 83: 204 -> 260 us.
+__host__ __device__ __forceinline__ bool sparse_lanes(const SceneDev& S, const TileShape& ts, bool conn) {
+    const long long nx = S.g.n[0], ny = S.g.n[1], nz = S.g.n[2];
+    const long long longest = nx > ny ? (nx > nz ? nx : nz) : (ny > nz ? ny : nz);
+    return (long long)tile_count(S, ts) * 32 <= (conn ? 24 : 12) * (nx * ny * nz / longest);
+}
+
 // Value and fraction derivatives of the cell polynomial.
 struct PolyGrad {
     Cell2 v, x, y, z;
@@ -528,7 +561,7 @@ __device__ __forceinline__ bool tile_needs_stages(const CkptDev& ck, const TileS
 // quasi-linear tracer, whose points lie on the straight line: the same recurrences for V and
 // the adjoints without the point adjoints (its outputs are linear in the sampled values), for
 // every ray.
-template <class E, bool CONN, bool QUASI = false>
+template <class E, bool CONN, bool QUASI, bool SCATTER>
 __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& ck, const AdjDev& adj,
                                              const CompField<E>& F, const TileShape& ts, int t, int lane, float* rows,
                                              float* acc, uint32_t ncells, int* err, int* deferred, double* xlum) {
@@ -675,7 +708,7 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                     moved = march_point<false, QUASI>(F, L, m, h, dr, f);
                 }
                 if (__any_sync(0xffffffffu, moved)) {
-                    rows_flush(rows, moved && used, key, row, acc, nx, nxy, ncells, err);
+                    rows_out<SCATTER>(rows, moved && used, key, row, acc, nx, nxy, ncells, err);
                     if (moved) key = march_key(m, (uint32_t)nx, (uint32_t)nxy);
                 }
                 if (on) {
@@ -730,7 +763,7 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                 moved = false;
                 if (on) moved = march_point<false, QUASI>(F, L, m, h, QUASI ? dr : fma3(0.75f, c, fma3(-0.5f, V, dr)), f);
                 if (__any_sync(0xffffffffu, moved)) {
-                    rows_flush(rows, moved && used, key, row, acc, nx, nxy, ncells, err);
+                    rows_out<SCATTER>(rows, moved && used, key, row, acc, nx, nxy, ncells, err);
                     if (moved) key = march_key(m, (uint32_t)nx, (uint32_t)nxy);
                 }
                 if (on) {
@@ -773,7 +806,7 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                 }
                 h = add2(h, splat2(-1.0f));
             }
-            rows_flush(rows, used, key, row, acc, nx, nxy, ncells, err);
+            rows_out<SCATTER>(rows, used, key, row, acc, nx, nxy, ncells, err);
             if constexpr (CONN) {
                 if (proj && act) {
                     Frac3 f;
@@ -1091,7 +1124,8 @@ __device__ __forceinline__ void adjoint_tile(const SceneDev& S, const CkptDev& c
 // recompute (relative L2 2e-7 .. 7e-7).  128 registers and 16 warps beat 168 and 12 by 2 to 3 %;
 // with the connection, whose spills then reach the loop, 168 are 7 % faster.  Summing the rows
 // of a whole warp one cell at a time, with branches around the row reads, took 62.7 ms.
-template <class E, bool CONN, bool QUASI, bool FEW>
+// SCATTER: rows_scatter (see sparse_lanes).
+template <class E, bool CONN, bool QUASI, bool FEW, bool SCATTER>
 __global__ void __launch_bounds__(kAdjWarps * 32, FEW ? 1 : CONN ? BOS_REV_CONN_MIN_BLOCKS : BOS_REV_MIN_BLOCKS)
     reverse_kernel(SceneDev S, CkptDev ck, AdjDev adj, WorkDev wk) {
     extern __shared__ float4 smem4[];
@@ -1108,7 +1142,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, FEW ? 1 : CONN ? BOS_REV_CONN_
         if (lane == 0) t = atomicAdd(wk.tile_counter, 1);
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= ntiles) break;
-        reverse_tile<E, CONN, QUASI>(S, ck, adj, F, ts, t, lane, rows, reinterpret_cast<float*>(adj.acc), ncells, S.g.err,
+        reverse_tile<E, CONN, QUASI, SCATTER>(S, ck, adj, F, ts, t, lane, rows, reinterpret_cast<float*>(adj.acc), ncells, S.g.err,
                               wk.tile_counter + 1, xlum);
     }
 }
@@ -1513,10 +1547,13 @@ __global__ void __launch_bounds__(kAdjWarps * 32, BOS_REV_MIN_BLOCKS)
         g = __shfl_sync(0xffffffffu, g, 0);
         if (g >= total) break;
         const BatchJob& J = jobs[batch_job_of(jobs, njobs, g)];
-        reverse_tile<E, false, QUASI>(J.S, J.ck, J.adj, comp_field<E>(J.S.g),
-                                      tile_shape(J.S.cam.width, J.S.cam.height, J.S.cam.spp), J.tile0 + (g - J.first),
-                                      lane, rows, reinterpret_cast<float*>(J.adj.acc),
-                                      (uint32_t)J.S.g.n[0] * J.S.g.n[1] * J.S.g.n[2], J.S.g.err, counter + 1, nullptr);
+        const TileShape ts = tile_shape(J.S.cam.width, J.S.cam.height, J.S.cam.spp);
+        const uint32_t ncells = (uint32_t)J.S.g.n[0] * J.S.g.n[1] * J.S.g.n[2];
+        float* const acc = reinterpret_cast<float*>(J.adj.acc);
+        const int t = J.tile0 + (g - J.first);
+        // (a choice of rows_scatter per job: 9.5 ms for a mix of six requests instead of 8.55, by spills)
+        reverse_tile<E, false, QUASI, false>(J.S, J.ck, J.adj, comp_field<E>(J.S.g), ts, t, lane, rows, acc, ncells,
+                                             J.S.g.err, counter + 1, nullptr);
     }
 }
 
@@ -1612,15 +1649,15 @@ cudaError_t launch_gradient(const GridDev& g, const float4* acc, const float* T,
     return cudaGetLastError();
 }
 
-template <class E, bool CONN, bool QUASI, bool FEW>
+template <class E, bool CONN, bool QUASI, bool FEW, bool SCATTER>
 static cudaError_t launch_reverse_f(const SceneDev& S, const CkptDev& ck, const AdjDev& adj, const WorkDev& w,
                                     int num_sms, cudaStream_t st) {
-    const size_t smem = (size_t)kAdjWarps * 32 * kRow * sizeof(float);
+    const size_t smem = SCATTER ? 0 : (size_t)kAdjWarps * 32 * kRow * sizeof(float);
     int per_sm = 0;
-    cudaError_t e = occupancy_prefer_l1(reverse_kernel<E, CONN, QUASI, FEW>, kAdjWarps * 32, smem, per_sm);
+    cudaError_t e = occupancy_prefer_l1(reverse_kernel<E, CONN, QUASI, FEW, SCATTER>, kAdjWarps * 32, smem, per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    reverse_kernel<E, CONN, QUASI, FEW><<<num_sms * per_sm, kAdjWarps * 32, smem, st>>>(S, ck, adj, w);
+    reverse_kernel<E, CONN, QUASI, FEW, SCATTER><<<num_sms * per_sm, kAdjWarps * 32, smem, st>>>(S, ck, adj, w);
     return cudaGetLastError();
 }
 
@@ -1630,9 +1667,13 @@ static cudaError_t launch_reverse_f(const SceneDev& S, const CkptDev& ck, const 
 template <class E, bool CONN, bool QUASI>
 static cudaError_t launch_reverse(const SceneDev& S, const CkptDev& ck, const AdjDev& adj, const WorkDev& w, int num_sms,
                                   cudaStream_t st) {
-    if (tile_count(S, tile_shape(S.cam.width, S.cam.height, S.cam.spp)) <= num_sms * kFewTiles)
-        return launch_reverse_f<E, CONN, QUASI, true>(S, ck, adj, w, num_sms, st);
-    return launch_reverse_f<E, CONN, QUASI, false>(S, ck, adj, w, num_sms, st);
+    const TileShape ts = tile_shape(S.cam.width, S.cam.height, S.cam.spp);
+    const bool sparse = sparse_lanes(S, ts, CONN);
+    if (tile_count(S, ts) <= num_sms * kFewTiles)
+        return sparse ? launch_reverse_f<E, CONN, QUASI, true, true>(S, ck, adj, w, num_sms, st)
+                      : launch_reverse_f<E, CONN, QUASI, true, false>(S, ck, adj, w, num_sms, st);
+    return sparse ? launch_reverse_f<E, CONN, QUASI, false, true>(S, ck, adj, w, num_sms, st)
+                  : launch_reverse_f<E, CONN, QUASI, false, false>(S, ck, adj, w, num_sms, st);
 }
 
 template <class E, bool CONN>
