@@ -108,6 +108,8 @@ L2_BYTES = 129 * 2 ** 20
 #     evaluations 3 x (6 + 4 x 36) = 450, the adjoint of D per stage 3 x 36 = 108, the
 #     transpose of the step's linear combinations 66, the path-length adjoint 11, and the
 #     corner scatter per stage (3 complements, 8 weights x 2, 8 x 4 FMAs) 3 x 83 = 249:  1240
+#     (reverse_kernel makes no recompute and two of the three stages' evaluations and scatters;
+#     the count stays that of the stage-by-stage adjoint, so that rates compare over time)
 #   one-sweep quasi-linear adjoint: per line sample the point, fractions and value 96, the
 #     adjoint of D 9 and the corner scatter 83 (2 samples: 376), the velocity adjoint 24:  400
 FLOPS_PER_STEP = {"rkn": 356, "quasi": 241}
