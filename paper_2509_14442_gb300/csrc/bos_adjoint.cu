@@ -1712,8 +1712,10 @@ cudaError_t launch_backward_fp64(const SceneDev& S, const CkptDev& ck, const Adj
                                  const float* T, void* dLdT, bool f64, int num_sms, cudaStream_t st) {
     if (S.it.integrator != 0 || S.L.mode == 2 || adj.seg == nullptr || ck.every > 64) return cudaErrorNotSupported;
     const int blocks = num_sms * 8 < kAdjMaxBlocks ? num_sms * 8 : kAdjMaxBlocks;
-    if (f64) adjoint_fp64_kernel<double><<<blocks, kAdjWarps * 32, 0, st>>>(S, ck, adj, w);
-    else adjoint_fp64_kernel<float><<<blocks, kAdjWarps * 32, 0, st>>>(S, ck, adj, w);
+    const int threads =
+        fp64_threads(tile_count(S, tile_shape(S.cam.width, S.cam.height, S.cam.spp)), num_sms, kAdjWarps * 32);
+    if (f64) adjoint_fp64_kernel<double><<<blocks, threads, 0, st>>>(S, ck, adj, w);
+    else adjoint_fp64_kernel<float><<<blocks, threads, 0, st>>>(S, ck, adj, w);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const double* acc = reinterpret_cast<const double*>(adj.acc);

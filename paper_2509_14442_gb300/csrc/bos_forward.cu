@@ -948,11 +948,12 @@ cudaError_t launch_build_store(const GridDev& g, const float* T, void* store, cu
 template <int MODE, int INTEG, bool CONN, bool FEW = false, bool SAVE = true>
 static cudaError_t launch_render_c(const SceneDev& S, const RenderOut& o, const WorkDev& w, const CkptDev& ck,
                                    int num_sms, cudaStream_t st) {
-    int per_sm = 0;
-    cudaError_t e = occupancy_prefer_l1(render_kernel<MODE, INTEG, CONN, FEW, SAVE>, 128, 0, per_sm);
+    int threads = kRenderThreads, per_sm = 0;
+    if (MODE == 4) threads = fp64_threads(tile_count(S, tile_shape(S.cam.width, S.cam.height, S.cam.spp)), num_sms, threads);
+    cudaError_t e = occupancy_prefer_l1(render_kernel<MODE, INTEG, CONN, FEW, SAVE>, threads, 0, per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    render_kernel<MODE, INTEG, CONN, FEW, SAVE><<<num_sms * per_sm, 128, 0, st>>>(S, o, w, ck);
+    render_kernel<MODE, INTEG, CONN, FEW, SAVE><<<num_sms * per_sm, threads, 0, st>>>(S, o, w, ck);
     return cudaGetLastError();
 }
 

@@ -53,6 +53,12 @@ struct RenderOut {
 // such a form (180 to 240 registers) keeps resident.
 constexpr int kFewTiles = 8;
 
+// Threads per block of a float64 tracer's launch.  Its few tiles are bound by the SMs' float64
+// pipes, and blocks of several warps give some SMs twice the tiles of others: a step of 864 tiles
+// (64x64x48 cells, 192 x 144 rays) took 10.61 ms so, 9.70 ms in blocks of one warp.  (The float32
+// tracers gain nothing: an SM's four schedulers do not share what bounds them.)
+inline int fp64_threads(int tiles, int num_sms, int block) { return tiles <= num_sms * kFewTiles ? 32 : block; }
+
 constexpr size_t kTileCounterBytes = 3 * sizeof(int);
 
 struct WorkDev {
