@@ -270,8 +270,8 @@ __device__ __forceinline__ void unpark_ray(volatile double* p, Ray& R) {
     R.ell = p[5 * kRenderThreads];
 }
 
-// Steps of one ray through the cell marcher (QUASI: quasi-linear, else Sharma's), in the scaled variables V = dt dv and
-// a = (dt^2 / 6) D (metres per step), so that
+// Steps of one ray through the cell marcher (QUASI: quasi-linear, else Sharma's), in the scaled
+// variables V = dt dv and a = (dt^2 / 6) D (metres per step), so that
 //   p2 = S(n+1/2) + dr + V/2 + 3a/4,   p3 = S(n+1) + dr + V + 3b
 //   dr += V + a + 2b,                  V += a + 4b + c
 // with a, b, c taken at dr, p2 and p3, and every constant exact in float32.  The next step's
@@ -282,9 +282,8 @@ __device__ __forceinline__ void unpark_ray(volatile double* p, Ray& R) {
 // excess sum |dS + inc| - |dS| is d.(sum of inc) + sum (|inc|^2 - (d.inc)^2) / (2L + d.inc):
 // the first term is the end deviation, so only the small second one is summed.
 // Quasi-linear tracing (Sec. 2.2) takes the same weights at the start, middle and end of each
-// step on the straight line: the end sample is the next step's start sample.  Render and adjoint
-// of 256x256x192 cells at 1024 x 768 rays: 14.21 ms with four gathers per step pair through the
-// 64-bit line position, 12.82 ms so.
+// step on the straight line: the end sample is the next step's start sample.  (Only where nothing
+// is kept for an adjoint, see line_run.)
 template <class E, bool QUASI>
 __device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
                                           volatile double* park, float dr_end[3], float dv_end[3], float& excess_end,
@@ -397,10 +396,12 @@ __device__ __forceinline__ P3 line_frac(const long long U[3]) {
     return p3(fr(U[0]), fr(U[1]), fr(U[2]));
 }
 
-// D = (1 + deta) grad eta at line position U (fractions fr) plus deviation q.
-template <class E>
+// D = (1 + deta) grad eta at line position U (fractions fr) plus deviation q (LINE: on the line
+// itself; q and ih are not looked at).
+template <bool LINE = false, class E>
 __device__ __forceinline__ P3 stage_rhs(const CompField<E>& F, const long long U[3], P3 fr, P3 ih, P3 q, StageCell& m) {
-    const P3 u = P3{fmaf(q.x, ih.x, fr.x), fma2(q.yz, ih.yz, fr.yz)};
+    P3 u = fr;
+    if constexpr (!LINE) u = P3{fmaf(q.x, ih.x, fr.x), fma2(q.yz, ih.yz, fr.yz)};
     float f[3] = {u.x, lo2(u.yz), hi2(u.yz)};
     const int c0 = (int)(U[0] >> 32), c1 = (int)(U[1] >> 32), c2 = (int)(U[2] >> 32);
     const uint32_t top = max(__float_as_uint(f[0]), max(__float_as_uint(f[1]), __float_as_uint(f[2])));
@@ -506,6 +507,54 @@ __device__ __forceinline__ void stage_run(const CompField<E>& F, const Ray& R, c
     }
 }
 
+// Quasi-linear steps of one ray whose end state is kept: Sharma's weights, the field at the start,
+// middle and end of every step on the line; the end sample is the next step's start sample.
+// Stage by stage on the fixed-point line like stage_run, and explicitly rounded for the same
+// reason: the luminance is read at a float32 texel coordinate, so an end state an ulp away moves
+// the pixels beside one of its steps by 1e-5 of the image, and a residual of one per cent, which
+// seeds the gradient, by a few per mille.  Render and adjoint of 256x256x192 cells at 1024 x 768
+// rays: 14.2 ms with an address and four gathers per pair of steps, 13.3 ms so (12.8 ms marched;
+// 168 registers 13.7 ms, 96 13.3 ms).
+template <class E>
+__device__ __forceinline__ void line_run(const CompField<E>& F, const Ray& R, const CompConst& k, CompState& st) {
+    const P3 d = p3(kept(k.dhat[0]), kept(k.dhat[1]), kept(k.dhat[2]));
+    const float dt = kept(k.dt), len2 = kept(2.0f * k.step_len);
+    long long U[3], dU[3];
+    for (int a = 0; a < 3; ++a) {
+        U[a] = st.U[a];
+        dU[a] = k.dU[a];
+        asm volatile("" : "+l"(U[a]), "+l"(dU[a]));   // see kept()
+    }
+    StageCell m;
+    m.c[0] = m.c[1] = m.c[2] = -2;   // no cell
+    m.bc = {0xffffffffu, 0u};
+    const P3 none = {0.0f, 0ull};
+    P3 dr = none, cr = none, dv = none, cv = none;
+    float excess = 0.0f;
+    P3 A = mul3(dt, stage_rhs<true>(F, U, line_frac(U), none, none, m));
+    for (int n = 0; n < R.N; ++n) {
+        long long U2[3];
+        for (int a = 0; a < 3; ++a) {
+            U2[a] = U[a] + (dU[a] >> 1);
+            U[a] += dU[a];
+        }
+        const P3 B = mul3(dt, stage_rhs<true>(F, U2, line_frac(U2), none, none, m));
+        const P3 C = mul3(dt, stage_rhs<true>(F, U, line_frac(U), none, none, m));
+        const P3 inc = mul3(dt, fma3(1.0f / 6.0f, fma3(2.0f, B, A), dv));
+        const P3 s = add3(fma3(4.0f, B, A), C);
+        kahan3(dr, cr, sub3(inc, cr));
+        kahan3(dv, cv, P3{fmaf(s.x, 1.0f / 6.0f, -cv.x), fma2(s.yz, splat2(1.0f / 6.0f), neg2(cv.yz))});
+        A = C;
+        const float di = dot3(d, inc);   // as in stage_run
+        excess = fmaf(fmaf(-di, di, dot3(inc, inc)), rcp_approx(__fadd_rn(len2, di)), excess);
+    }
+    st.dr[0] = dr.x, st.dr[1] = lo2(dr.yz), st.dr[2] = hi2(dr.yz);
+    st.cr[0] = cr.x, st.cr[1] = lo2(cr.yz), st.cr[2] = hi2(cr.yz);
+    st.dv[0] = dv.x, st.dv[1] = lo2(dv.yz), st.dv[2] = hi2(dv.yz);
+    st.cv[0] = cv.x, st.cv[1] = lo2(cv.yz), st.cv[2] = hi2(cv.yz);
+    st.excess = __fadd_rn(excess, dot3(d, sub3(dr, cr)));
+}
+
 // Integrate one ray of the comp path (N > 0) from the pinhole rs; optionally store its
 // checkpoints every K steps in `state` (slot `ray`).  Leaves the end state in st.
 template <class E, int INTEG>
@@ -517,6 +566,8 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
     comp_setup(S, F, rs, R, st, k, eta_in, rin);
     if constexpr (INTEG == 0) {
         stage_run(F, R, k, ck, state, ray, st, apart_cells);
+    } else if constexpr (INTEG == 2) {
+        line_run(F, R, k, st);
     } else {
         BrickCache bc = {0xffffffffu, 0u};
         const int K = ck.every;
@@ -539,20 +590,16 @@ __device__ __forceinline__ void comp_end(const CompState& st, float dr[3], float
     }
 }
 
-// End deviation, path excess and entry index of a ray: Sharma without checkpoints and the
-// quasi-linear tracer march from cell to cell, everything else goes stage by stage.
+// End deviation, path excess and entry index of a ray: Sharma and the quasi-linear tracer march
+// from cell to cell where nothing is kept for an adjoint; everything else goes stage by stage.
 template <class E, int INTEG, bool CONN, bool SAVE>
 __device__ __forceinline__ void trace_end(const SceneDev& S, const CompField<E>& F, const double rs[3], Ray& R,
                                           volatile double* park,
                                           const CkptDev& ck, float4* state, long long ray, float dr[3], float dv[3],
                                           float& excess, float& eta, float* apart) {
     if constexpr (INTEG != 1) park_ray(park, R);   // (classical steps have registers to spare)
-    if constexpr (INTEG == 2 || (INTEG == 0 && !SAVE)) {
+    if constexpr (INTEG != 1 && !SAVE) {
         march_run<E, INTEG == 2>(S, F, rs, R, park, dr, dv, excess, eta);
-        if (INTEG == 2 && state != nullptr) {   // the end state, from which the adjoint reverses the ray
-            state[0 * ck.nrays + ray] = make_float4(dr[0], dr[1], dr[2], excess);
-            state[1 * ck.nrays + ray] = make_float4(dv[0], dv[1], dv[2], 0.0f);
-        }
     } else {
         CompState st;
         double eta_in;
@@ -560,6 +607,10 @@ __device__ __forceinline__ void trace_end(const SceneDev& S, const CompField<E>&
         eta = (float)eta_in;
         comp_end(st, dr, dv);
         excess = st.excess;
+        if (INTEG == 2 && state != nullptr) {   // the end state, from which the adjoint reverses the ray
+            state[0 * ck.nrays + ray] = make_float4(dr[0], dr[1], dr[2], excess);
+            state[1 * ck.nrays + ray] = make_float4(dv[0], dv[1], dv[2], 0.0f);
+        }
     }
     if constexpr (INTEG != 1) unpark_ray(park, R);
 }
@@ -726,13 +777,17 @@ __device__ __forceinline__ RayResult trace_ray(const SceneDev& S, const Ray& R, 
 #define BOS_FWD_STAGE_CONN_MIN_BLOCKS 3   // the same with the refracted connection
 #endif
 #ifndef BOS_FWD_QUASI_MIN_BLOCKS
-#define BOS_FWD_QUASI_MIN_BLOCKS 4        // quasi-linear tracing through the cell marcher (3 blocks: 3 % slower a step)
+#define BOS_FWD_QUASI_MIN_BLOCKS 4        // quasi-linear tracing through the cell marcher
+#endif
+#ifndef BOS_FWD_LINE_MIN_BLOCKS
+#define BOS_FWD_LINE_MIN_BLOCKS 4         // quasi-linear tracing whose end state is kept
 #endif
 #ifndef BOS_FWD_FP64_MIN_BLOCKS
 #define BOS_FWD_FP64_MIN_BLOCKS 3         // float64: its pipe is full with a few warps, the cell's polynomial is 64 registers
 #endif
 constexpr int render_min_blocks(int mode, int integ, bool conn, bool save) {
-    return mode == 4 ? BOS_FWD_FP64_MIN_BLOCKS : integ == 2 ? BOS_FWD_QUASI_MIN_BLOCKS
+    return mode == 4 ? BOS_FWD_FP64_MIN_BLOCKS
+           : integ == 2 ? (save ? BOS_FWD_LINE_MIN_BLOCKS : BOS_FWD_QUASI_MIN_BLOCKS)
            : (mode != 1 && mode != 2) || integ != 0 ? BOS_FWD_MIN_BLOCKS
            : save ? (conn ? BOS_FWD_STAGE_CONN_MIN_BLOCKS : BOS_FWD_STAGE_MIN_BLOCKS) : BOS_FWD_MARCH_MIN_BLOCKS;
 }
@@ -841,7 +896,7 @@ __global__ void __launch_bounds__(128, render_min_blocks(MODE, INTEG, false, fal
         const TileShape ts = tile_shape(J.S.cam.width, J.S.cam.height, J.S.cam.spp);
         unsigned long long my_steps = 0;
         const int t = J.tile0 + (g - J.first);
-        if (INTEG == 0 && J.ck.state == nullptr)
+        if (J.ck.state == nullptr)
             render_tile<MODE, INTEG, false, false>(J.S, J.out, J.wk, J.ck, ts, t, lane, my_steps);
         else
             render_tile<MODE, INTEG, false, true>(J.S, J.out, J.wk, J.ck, ts, t, lane, my_steps);
@@ -964,15 +1019,17 @@ static cudaError_t launch_render_t(const SceneDev& S, const RenderOut& o, const 
                                    int num_sms, cudaStream_t st) {
     if constexpr (MODE == 1 || MODE == 2) {
         const bool few = tile_count(S, tile_shape(S.cam.width, S.cam.height, S.cam.spp)) <= num_sms * kFewTiles;
-        // Sharma without checkpoints marches from cell to cell; with them the image, which seeds
-        // a gradient, keeps the stage-by-stage arithmetic that the adjoint's recompute repeats
-        if constexpr (INTEG == 0) {
+        // renders that keep nothing march from cell to cell; where the image seeds a gradient it
+        // keeps the stage-by-stage arithmetic on the fixed-point line
+        if constexpr (INTEG != 1) {
             if (ck.state == nullptr)
                 return S.L.mode == 2 ? launch_render_c<MODE, INTEG, true, false, false>(S, o, w, ck, num_sms, st)
                        : few ? launch_render_c<MODE, INTEG, false, true, false>(S, o, w, ck, num_sms, st)
                              : launch_render_c<MODE, INTEG, false, false, false>(S, o, w, ck, num_sms, st);
         }
-        if (S.L.mode == 2) return launch_render_c<MODE, INTEG, true>(S, o, w, ck, num_sms, st);
+        if constexpr (INTEG != 2) {   // (no adjoint of the refracted connection for quasi-linear rays)
+            if (S.L.mode == 2) return launch_render_c<MODE, INTEG, true>(S, o, w, ck, num_sms, st);
+        }
         // a few tiles (up to 8 warps per SM): the uncapped form
         if constexpr (INTEG != 1) {
             if (few) return launch_render_c<MODE, INTEG, false, true>(S, o, w, ck, num_sms, st);
