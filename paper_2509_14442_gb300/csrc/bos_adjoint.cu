@@ -678,15 +678,21 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
             P3 rseg = rb;
             int seg0 = n_max - to_ckpt;       // first node of the segment (the refracted sums)
             int origin = n_max / kLineSteps * kLineSteps;   // the step that the line is set up from
-            if (origin > 0 && act) set_line(S, F, rs, RR, origin, L, m);
+            if (origin > 0 && act) {
+                set_line(S, F, rs, RR, origin, L, m);
+                march_leave(m);
+            }
             f32x2 h = splat2(2.0f * (float)(n_max - origin));
             bool used = false;                // the rows hold something
             bool later = false;               // a later step of this ray has been reversed
             for (int n = n_max;; --n, --to_ckpt) {
                 const bool on = n <= N;
-                if (n < origin) {   // (the next point finds its cell again)
+                if (n < origin) {
                     origin -= kLineSteps;
-                    if (act) set_line(S, F, rs, RR, origin, L, m);
+                    if (act) {
+                        set_line(S, F, rs, RR, origin, L, m);
+                        march_leave(m);
+                    }
                     h = splat2(2.0f * (float)(n - origin));
                 }
                 // ---- the point between steps n - 1 and n

@@ -157,6 +157,17 @@ __device__ __forceinline__ void march_line(const float inv_h[3], const double u0
     m.ci = P3{kCellBias, splat2(kCellBias)};
 }
 
+// march_line leaves the ray in cell (0, 0, 0), whose polynomial is not loaded yet: the next point
+// is found by march_point<true>, or, where that would be a second copy of it, after this: the
+// indices go to -2^14 on every axis, outside any grid (at most 8192 cells), so that march_point
+// sees a change of cell and of brick (the base stays exact, and the estimate of the new cell is
+// off by one only within 2^-9 of a face, where both cells' polynomials agree to that).
+__device__ __forceinline__ void march_leave(MarchCell& m) {
+    const P3 away = {16384.0f, splat2(16384.0f)};
+    m.ci = sub3(m.ci, away);
+    m.base = add3(m.base, away);
+}
+
 // LINE: the point on the line itself (q is not looked at).
 template <bool LINE>
 __device__ __forceinline__ P3 march_frac(const MarchLine& L, const MarchCell& m, f32x2 h, P3 q) {
