@@ -673,7 +673,6 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
             float work = 0.0f;                // sum of a_.a + b_.b + c_.c
             const P3 VbN = Vb;
             P3 ulen = {0.0f, 0ull};           // quasi-linear: lenb times the unit directions so far
-            float back = 0.0f;                // and the steps reversed so far
             float tps[3] = {0.0f, 0.0f, 0.0f};
             P3 rseg = rb;
             int seg0 = n_max - to_ckpt;       // first node of the segment (the refracted sums)
@@ -791,10 +790,10 @@ __device__ __forceinline__ void reverse_tile(const SceneDev& S, const CkptDev& c
                     ab = add3(sg, Vb);
                     if (QUASI) {
                         // r_ is constant: V_ from its closed form, whose float32 error does not
-                        // build up over the steps
-                        back += 1.0f;
+                        // build up over the steps (their number from the integers: a float that
+                        // counts them stops at 2^24)
                         ulen = fma3(ln, step, ulen);
-                        Vb = add3(fma3(back, rb, VbN), ulen);
+                        Vb = add3(fma3((float)(N - n + 1), rb, VbN), ulen);
                     } else {
                         Vb = add3(Vb, sg);
                     }
