@@ -363,9 +363,9 @@ constexpr int kSegFloats = 12;
 //   r' = r + V + a + 2b,  V' = V + a + 4b + c,  p2 = r + V/2 + 3a/4,  p3 = r + V + 3b
 // and solving it backwards gives, exactly,
 //   p2 = r' - V'/2 + a/4 + c/2,  r = r' - V' + 2b + c,  V = V' - a - 4b - c.
-// p3 and r' differ by b - a, second order in the step: where the forward found that below
-// kSameReverse of a cell for all steps of a ray, c is the acceleration at r' and a may stand
-// for c in p2 (it enters with a/4), so the step is reversed from (r', V') alone: no segment
+// p3 and r' differ by b - a, second order in the step.  Where the forward found |b - a| and
+// |a - c| / 4 below kSameReverse of a cell for all steps of a ray, c is the acceleration at r' and
+// c may stand for a in p2, so the step is reversed from (r', V') alone: no segment
 // recompute, no kept stage terms, and the third stage of a step and the first stage of the
 // next one are one field point with one evaluation and one scatter.  Per step that is two value
 // and gradient evaluations and two scatters, where recomputing the segment and reversing the

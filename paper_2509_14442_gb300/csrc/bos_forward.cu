@@ -449,7 +449,7 @@ __device__ __forceinline__ void stage_run(const CompField<E>& F, const Ray& R, c
     m.c[0] = m.c[1] = m.c[2] = -2;   // no cell
     m.bc = {0xffffffffu, 0u};
     P3 dr = {0.0f, 0ull}, cr = dr, dv = dr, cv = dr;
-    float excess = 0.0f, apart = 0.0f;   // apart: largest |A - B| of the steps
+    float excess = 0.0f, apart = 0.0f, change = 0.0f;   // largest |A - B| and |A - C| of the steps
     P3 A = mul3(dt, stage_rhs(F, U, line_frac(U), ih, dr, m));
     const int K = ck.every;
     int left = K;                        // steps before the next checkpoint
@@ -474,14 +474,15 @@ __device__ __forceinline__ void stage_run(const CompField<E>& F, const Ray& R, c
         const P3 inc = mul3(dt, X);
         const P3 y = P3{fmaf(dt, X.x, -cr.x), fma2(splat2(dt), X.yz, neg2(cr.yz))};
         const P3 fr = line_frac(U);
-        const P3 D = stage_rhs(F, U, fr, ih, q, m);
+        const P3 D = stage_rhs(F, U, fr, ih, q, m), C = mul3(dt, D);
+        change = fmaxf(change, maxabs3(sub3(A, C)));
         kahan3(dr, cr, y);
         // the third stage's point and the new position differ by second order in the step: where
         // their fractions round to the same bits, so does D there
         P3 A1 = {0.0f, 0ull};
         const P3 u1 = P3{fmaf(q.x, ih.x, fr.x), fma2(q.yz, ih.yz, fr.yz)};
         const P3 u2 = P3{fmaf(dr.x, ih.x, fr.x), fma2(dr.yz, ih.yz, fr.yz)};
-        if (u1.yz == u2.yz && __float_as_uint(u1.x) == __float_as_uint(u2.x)) A1 = mul3(dt, D);
+        if (u1.yz == u2.yz && __float_as_uint(u1.x) == __float_as_uint(u2.x)) A1 = C;
         else if (n + 1 < R.N) A1 = mul3(dt, stage_rhs(F, U, fr, ih, dr, m));
         const P3 s = fma3(dt, D, fma3(4.0f, B, A));
         kahan3(dv, cv, P3{fmaf(s.x, 1.0f / 6.0f, -cv.x), fma2(s.yz, splat2(1.0f / 6.0f), neg2(cv.yz))});
@@ -500,10 +501,12 @@ __device__ __forceinline__ void stage_run(const CompField<E>& F, const Ray& R, c
         state[0 * ck.nrays + ray] = make_float4(st.dr[0], st.dr[1], st.dr[2], st.cr[0]);
         state[1 * ck.nrays + ray] = make_float4(st.dv[0], st.dv[1], st.dv[2], st.cr[1]);
         state[2 * ck.nrays + ray] = make_float4(st.cv[0], st.cv[1], st.cv[2], st.cr[2]);
-        // steps that the adjoint can reverse without their stage terms: dt |A - B| / 6 within
-        // kSameReverse cells (not so: NaN, too)
+        // steps that the adjoint can reverse without their stage terms (see bos_adjoint.cu): the
+        // third stage's point is the new position, dt |A - B| / 6, and the second stage's point may
+        // take C for A, dt |A - C| / 24, both within kSameReverse cells (not so: NaN, too).  The one
+        // does not bound the other: a layer may lie between a step's middle and its end.
         const float ihm = fmaxf(F.inv_h[0], fmaxf(F.inv_h[1], F.inv_h[2]));
-        *apart_cells = apart * dt * (ihm * (1.0f / 6.0f));
+        *apart_cells = fmaxf(apart, 0.25f * change) * dt * (ihm * (1.0f / 6.0f));
     }
 }
 
