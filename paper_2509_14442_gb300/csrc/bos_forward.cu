@@ -468,14 +468,14 @@ __device__ __forceinline__ void stage_run(const CompField<E>& F, const Ray& R, c
             U[a] += dU[a];
         }
         const P3 B = mul3(dt, stage_rhs(F, U2, line_frac(U2), ih, fma3(e1, A, fma3(h1, dv, dr)), m));
-        apart = fmaxf(apart, maxabs3(sub3(A, B)));
+        apart = max_nan(apart, maxabs3(sub3(A, B)));
         const P3 q = fma3(h1, B, fma3(dt, dv, dr));
         const P3 X = fma3(1.0f / 6.0f, fma3(2.0f, B, A), dv);
         const P3 inc = mul3(dt, X);
         const P3 y = P3{fmaf(dt, X.x, -cr.x), fma2(splat2(dt), X.yz, neg2(cr.yz))};
         const P3 fr = line_frac(U);
         const P3 D = stage_rhs(F, U, fr, ih, q, m), C = mul3(dt, D);
-        change = fmaxf(change, maxabs3(sub3(A, C)));
+        change = max_nan(change, maxabs3(sub3(A, C)));
         kahan3(dr, cr, y);
         // the third stage's point and the new position differ by second order in the step: where
         // their fractions round to the same bits, so does D there
@@ -506,7 +506,7 @@ __device__ __forceinline__ void stage_run(const CompField<E>& F, const Ray& R, c
         // take C for A, dt |A - C| / 24, both within kSameReverse cells (not so: NaN, too).  The one
         // does not bound the other: a layer may lie between a step's middle and its end.
         const float ihm = fmaxf(F.inv_h[0], fmaxf(F.inv_h[1], F.inv_h[2]));
-        *apart_cells = fmaxf(apart, 0.25f * change) * dt * (ihm * (1.0f / 6.0f));
+        *apart_cells = max_nan(apart, 0.25f * change) * dt * (ihm * (1.0f / 6.0f));
     }
 }
 
@@ -656,7 +656,7 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, Ray R,
                     float pr[3], pv[3], pexcess, papart = 0.0f;
                     trace_end<E, INTEG, CONN, SAVE>(S, F, P, Rp, ray_park<1>(), ck, m == 0 ? ck.pstate : nullptr, ray, pr, pv, pexcess,
                                                     eta_p, &papart);
-                    if (!(papart <= apart)) apart = papart;
+                    apart = max_nan(apart, papart);
                     steps += (unsigned long long)Rp.N;
                     const WallRel hp = comp_wall(S, Rp, eta_p, pr, pv, 0.0f);
                     if (hp.valid)

@@ -61,7 +61,18 @@ __device__ __forceinline__ float dot3(P3 a, P3 b) {
     const f32x2 p = mul2(a.yz, b.yz);
     return fmaf(a.x, b.x, __fadd_rn(lo2(p), hi2(p)));
 }
-__device__ __forceinline__ float maxabs3(P3 a) { return fmaxf(fabsf(a.x), fmaxf(fabsf(lo2(a.yz)), fabsf(hi2(a.yz)))); }
+// The largest one; NaN where any is (fmaxf drops a NaN).
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float max_nan(float a, float b, float c) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float maxabs3(P3 a) { return max_nan(fabsf(a.x), fabsf(lo2(a.yz)), fabsf(hi2(a.yz))); }
 
 // s += x with Kahan compensation c, x already reduced by c (y = x - c).
 __device__ __forceinline__ void kahan3(P3& s, P3& c, P3 y) {
