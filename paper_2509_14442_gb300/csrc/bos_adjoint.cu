@@ -33,7 +33,6 @@ struct InterpGrad {
     float4 v, d0, d1, d2;   // value and derivatives with respect to the three fractions
 };
 
-__device__ __forceinline__ Cell2 subc(Cell2 a, Cell2 b) { return Cell2{sub2(a.lo, b.lo), sub2(a.hi, b.hi)}; }
 __device__ __forceinline__ float4 to4(Cell2 c) {
     float4 v;
     unpack2(c.lo, v.x, v.y);
@@ -54,8 +53,8 @@ __device__ __forceinline__ InterpGrad trilinear_grad2(const E* s, uint32_t o, fl
     const Cell2 b0 = lerpc(a0, a1, t1), b1 = lerpc(a2, a3, t1);
     InterpGrad r;
     r.v = to4(lerpc(b0, b1, t2));
-    r.d2 = to4(subc(b1, b0));
-    r.d1 = to4(lerpc(subc(a1, a0), subc(a3, a2), t2));
+    r.d2 = to4(csub(b1, b0));
+    r.d1 = to4(lerpc(csub(a1, a0), csub(a3, a2), t2));
     r.d0 = to4(lerpc(lerpc(e0, e1, t1), lerpc(e2, e3, t1), t2));
     return r;
 }
@@ -350,9 +349,7 @@ __device__ __forceinline__ void aim_adjoint(const SceneDev& S, const Ray& RR, do
     for (int a = 0; a < 3; ++a) xlb[a] += (db[a] - dd * RR.d[a]) / nq;
 }
 
-__host__ __device__ constexpr size_t adj_warp_floats(int K) {
-    return (size_t)32 * kRow;   // K is carried by the global segment states
-}
+constexpr size_t kWarpRows = (size_t)32 * kRow;   // shared floats of a warp's lane rows
 
 // Floats per lane and step of the recomputed segment: (dr, dv, A, B) of Sharma's step.
 constexpr int kSegFloats = 12;
@@ -1137,7 +1134,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, FEW ? 1 : CONN ? BOS_REV_CONN_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __shared__ double conn_sh[CONN ? kAdjWarps * 32 * kConnDoubles : 1];   // as in adjoint_kernel
     double* const xlum = conn_sh + (CONN ? (warp * 32 + lane) * kConnDoubles : 0);
-    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * 32 * kRow;
+    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * kWarpRows;
     const CompField<E> F = comp_field<E>(S.g);
     const TileShape ts = tile_shape(S.cam.width, S.cam.height, S.cam.spp);
     const int ntiles = tile_count(S, ts);
@@ -1166,7 +1163,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, BOS_ADJ_MIN_BLOCKS) adjoint_ke
     __shared__ double conn_sh[CONN ? kAdjWarps * 32 * kConnDoubles : 1];
     double* const xlum = conn_sh + (CONN ? (warp * 32 + lane) * kConnDoubles : 0);
     const int K = ck.every;
-    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * adj_warp_floats(K);      // [32][kRow]
+    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * kWarpRows;      // [32][kRow]
     // [K][12][32] step states and stage terms (dr, dv, A, B) of the segment being reversed
     // (this warp's slice)
     float* st_buf = adj.seg + ((size_t)blockIdx.x * kAdjWarps + warp) * ((size_t)K * kSegFloats * 32);
@@ -1282,7 +1279,8 @@ __device__ __forceinline__ void flush_rows_d(double* rows, bool flag, uint32_t& 
 // Warp-collective: add w_c(f) Q to the lane's row (flushed first where the cell changes).
 __device__ __forceinline__ void accumulate_d(double* rows, bool act, const int i[3], const double f[3], const double Q[4],
                                              uint32_t& key, double* acc, const GridDev& g) {
-    const uint32_t cell = (uint32_t)i[0] + (uint32_t)g.n[0] * ((uint32_t)i[1] + (uint32_t)g.n[1] * (uint32_t)i[2]);
+    const uint32_t cell =
+        act ? (uint32_t)i[0] + (uint32_t)g.n[0] * ((uint32_t)i[1] + (uint32_t)g.n[1] * (uint32_t)i[2]) : kNoKey;
     flush_rows_d(rows, act && key != kNoKey && key != cell, key, acc, g);
     if (!act) return;
     key = cell;
@@ -1545,7 +1543,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, BOS_REV_MIN_BLOCKS)
     reverse_batch_kernel(const BatchJob* __restrict__ jobs, int njobs, int total, int* counter) {
     extern __shared__ float4 smem4[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * 32 * kRow;
+    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * kWarpRows;
     for (;;) {
         int g = 0;
         if (lane == 0) g = atomicAdd(counter, 1);
@@ -1572,7 +1570,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, BOS_ADJ_MIN_BLOCKS)
     if (counter[1] == 0) return;
     extern __shared__ float4 smem4[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * 32 * kRow;
+    float* rows = reinterpret_cast<float*>(smem4) + (size_t)warp * kWarpRows;
     float* st_buf = seg_base + ((size_t)blockIdx.x * kAdjWarps + warp) * ((size_t)k_max * kSegFloats * 32);
     {
         float4* row = reinterpret_cast<float4*>(rows + lane * kRow);
@@ -1612,7 +1610,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, BOS_ADJ_MIN_BLOCKS)
 template <class E, bool QUASI>
 static cudaError_t launch_adjoint_batch_c(const BatchJob* jobs, int njobs, int total, int* counter, float* seg_base,
                                           int k_max, int num_sms, cudaStream_t st) {
-    const size_t smem = (size_t)kAdjWarps * 32 * kRow * sizeof(float);
+    const size_t smem = (size_t)kAdjWarps * kWarpRows * sizeof(float);
     int per_sm = 0;
     cudaError_t e = occupancy_prefer_l1(reverse_batch_kernel<E, QUASI>, kAdjWarps * 32, smem, per_sm);
     if (e != cudaSuccess) return e;
@@ -1657,7 +1655,7 @@ cudaError_t launch_gradient(const GridDev& g, const float4* acc, const float* T,
 template <class E, bool CONN, bool QUASI, bool FEW, bool SCATTER>
 static cudaError_t launch_reverse_f(const SceneDev& S, const CkptDev& ck, const AdjDev& adj, const WorkDev& w,
                                     int num_sms, cudaStream_t st) {
-    const size_t smem = SCATTER ? 0 : (size_t)kAdjWarps * 32 * kRow * sizeof(float);
+    const size_t smem = SCATTER ? 0 : (size_t)kAdjWarps * kWarpRows * sizeof(float);
     int per_sm = 0;
     cudaError_t e = occupancy_prefer_l1(reverse_kernel<E, CONN, QUASI, FEW, SCATTER>, kAdjWarps * 32, smem, per_sm);
     if (e != cudaSuccess) return e;
@@ -1684,7 +1682,7 @@ static cudaError_t launch_reverse(const SceneDev& S, const CkptDev& ck, const Ad
 template <class E, bool CONN>
 static cudaError_t launch_adjoint_c(const SceneDev& S, const CkptDev& ck, const AdjDev& adj, const WorkDev& w,
                                     int num_sms, cudaStream_t st) {
-    size_t smem = (size_t)kAdjWarps * adj_warp_floats(ck.every) * sizeof(float);
+    const size_t smem = (size_t)kAdjWarps * kWarpRows * sizeof(float);
     cudaError_t e =
         cudaFuncSetAttribute(adjoint_kernel<E, CONN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -1,5 +1,7 @@
-// Float32 deviation integrator (FP32_COMP / BF16_COMP), shared by the forward and the
-// adjoint kernels so that the adjoint recomputes exactly the forward's arithmetic.
+// Float32 deviation integrator (FP32_COMP / BF16_COMP), shared by the forward and the adjoint
+// kernels.  comp_step is written in plain arithmetic: which products and sums are fused is the
+// compiler's choice in each kernel, so that a segment recomputed by the adjoint agrees with the
+// forward's explicitly rounded steps (stage_run in bos_forward.cu) to rounding, not bit for bit.
 #pragma once
 
 #include "bos_device.cuh"

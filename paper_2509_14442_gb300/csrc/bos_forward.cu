@@ -240,8 +240,6 @@ __global__ void __launch_bounds__(256) build_split_kernel(GridDev g, BuildConst 
         write_elem(store + (size_t)slot * kBrickCells + local, rec, local, local % kBrickSide < kBrickSide - 1);
 }
 
-// ===================================================================== a3: integrators
-
 // ===================================================================== a2-a5: render
 
 struct Sums {
@@ -368,8 +366,8 @@ __device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>&
 }
 
 // Sharma steps of one ray with checkpoints, stage by stage on the 32.32 fixed-point line: the
-// arithmetic whose result seeds a gradient and which adjoint_kernel repeats.  Every operation
-// is explicitly rounded (left to the assembler, a product and a sum are fused or not depending
+// arithmetic whose result seeds a gradient.  (Where adjoint_kernel recomputes a segment it takes
+// comp_step, which agrees with this to rounding.)  Every operation is explicitly rounded (left to the assembler, a product and a sum are fused or not depending
 // on the register budget), in packed pairs where three components do the same.  The next
 // step's first stage needs only the new position, not C, so it is evaluated beside this
 // step's third stage.
@@ -558,8 +556,9 @@ __device__ __forceinline__ void line_run(const CompField<E>& F, const Ray& R, co
     st.excess = __fadd_rn(excess, dot3(d, sub3(dr, cr)));
 }
 
-// Integrate one ray of the comp path (N > 0) from the pinhole rs; optionally store its
-// checkpoints every K steps in `state` (slot `ray`).  Leaves the end state in st.
+// Integrate one ray of the comp path (N > 0) from the pinhole rs stage by stage; Sharma's tracer
+// stores its checkpoints every K steps in `state` (slot `ray`) where that is set (renders of the
+// classical integrator keep none).  Leaves the end state in st.
 template <class E, int INTEG>
 __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& F, const double rs[3], const Ray& R,
                                          const CkptDev& ck, float4* state, long long ray, CompState& st,
@@ -573,16 +572,7 @@ __device__ __forceinline__ void comp_run(const SceneDev& S, const CompField<E>& 
         line_run(F, R, k, st);
     } else {
         BrickCache bc = {0xffffffffu, 0u};
-        const int K = ck.every;
-        for (int n = 0; n < R.N; ++n) {
-            if (state != nullptr && n % K == 0) {
-                const size_t c = bounded((size_t)(n / K), (size_t)ck.max_ckpt, ck.err);
-                state[(c * 3 + 0) * ck.nrays + ray] = make_float4(st.dr[0], st.dr[1], st.dr[2], st.cr[0]);
-                state[(c * 3 + 1) * ck.nrays + ray] = make_float4(st.dv[0], st.dv[1], st.dv[2], st.cr[1]);
-                state[(c * 3 + 2) * ck.nrays + ray] = make_float4(st.cv[0], st.cv[1], st.cv[2], st.cr[2]);
-            }
-            comp_step<E, INTEG>(F, st, k, bc);
-        }
+        for (int n = 0; n < R.N; ++n) comp_step<E, INTEG>(F, st, k, bc);
     }
 }
 
@@ -595,7 +585,7 @@ __device__ __forceinline__ void comp_end(const CompState& st, float dr[3], float
 
 // End deviation, path excess and entry index of a ray: Sharma and the quasi-linear tracer march
 // from cell to cell where nothing is kept for an adjoint; everything else goes stage by stage.
-template <class E, int INTEG, bool CONN, bool SAVE>
+template <class E, int INTEG, bool SAVE>
 __device__ __forceinline__ void trace_end(const SceneDev& S, const CompField<E>& F, const double rs[3], Ray& R,
                                           volatile double* park,
                                           const CkptDev& ck, float4* state, long long ray, float dr[3], float dv[3],
@@ -631,7 +621,7 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, Ray R,
     if (R.N > 0) {
         float dr[3], dv[3], excess;
         float eta_in;
-        trace_end<E, INTEG, CONN, SAVE>(S, F, S.cam.pos, R, ray_park<0>(), ck, ck.state, ray, dr, dv, excess, eta_in, &apart);
+        trace_end<E, INTEG, SAVE>(S, F, S.cam.pos, R, ray_park<0>(), ck, ck.state, ray, dr, dv, excess, eta_in, &apart);
         path = excess;
         steps += (unsigned long long)R.N;
         h = comp_wall(S, R, eta_in, dr, dv, excess);
@@ -654,7 +644,7 @@ __device__ RayResult trace_comp(const SceneDev& S, const CompField<E>& F, Ray R,
                 if (Rp.wall && Rp.N > 0) {
                     float eta_p;
                     float pr[3], pv[3], pexcess, papart = 0.0f;
-                    trace_end<E, INTEG, CONN, SAVE>(S, F, P, Rp, ray_park<1>(), ck, m == 0 ? ck.pstate : nullptr, ray, pr, pv, pexcess,
+                    trace_end<E, INTEG, SAVE>(S, F, P, Rp, ray_park<1>(), ck, m == 0 ? ck.pstate : nullptr, ray, pr, pv, pexcess,
                                                     eta_p, &papart);
                     apart = max_nan(apart, papart);
                     steps += (unsigned long long)Rp.N;

@@ -1,7 +1,8 @@
 // Full-state integration in absolute coordinates, T = float (plain FP32 tracer) or
 // double (FP64 tracer and its adjoint): the field at a point and one Sharma RKN or classic
 // RK4 step of dr/dt = v, dv/dt = eta grad eta (Sec. 2.2, Eq. 1).  Shared by the forward
-// and the adjoint so that the adjoint recomputes exactly the forward's arithmetic.
+// and the adjoint, which recomputes the forward's steps with it (to rounding: what is fused is the
+// compiler's choice in each kernel).
 #pragma once
 
 #include "bos_comp.cuh"
