@@ -480,9 +480,12 @@ __device__ __forceinline__ void rows_out(float* rows, bool flag, uint32_t key, C
 // Whether a launch's lanes are sparse enough for that: per cell of the grid's smallest cross
 // section at most 12, with the refracted connection (whose two rays visit other cells) at most
 // 24.  Whole steps at n lanes per cell, rows_flush -> rows_scatter: 200x200x150 cells, n = 0.7: 1306 ->
-// 1075 us; 64x64x48 cells, n = 7: 357 -> 335; a 64^3 minibatch, n = 2.4: 437 -> 390; 128x128x96 cells with
-// the connection, n = 21: 6.37 -> 5.70 ms; even at n = 12; 200x200x150 cells, n = 19: 9.6 -> 10.0 ms, 40: 19.0 ->
-// 20.7 ms; 24x24x18 cells, n = 83: 204 -> 260 us.
+// 1075 us; 64x64x48 cells, n = 7: 357 -> 335; a 64^3 minibatch, n = 2.4: 437 -> 390; even at n = 12;
+// 200x200x150 cells, n = 19: 9.6 -> 10.0 ms, 40: 19.0 -> 20.7 ms; 24x24x18 cells, n = 83: 204 -> 260 us.
+// With the connection the line lies where the first grid turns: 32x32x24 cells, n = 20: 446 -> 432 us,
+// 24: 444 -> 439, 28: 444 -> 445, 36: 443 -> 453, 120: 960 -> 1026.  24x24x18 turns at 34 (24: 384 -> 375 us; 80: 380
+// -> 428); finer grids would gain beyond it, 64x64x48 at n = 28: 1478 -> 1368 us, 80: 3448 -> 3350,
+// 128x128x96 at 22: 6.48 -> 5.81 ms, 45: 12.4 -> 11.4 ms.
 __host__ __device__ __forceinline__ bool sparse_lanes(const SceneDev& S, const TileShape& ts, bool conn) {
     const long long nx = S.g.n[0], ny = S.g.n[1], nz = S.g.n[2];
     const long long longest = nx > ny ? (nx > nz ? nx : nz) : (ny > nz ? ny : nz);

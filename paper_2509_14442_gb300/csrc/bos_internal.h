@@ -50,12 +50,16 @@ struct RenderOut {
 };
 
 // Warp tiles per SM up to which a launch takes a tracer's form without a register cap: what
-// such a form (180 to 240 registers) keeps resident.
+// such a form (180 to 240 registers) keeps resident.  96x96x72 cells at t tiles per SM, capped ->
+// uncapped: frame t = 6: 227 -> 163 us, 8: 231 -> 236, 9: 232 -> 252, 12: 238 -> 261; step t = 6: 776 -> 451, 8: 784 ->
+// 688, 10: 790 -> 708, 12: 802 -> 783, 14: 809 -> 813 (48x48x36 cells turn at the same places): a step's
+// adjoint would gain up to 12, a frame loses from 8 on.
 constexpr int kFewTiles = 8;
 
 // Threads per block of a float64 tracer's launch.  Its few tiles are bound by the SMs' float64
 // pipes, and blocks of several warps give some SMs twice the tiles of others: a step of 864 tiles
-// (64x64x48 cells, 192 x 144 rays) took 10.61 ms so, 9.70 ms in blocks of one warp.  (The float32
+// (64x64x48 cells, 192 x 144 rays) took 10.61 ms so, 9.70 ms in blocks of one warp; 32x32x24 cells at
+// 8 tiles per SM 7.26 -> 6.73 ms, at 9: 7.43 -> 7.43.  (The float32
 // tracers gain nothing: an SM's four schedulers do not share what bounds them.)
 inline int fp64_threads(int tiles, int num_sms, int block) { return tiles <= num_sms * kFewTiles ? 32 : block; }
 
