@@ -775,13 +775,17 @@ __device__ __forceinline__ RayResult trace_ray(const SceneDev& S, const Ray& R, 
 #ifndef BOS_FWD_LINE_MIN_BLOCKS
 #define BOS_FWD_LINE_MIN_BLOCKS 4         // quasi-linear tracing whose end state is kept
 #endif
+#ifndef BOS_FWD_RK4_MIN_BLOCKS
+#define BOS_FWD_RK4_MIN_BLOCKS 5          // classical steps on the paired stores (96x96x72 cells, 512^2: 6: 1190 us, 5: 995, 4: 1047)
+#endif
 #ifndef BOS_FWD_FP64_MIN_BLOCKS
 #define BOS_FWD_FP64_MIN_BLOCKS 3         // float64: its pipe is full with a few warps, the cell's polynomial is 64 registers
 #endif
 constexpr int render_min_blocks(int mode, int integ, bool conn, bool save) {
     return mode == 4 ? BOS_FWD_FP64_MIN_BLOCKS
            : integ == 2 ? (save ? BOS_FWD_LINE_MIN_BLOCKS : BOS_FWD_QUASI_MIN_BLOCKS)
-           : (mode != 1 && mode != 2) || integ != 0 ? BOS_FWD_MIN_BLOCKS
+           : mode != 1 && mode != 2 ? BOS_FWD_MIN_BLOCKS
+           : integ == 1 ? BOS_FWD_RK4_MIN_BLOCKS
            : save ? (conn ? BOS_FWD_STAGE_CONN_MIN_BLOCKS : BOS_FWD_STAGE_MIN_BLOCKS) : BOS_FWD_MARCH_MIN_BLOCKS;
 }
 // One warp tile of a render: the rays of its (up to) 32 lanes, averaged per pixel, written
