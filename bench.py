@@ -81,7 +81,12 @@ WORKLOADS = {
                                  make=lambda seed: quasi(S.room((256, 256, 192), 512, 512, 1, seed)), adjoint=True,
                                  fwd_bytes=256, adj_bytes=512),
 }
-# Algorithmic bytes of one Sharma ray-step of the forward tracer: 3 field evaluations x 8
+# ---- Two counts of the work of a ray-step.  Stage by stage: what the method's formulas take when
+# every stage gathers its corners and the adjoint recomputes its segments; printed beside each
+# kernel ("stage_by_stage"), so that lines compare over time, and never divided by a peak.  Done:
+# what the kernels do (*_DONE, CELL_BYTES below), which the fractions of the peaks are made of.
+#
+# Stage by stage, bytes of one Sharma ray-step of the forward tracer: 3 field evaluations x 8
 # trilinear corners x one (deta, grad eta) record (16 B in float32).
 BYTES_PER_STEP = {"fp32_comp": 384, "fp32": 384, "bf16_comp": 192, "fp64": 768}
 # Adjoint, per ray-step: the segment recompute gathers 384 B, the reverse step gathers the
@@ -94,7 +99,7 @@ ADJ_BYTES_PER_STEP = {"fp32_comp": 3 * 384, "bf16_comp": 2 * 192 + 384}
 L1_BYTES_PER_STEP = {"fp32_comp": 384, "fp32": 384, "bf16_comp": 192, "fp64": 768}
 ADJ_L1_BYTES_PER_STEP = {"fp32_comp": 2 * 384, "bf16_comp": 2 * 192}
 L2_BYTES = 129 * 2 ** 20
-# Algorithmic floating-point operations of one ray-step (an FMA counts 2), counted from the
+# Stage by stage, floating-point operations of one ray-step (an FMA counts 2), counted from the
 # method's formulas, not from the kernels (which add the compensation of the fixed-point
 # straight line, bounds tests and index arithmetic):
 #   field evaluation D(r) = (1 + deta) grad eta at a point: 3 fractions (sub, mul) = 6,
@@ -108,12 +113,44 @@ L2_BYTES = 129 * 2 ** 20
 #     evaluations 3 x (6 + 4 x 36) = 450, the adjoint of D per stage 3 x 36 = 108, the
 #     transpose of the step's linear combinations 66, the path-length adjoint 11, and the
 #     corner scatter per stage (3 complements, 8 weights x 2, 8 x 4 FMAs) 3 x 83 = 249:  1240
-#     (reverse_kernel makes no recompute and two of the three stages' evaluations and scatters;
-#     the count stays that of the stage-by-stage adjoint, so that rates compare over time)
 #   one-sweep quasi-linear adjoint: per line sample the point, fractions and value 96, the
 #     adjoint of D 9 and the corner scatter 83 (2 samples: 376), the velocity adjoint 24:  400
 FLOPS_PER_STEP = {"rkn": 356, "quasi": 241}
 ADJ_FLOPS_PER_STEP = {"rkn": 1240, "quasi": 400}
+# Done, by the same counts: a Sharma step's last point and the next step's first one are one
+# evaluation (2 of 3: 356 - 94); reversing it takes 2 value-and-derivative evaluations 300, 3
+# position adjoints 108, the transposes 66, the path length 11 and 2 scatters 166, no recompute.
+FLOPS_DONE = {"rkn": 262, "quasi": 241}
+ADJ_FLOPS_DONE = {"rkn": 651, "quasi": 400}
+# Done, bytes: a ray gathers a cell's 4 paired records when it enters the cell (32 B each, bfloat16
+# 16 B); its adjoint also adds the cell's 8 corners of 16 B to the node accumulators.  The stores
+# without such a ray cache gather as counted stage by stage.
+CELL_BYTES = {"fp32_comp": 128, "bf16_comp": 64}
+CELL_SCATTER_BYTES = 128
+
+
+def cells_per_ray_step(scene) -> float:
+    """Cells that the straight pixel-centre rays visit per step (4096 pixels or so)."""
+    c, g = scene.camera, scene.grid
+    pix = np.arange(0, c.width * c.height, max(1, c.width * c.height // 4096))
+    fwd, up, pos = (np.array(v, dtype=np.float64) for v in (c.fwd, c.up, c.pos))
+    a, b = (pix % c.width + 0.5 - c.cx) / c.fx, (pix // c.width + 0.5 - c.cy) / c.fy
+    d = a[:, None] * np.cross(fwd, up) - b[:, None] * up + fwd
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    o, e, n = np.array(g.origin), np.array(g.extent), np.array(g.n)
+    with np.errstate(divide="ignore", invalid="ignore"):
+        t0, t1 = (o - pos) / d, (o + e - pos) / d
+        tw = ((np.array(scene.wall.origin) - pos) @ np.array(scene.wall.normal)) / (d @ np.array(scene.wall.normal))
+    t_in = np.maximum(np.nanmax(np.minimum(t0, t1), axis=1), 0.0)
+    t_out = np.minimum(np.nanmin(np.maximum(t0, t1), axis=1), tw)
+    hit = t_out > t_in
+    ends = [np.clip(np.floor((pos + t[:, None] * d - o) * n / e - 0.5), 0, n - 2)[hit] for t in (t_in, t_out)]
+    cells = 1 + np.abs(ends[1] - ends[0]).sum(axis=1)
+    step = scene.integ.max_step_vox * (e / n).min()
+    N = scene.integ.fixed_steps or np.ceil((t_out - t_in)[hit] / step)
+    return float(cells.sum() / (N * np.ones(cells.shape)).sum())
+
+
 # The arithmetic peak: 152 SMs x 128 float32 FMA lanes x 2 flops x the SM clock (derived
 # from the unit counts; the in-run probe measures it as well).  Float64: GB300's nominal
 # 1.25 TFLOP/s at 2070 MHz.
@@ -127,7 +164,8 @@ FP64_NOMINAL_FLOPS = 1.25e12
 # timed launch (`algorithmic_hbm`): the per-grid part (the field store, the accumulators)
 # is the same at both sizes.  Reported only while the kernel sources still hash to the
 # captured ones.
-TRAFFIC_SOURCES = ("bos_forward.cu", "bos_adjoint.cu", "bos_comp.cuh", "bos_device.cuh", "bos_full.cuh")
+TRAFFIC_SOURCES = ("bos_forward.cu", "bos_adjoint.cu", "bos_comp.cuh", "bos_device.cuh", "bos_full.cuh",
+                   "bos_march.cuh")
 TRAFFIC_CAPTURE = {"workload": "room_adj_small", "sha256": "7fac1ee6e2e1104ea8741aca7bf56e4f7191c9d44ffaa67a74c5589f51ee5e94",
                    "render_kernel": 409746176 + 430900736, "adjoint_kernel": 952656896 + 245624320,
                    # per-ray algorithmic bytes of the captured launches (512^2 rays, 8,650,752 checkpoints)
@@ -517,7 +555,9 @@ def frame_bench(args, wl_name: str, ctxs: dict, rank: int = 0, world: int = 1, d
             bos.check(L.bos_backward(ctx.h, dLdI.data_ptr(), dLdT.data_ptr(), sp), "backward")
             if ev is not None:
                 ev[3].record(stream)
-            launches["n"] = 5          # build_store, render, loss_l2, adjoint, gradient
+            # build_store, render, loss_l2, reverse (float64: adjoint), gradient; and for compensated
+            # Sharma rays the adjoint of the tiles that reverse left
+            launches["n"] = 6 if scene.integ.integrator == 0 and args.prec in CELL_BYTES else 5
         else:
             bos.check(L.bos_render_reference(ctx.h, Iref.data_ptr(), None, None, sp), "render_ref")
             launches["n"] = 3          # build_store, render, render (reference)
@@ -616,17 +656,26 @@ def alu_peak_of(prec: str, P: dict):
 
 def kernel_entries(res, prec: str, P: dict) -> dict:
     """Roofline figures of the render and (adjoint workloads) the backward of one frame
-    benchmark: arithmetic (algorithmic flops per ray-step), L1 and L2 gathered bytes."""
+    benchmark: arithmetic, L1 and L2 bytes of what the kernels do per ray-step, and beside them
+    the stage-by-stage counts."""
     wl, scene, spf = res["wl"], res["scene"], res["steps_per_frame"]
     alu_peak, _ = alu_peak_of(prec, P)
     integ = {0: "rkn", 2: "quasi"}.get(scene.integ.integrator)
-    fwd_b = wl.get("fwd_bytes", BYTES_PER_STEP[prec])
-    adj_b = wl.get("adj_bytes", ADJ_BYTES_PER_STEP.get(prec, 0))
-    fwd_l1 = wl.get("fwd_bytes", L1_BYTES_PER_STEP[prec])
-    adj_l1 = wl.get("fwd_bytes", ADJ_L1_BYTES_PER_STEP.get(prec, 0))
+    stages = {"render_kernel": {"flops": FLOPS_PER_STEP.get(integ), "bytes": wl.get("fwd_bytes", BYTES_PER_STEP[prec]),
+                                "l1_bytes": wl.get("fwd_bytes", L1_BYTES_PER_STEP[prec])},
+              "adjoint_kernel": {"flops": ADJ_FLOPS_PER_STEP.get(integ),
+                                 "bytes": wl.get("adj_bytes", ADJ_BYTES_PER_STEP.get(prec, 0)),
+                                 "l1_bytes": wl.get("fwd_bytes", ADJ_L1_BYTES_PER_STEP.get(prec, 0))}}
+    done = {k: dict(v) for k, v in stages.items()}
+    if prec in CELL_BYTES:
+        gathered = CELL_BYTES[prec] * cells_per_ray_step(scene)
+        scattered = CELL_SCATTER_BYTES * cells_per_ray_step(scene)
+        done = {"render_kernel": {"flops": FLOPS_DONE.get(integ), "bytes": gathered, "l1_bytes": gathered},
+                "adjoint_kernel": {"flops": ADJ_FLOPS_DONE.get(integ), "bytes": gathered + scattered, "l1_bytes": gathered}}
     alg = algorithmic_hbm(scene, res["ckpt_slots"], res["store_bytes"]) if wl["adjoint"] else None
 
-    def entry(ms, flops_per_step, bytes_per_step, l1_bytes_per_step, name):
+    def entry(ms, name):
+        flops_per_step, bytes_per_step, l1_bytes_per_step = (done[name][k] for k in ("flops", "bytes", "l1_bytes"))
         tflops = flops_per_step * spf / (ms * 1e-3) / 1e12 if flops_per_step else None
         gbs = bytes_per_step * spf / (ms * 1e-3) / 1e9
         l1_gbs = l1_bytes_per_step * spf / (ms * 1e-3) / 1e9
@@ -634,18 +683,15 @@ def kernel_entries(res, prec: str, P: dict) -> dict:
                 "frac": tflops / alu_peak if tflops is not None else None,
                 "bytes_per_ray_step": bytes_per_step, "achieved_gbs": gbs, "l2_frac": gbs / P["l2"],
                 "l1_bytes_per_ray_step": l1_bytes_per_step, "l1_achieved_gbs": l1_gbs, "l1_frac": l1_gbs / P["l1"],
+                "stage_by_stage": {k + "_per_ray_step": v for k, v in stages[name].items()},
                 "algorithmic_hbm_bytes": alg[name]["total"] if alg else None,
                 "traffic": kernel_traffic(name, alg) if alg else None}
 
-    k = {"render_kernel": entry(statistics.mean(res["render_ms"]), FLOPS_PER_STEP.get(integ), fwd_b, fwd_l1,
-                                "render_kernel")}
-    if prec == "fp32_comp" and integ == "rkn" and scene.light.mode != 2:
-        k["render_kernel"]["l1_note"] = ("algorithmic gathered bytes: the tracer keeps each ray's last cell in "
-                                         "registers, so most stages load nothing through L1")
+    k = {"render_kernel": entry(statistics.mean(res["render_ms"]), "render_kernel")}
     if wl["adjoint"]:
-        k["adjoint_kernel"] = entry(statistics.mean(res["back_ms"]), ADJ_FLOPS_PER_STEP.get(integ), adj_b, adj_l1,
-                                    "adjoint_kernel")
-        k["adjoint_kernel"]["timed"] = "bos_backward: accumulator clear + adjoint_kernel + gradient_kernel"
+        k["adjoint_kernel"] = entry(statistics.mean(res["back_ms"]), "adjoint_kernel")
+        k["adjoint_kernel"]["timed"] = ("bos_backward: accumulator clear + reverse_kernel + (Sharma) adjoint_kernel for "
+                                        "the tiles it leaves + gradient_kernel")
     return k
 
 
@@ -715,20 +761,21 @@ def gpu_arm(args):
                 "unit": "TFLOP/s", "frac": dk["frac"], "traffic": traffic, "peak_source": alu_src,
                 "flops_per_ray_step": dk["flops_per_ray_step"],
                 "fma_probe_tflops": P["fma"],
-                "note": ("algorithmic flops per ray-step counted from the method's formulas; the gathers are "
+                "note": ("flops per ray-step that the kernels do, counted from the method's formulas "
+                         "(stage_by_stage: with every stage evaluated and every segment recomputed); the gathers are "
                          "served on chip and DRAM carries only the store, checkpoints and outputs, so the "
                          "arithmetic roof is the one that applies"),
                 "kernels": kernels,
                 "l2": {"achieved": dk["achieved_gbs"], "peak": P["l2"], "unit": "GB/s", "frac": dk["l2_frac"],
                        "bytes_per_ray_step": dk["bytes_per_ray_step"],
                        "peak_source": "in-run L2 read probe (bos_probe_read, 24 MiB x 50 passes, best of 10)",
-                       "note": ("gather roofline R = L2 read bandwidth / algorithmic gathered bytes per ray-step; "
-                                "the gathers hit L1, so a kernel can exceed R")},
+                       "note": "records gathered (and corners added) per cell that a ray visits, over the L2 read "
+                               "bandwidth; most of the gathers hit L1"},
                 "l1": {"achieved": dk["l1_achieved_gbs"], "peak": P["l1"], "unit": "GB/s", "frac": dk["l1_frac"],
                        "bytes_per_ray_step": dk["l1_bytes_per_ray_step"],
                        "peak_source": "in-run L1 read probe (bos_probe_read_l1, 256-bit loads, 64 KiB x 200 passes "
                                       "per block, best of 10)",
-                       "note": "the gathers' algorithmic bytes per ray-step over the L1 read bandwidth"},
+                       "note": "records gathered per cell that a ray visits, over the L1 read bandwidth"},
                 "hbm_peak_gbs": P["file"].get("hbm_gbs")}
     if P["file"].get("hbm_gbs"):
         # the same kernel against the HBM roofline: DRAM bytes per launch (measured on the
@@ -1011,7 +1058,7 @@ def precision_record(args, ctxs, P, scene, orc) -> dict:
         ctx.status()
         steps = ctx.last_ray_steps()
         rate = steps / (statistics.mean(ms) * 1e-3)
-        tflops = rate * FLOPS_PER_STEP["rkn"] / 1e12
+        tflops = rate * (FLOPS_DONE if name in CELL_BYTES else FLOPS_PER_STEP)["rkn"] / 1e12
         peak = fp64_peak if name == "fp64" else fp32_peak
         r = {"render_ms": statistics.mean(ms), "ray_steps_per_s": rate,
              "alu": {"achieved_tflops": tflops, "peak_tflops": peak, "frac": tflops / peak,
