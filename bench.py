@@ -166,10 +166,11 @@ FP64_NOMINAL_FLOPS = 1.25e12
 # captured ones.
 TRAFFIC_SOURCES = ("bos_forward.cu", "bos_adjoint.cu", "bos_comp.cuh", "bos_device.cuh", "bos_full.cuh",
                    "bos_march.cuh")
-TRAFFIC_CAPTURE = {"workload": "room_adj_small", "sha256": "7fac1ee6e2e1104ea8741aca7bf56e4f7191c9d44ffaa67a74c5589f51ee5e94",
-                   "render_kernel": 409746176 + 430900736, "adjoint_kernel": 952656896 + 245624320,
-                   # per-ray algorithmic bytes of the captured launches (512^2 rays, 8,650,752 checkpoints)
-                   "rays": {"render_kernel": 417333248, "adjoint_kernel": 417333248}}
+TRAFFIC_CAPTURE = {"workload": "room_adj_small", "sha256": "59f43e6ab98cb180ad035889f890bc97e6ff714fa6e0cbb7a06c0908436e642c",
+                   "render_kernel": 385508352 + 395865088, "reverse_kernel": 530590464 + 172305152,
+                   # per-ray algorithmic bytes of the captured launches (512^2 rays, 8,650,752 checkpoints);
+                   # adjoint_kernel: were it to reverse every tile (it runs on what reverse_kernel leaves)
+                   "rays": {"render_kernel": 417333248, "reverse_kernel": 14680064, "adjoint_kernel": 417333248}}
 
 
 def kernel_sources_sha256() -> str:
@@ -188,10 +189,13 @@ def algorithmic_hbm(scene, ckpt_slots: int, store_bytes: int) -> dict:
     rays of ceil(N/K) checkpoints of 48 B, 4 B of path-length record per ray, the render's
     4 B image or the adjoint's 4 B of dL/dI per pixel) and the part fixed by the grid
     ("grid": the field store read once; for the adjoint also its float4 node accumulators,
-    read and written by the atomics, 32 B per cell).  "total" = their sum."""
+    read and written by the atomics, 32 B per cell).  "total" = their sum.  reverse_kernel: the
+    adjoint that reads one end state per ray (48 B, quasi-linear 32 B) in place of the checkpoints."""
     rays = ckpt_slots * 48 + scene.rays * 4 + scene.pixels * 4
-    grid = {"render_kernel": store_bytes, "adjoint_kernel": store_bytes + scene.grid.cells * 32}
-    return {k: {"rays": rays, "grid": g, "total": rays + g} for k, g in grid.items()}
+    ends = scene.rays * (52 if scene.integ.integrator == 0 else 32) + scene.pixels * 4
+    adjoint = store_bytes + scene.grid.cells * 32
+    parts = {"render_kernel": (rays, store_bytes), "adjoint_kernel": (rays, adjoint), "reverse_kernel": (ends, adjoint)}
+    return {k: {"rays": r, "grid": g, "total": r + g} for k, (r, g) in parts.items()}
 
 
 def kernel_traffic(name: str, alg: dict):
@@ -674,7 +678,10 @@ def kernel_entries(res, prec: str, P: dict) -> dict:
                 "adjoint_kernel": {"flops": ADJ_FLOPS_DONE.get(integ), "bytes": gathered + scattered, "l1_bytes": gathered}}
     alg = algorithmic_hbm(scene, res["ckpt_slots"], res["store_bytes"]) if wl["adjoint"] else None
 
+    captured = prec == "fp32_comp" and integ == "rkn" and scene.light.mode != 2   # the kernels of the capture
+
     def entry(ms, name):
+        launch = "reverse_kernel" if name == "adjoint_kernel" and prec in CELL_BYTES else name
         flops_per_step, bytes_per_step, l1_bytes_per_step = (done[name][k] for k in ("flops", "bytes", "l1_bytes"))
         tflops = flops_per_step * spf / (ms * 1e-3) / 1e12 if flops_per_step else None
         gbs = bytes_per_step * spf / (ms * 1e-3) / 1e9
@@ -684,8 +691,8 @@ def kernel_entries(res, prec: str, P: dict) -> dict:
                 "bytes_per_ray_step": bytes_per_step, "achieved_gbs": gbs, "l2_frac": gbs / P["l2"],
                 "l1_bytes_per_ray_step": l1_bytes_per_step, "l1_achieved_gbs": l1_gbs, "l1_frac": l1_gbs / P["l1"],
                 "stage_by_stage": {k + "_per_ray_step": v for k, v in stages[name].items()},
-                "algorithmic_hbm_bytes": alg[name]["total"] if alg else None,
-                "traffic": kernel_traffic(name, alg) if alg else None}
+                "algorithmic_hbm_bytes": alg[launch]["total"] if alg else None,
+                "traffic": kernel_traffic(launch, alg) if alg and captured else None}
 
     k = {"render_kernel": entry(statistics.mean(res["render_ms"]), "render_kernel")}
     if wl["adjoint"]:

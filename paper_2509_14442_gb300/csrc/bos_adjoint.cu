@@ -1120,10 +1120,10 @@ __device__ __forceinline__ void adjoint_tile(const SceneDev& S, const CkptDev& c
 #ifndef BOS_REV_CONN_MIN_BLOCKS
 #define BOS_REV_CONN_MIN_BLOCKS 6         // the same with the refracted connection
 #endif
-// What bounds it: instruction issue and dependent arithmetic (54 % of the issue slots and half of
-// the float32 FMA pipe at 12 to 16 warps per SM), ~550 warp instructions per step of a tile, a
-// quarter of them in the row flushes; memory is at 32 % (L1) and 1 % (DRAM).  256x256x192 cells,
-// 2048^2 rays: 49.6 ms, where recomputing the segments took 128.4 ms; 192x192x144 cells in
+// What bounds it: instruction issue and dependent arithmetic (45 to 58 % of the issue slots, FMA
+// instructions 28 % of their pipe's, at 12 to 16 warps per SM), ~500 warp instructions per step of a
+// tile, a quarter of them in the row flushes; memory is at 44 to 61 % (L1) and 1 to 3 % (DRAM).
+// 256x256x192 cells, 2048^2 rays: 48.8 ms, where recomputing the segments took 128.4 ms; 192x192x144 cells in
 // bfloat16 at 768^2: 6.0 ms, 18.6 ms; with the refracted connection, 128x128x96 cells at 512^2:
 // 4.3 ms, 11.2 ms.  Against the float64 oracle the gradients are 10 to 35 % nearer than with the
 // recompute (relative L2 2e-7 .. 7e-7).  128 registers and 16 warps beat 168 and 12 by 2 to 3 %;

@@ -376,11 +376,12 @@ __device__ __forceinline__ void march_run(const SceneDev& S, const CompField<E>&
 // position is in the same cell and whose fractions are in [0, 1) takes the records as they
 // are, without an address.
 //
-// What bounds it: instruction issue (58 %) and the FMA pipe (48 %) at 16 warps per SM.  256x256x192
-// cells, 2048^2 rays with checkpoints: 28.7 ms with an address per point and scalar updates,
-// 21.8 ms so (27.1 ms with the address kept and explicit rounding only, 25.6 without the
-// address, 23.9 with the equal-fractions test, 21.8 with the ray parked); 96 registers and 20
-// warps 24.1 ms, 168 and 12 23.3 ms.  Same bits.  With the refracted connection 168 registers are
+// What bounds it: instruction issue (57 % of the slots, FMA instructions 33 % of their pipe's) at 16
+// warps per SM.  256x256x192 cells, 2048^2 rays with checkpoints: 28.7 ms with an address per point
+// and scalar updates, 22.5 ms so (27.1 ms with the address kept and explicit rounding only, 25.6
+// without the address, 23.9 with the equal-fractions test, 21.9 with the ray parked, 22.5 with the
+// bound on A - C); before that bound 96 registers and 20 warps 24.1 ms, 168 and 12 23.3 ms.  Same
+// bits.  With the refracted connection 168 registers are
 // best (1.79 ms; 128: 2.08; 96: 2.85; before: 2.11, 128x128x96 cells at 512^2).
 struct StageCell {
     int c[3];
@@ -513,8 +514,8 @@ __device__ __forceinline__ void stage_run(const CompField<E>& F, const Ray& R, c
 // Stage by stage on the fixed-point line like stage_run, and explicitly rounded for the same
 // reason: the luminance is read at a float32 texel coordinate, so an end state an ulp away moves
 // the pixels beside one of its steps by 1e-5 of the image, and a residual of one per cent, which
-// seeds the gradient, by a few per mille.  Render and adjoint of 256x256x192 cells at 1024 x 768
-// rays: 14.2 ms with an address and four gathers per pair of steps, 13.3 ms so (12.8 ms marched;
+// seeds the gradient, by a few per mille.  What bounds it: instruction issue (60 % of the slots, FMA
+// 36 %, L1 24 %) at 16 warps per SM.  Render and adjoint of 256x256x192 cells at 1024 x 768 rays: 14.2 ms with an address and four gathers per pair of steps, 13.3 ms so (12.8 ms marched;
 // 168 registers 13.7 ms, 96 13.3 ms).
 template <class E>
 __device__ __forceinline__ void line_run(const CompField<E>& F, const Ray& R, const CompConst& k, CompState& st) {

@@ -8,8 +8,8 @@
 //     packed FMAs and no load;
 //   - its line split into float32 parts relative to that cell, so a point's fraction is three
 //     operations per axis and needs no integer arithmetic or conversions.
-// What bounds it: instruction issue (63 % of the slots) and the float32 FMA pipe (57 %).  A
-// point inside its cell takes ~35 instructions where gathering each stage through the 64-bit
+// What bounds it: instruction issue (63 % of the slots; float32 FMA instructions, most of them
+// packed, fill 39 % of their pipe's, L1 is at 20 %) with 16 warps per SM.  A point inside its cell takes ~35 instructions where gathering each stage through the 64-bit
 // line position, the brick address and seven packed lerps took ~90; the rest is cell changes
 // (~80 each, and rays of a warp that cross an x or z face one after the other each pay theirs).
 // Flow render of 128x128x96 cells, 1024^2 x 4 rays: 13.71 ms stage by stage, 10.45 ms so; of
