@@ -1469,34 +1469,40 @@ __global__ void __launch_bounds__(kAdjWarps * 32) adjoint_fp64_kernel(SceneDev S
     }
 }
 
-// dL/dT per node: transpose of the difference stencil of grad eta, plus d L/d deta, times
-// d deta/dT = -K / T^2.  Float64 accumulators (A = double) are summed in float64.
-template <class O>
-__global__ void gradient_fp64_kernel(GridDev g, const double* __restrict__ acc, const float* __restrict__ T,
-                                     O* __restrict__ dLdT) {
-    const uint32_t n = (uint32_t)g.n[0] * g.n[1] * g.n[2], c = blockIdx.x * 256u + threadIdx.x;
-    if (c >= n) return;
+// Transpose of the difference stencil of grad eta at node c, plus d L/d deta, in float64.
+template <class A>
+__device__ __forceinline__ double stencil_fp64(const GridDev& g, const A* __restrict__ acc, uint32_t c) {
     const uint32_t stride[3] = {1u, (uint32_t)g.n[0], (uint32_t)g.n[0] * (uint32_t)g.n[1]};
     const int idx[3] = {(int)(c % stride[1]), (int)(c / stride[1] % (uint32_t)g.n[1]), (int)(c / stride[2])};
     double tot = acc[(size_t)c * 4];
     for (int a = 0; a < 3; ++a) {
         const int i = idx[a], na = g.n[a];
         const double ih = g.inv_h[a], ih2 = 0.5 * g.inv_h[a];
-        const double* p = acc + 1 + a;
+        const A* p = acc + 1 + a;
         if (i - 1 >= 0) tot += p[(size_t)(c - stride[a]) * 4] * (i - 1 == 0 ? ih : ih2);        // node i-1 reads i as hi
         if (i + 1 <= na - 1) tot -= p[(size_t)(c + stride[a]) * 4] * (i + 1 == na - 1 ? ih : ih2);  // node i+1 reads i as lo
         if (i == 0) tot -= p[(size_t)c * 4] * ih;                                               // one-sided at the faces
         if (i == na - 1) tot += p[(size_t)c * 4] * ih;
     }
+    return tot;
+}
+
+// dL/dT per node: that times d deta/dT = -K / T^2 (float64 accumulators).
+template <class O>
+__global__ void gradient_fp64_kernel(GridDev g, const double* __restrict__ acc, const float* __restrict__ T,
+                                     O* __restrict__ dLdT) {
+    const uint32_t n = (uint32_t)g.n[0] * g.n[1] * g.n[2], c = blockIdx.x * 256u + threadIdx.x;
+    if (c >= n) return;
     const double Tc = (double)T[c];
-    dLdT[c] = (O)(tot * (-g.K / (Tc * Tc)));
+    dLdT[c] = (O)(stencil_fp64(g, acc, c) * (-g.K / (Tc * Tc)));
 }
 
 // The same for float32 accumulators.  The sum is carried in two float32 terms (products and
 // sums with their rounding errors, Knuth's two-sum), which keeps ~2^-46 of its largest term:
 // the float64 sum it replaces held the 12.6 M cells of a 256x256x192 grid for 611 us on the
 // float64 pipe and in 64-bit index divisions; this takes 121 us, against 45 us to read the
-// accumulators and T and write dL/dT (five rows of accumulators pass through L2 per row).
+// accumulators and T and write dL/dT (five rows of accumulators pass through L2 per row).  Where a
+// product or the sum leaves float32's range the rounding errors are NaN: there the sum is float64's.
 struct GradConst {
     float hi[3][2], lo[3][2];   // 1 / (2 h), 1 / h in two terms
     float K;
@@ -1534,8 +1540,10 @@ __global__ void __launch_bounds__(256) gradient_kernel(GridDev g, GradConst k, c
         if (i == 0u) add_term(s, e, -p[0], k.hi[a][1], k.lo[a][1]);      // one-sided at the faces
         if (i == last) add_term(s, e, p[0], k.hi[a][1], k.lo[a][1]);
     }
+    s = __fadd_rn(s, e);
+    if (!(fabsf(s) <= 3.4028235e38f)) s = (float)stencil_fp64(g, reinterpret_cast<const float*>(acc4), c);
     const float Tc = T[c];
-    dLdT[c] = __fadd_rn(s, e) * (-k.K / (Tc * Tc));
+    dLdT[c] = s * (-k.K / (Tc * Tc));
 }
 
 // Batched adjoints (the request server): one launch covers warp tiles of several jobs,
