@@ -166,8 +166,8 @@ FP64_NOMINAL_FLOPS = 1.25e12
 # captured ones.
 TRAFFIC_SOURCES = ("bos_forward.cu", "bos_adjoint.cu", "bos_comp.cuh", "bos_device.cuh", "bos_full.cuh",
                    "bos_march.cuh")
-TRAFFIC_CAPTURE = {"workload": "room_adj_small", "sha256": "59f43e6ab98cb180ad035889f890bc97e6ff714fa6e0cbb7a06c0908436e642c",
-                   "render_kernel": 385508352 + 395865088, "reverse_kernel": 530590464 + 172305152,
+TRAFFIC_CAPTURE = {"workload": "room_adj_small", "sha256": "3776a23d0753c1d1fda77401b38bfef5370f9d4715b9a558dd317c1a9e06e30d",
+                   "render_kernel": 385297664 + 395929600, "reverse_kernel": 530538240 + 171971840,
                    # per-ray algorithmic bytes of the captured launches (512^2 rays, 8,650,752 checkpoints);
                    # adjoint_kernel: were it to reverse every tile (it runs on what reverse_kernel leaves)
                    "rays": {"render_kernel": 417333248, "reverse_kernel": 14680064, "adjoint_kernel": 417333248}}
